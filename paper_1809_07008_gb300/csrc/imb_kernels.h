@@ -28,6 +28,27 @@ static cudaError_t launch_dependent(void (*kernel)(P...), int grid, int block, i
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<A &&>(args)...);
 }
 
+// The device address of a pinned host array the device can address (page-locked and mapped,
+// as cudaHostAlloc / cudaHostRegister give under unified addressing), else NULL.
+template <typename T>
+static inline T *device_view(T *p) {
+    if (!p) return nullptr;
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();   // clear the error an unknown pointer leaves
+        return nullptr;
+    }
+    return at.type == cudaMemoryTypeHost ? static_cast<T *>(at.devicePointer) : nullptr;
+}
+
+// The same for an array of n elements: its first and its last one lie in such memory, the
+// right distance apart.
+template <typename T>
+static inline T *device_span(T *p, size_t n) {
+    T *a = device_view(p);
+    return a && n && device_view(p + (n - 1)) == a + (n - 1) ? a : nullptr;
+}
+
 struct PRec;
 struct TileCand;
 struct GridBarrier;

@@ -23,6 +23,7 @@
 
 #include "../../include/imblbm.h"
 #include "imb_device.cuh"
+#include "imb_kernels.h"
 
 namespace imb3 {
 
@@ -898,6 +899,16 @@ extern "C" int imb3_step(imb3_ctx *c, int nsteps) {
 extern "C" int imb3_get_populations(imb3_ctx *c, double *f) {
     if (!c || !f) return fail3(c, IMB_E_INVALID_ARG, "bad arguments");
     CK3(cudaSetDevice(c->device), "cudaSetDevice");
+    if (double *h = imb::device_span(f, 19 * c->a.plane)) {   // written straight into pinned host memory
+        CK3(by_storage3(c->p.storage, [&](auto tag) {
+                using S = std::remove_pointer_t<decltype(tag)>;
+                k3_gather<S><<<(unsigned)((c->a.plane + 255) / 256), 256, 0, c->stream>>>((const S *)c->buf[c->cur], c->a, h);
+                return cudaGetLastError();
+            }),
+            "populations");
+        c->launches++;
+        return wait3(c);
+    }
     double *d = nullptr;
     CK3(cudaMalloc(&d, sizeof(double) * 19 * c->a.plane), "readback buffer");
     cudaError_t e = by_storage3(c->p.storage, [&](auto tag) {
@@ -917,8 +928,21 @@ extern "C" int imb3_get_populations(imb3_ctx *c, double *f) {
 extern "C" int imb3_get_macro(imb3_ctx *c, double *rho, double *ux, double *uy, double *uz) {
     if (!c || !rho || !ux || !uy || !uz) return fail3(c, IMB_E_INVALID_ARG, "bad arguments");
     CK3(cudaSetDevice(c->device), "cudaSetDevice");
-    double *d = nullptr;
     const size_t n = c->a.plane;
+    // pinned arrays the device can address are written by the kernel itself (as imb_get_macro)
+    double *h[4] = {imb::device_span(rho, n), imb::device_span(ux, n), imb::device_span(uy, n), imb::device_span(uz, n)};
+    if (h[0] && h[1] && h[2] && h[3]) {
+        CK3(by_storage3(c->p.storage, [&](auto tag) {
+                using S = std::remove_pointer_t<decltype(tag)>;
+                k3_macro<S><<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>((const S *)c->buf[c->cur], c->a, h[0], h[1],
+                                                                                h[2], h[3]);
+                return cudaGetLastError();
+            }),
+            "macroscopic fields");
+        c->launches++;
+        return wait3(c);
+    }
+    double *d = nullptr;
     CK3(cudaMalloc(&d, sizeof(double) * 4 * n), "readback buffer");
     cudaError_t e = by_storage3(c->p.storage, [&](auto tag) {
         using S = std::remove_pointer_t<decltype(tag)>;
