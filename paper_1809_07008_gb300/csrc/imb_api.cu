@@ -59,7 +59,7 @@ struct imb_ctx {
     double *wall_xi = nullptr;
     int *free_ids = nullptr, *coupled_ids = nullptr, *counters = nullptr;
     int *parent = nullptr, *label = nullptr, *isz = nullptr, *ifill = nullptr, *istart = nullptr;
-    int *members = nullptr, *roots = nullptr, *big_ids = nullptr;
+    int *members = nullptr, *roots = nullptr, *big_ids = nullptr, *big_pos = nullptr, *big_ord = nullptr;
     int *loud = nullptr, *iloud = nullptr;
     double *exc = nullptr;
     int *pbin = nullptr;
@@ -249,6 +249,8 @@ static DemArgs dem_args(imb_ctx *c) {
     d.loud = c->loud;
     d.iloud = c->iloud;
     d.big_ids = c->big_ids;
+    d.big_pos = c->big_pos;
+    d.big_ord = c->big_ord;
     d.bin_start = c->bin_start;
     d.bin_ids = c->bin_ids;
     d.pbin = c->pbin;
@@ -275,7 +277,7 @@ static void free_particles(imb_ctx *c) {
     for (double **q : dp) { dfree(*q); *q = nullptr; }
     int **ip[] = {&c->nbr_cnt[0], &c->nbr_cnt[1], &c->nbr_id[0], &c->nbr_id[1], &c->free_ids,
                   &c->coupled_ids, &c->pbin, &c->pslot, &c->bin_ids, &c->parent, &c->label, &c->isz, &c->ifill,
-                  &c->istart, &c->members, &c->roots, &c->big_ids, &c->loud, &c->iloud};
+                  &c->istart, &c->members, &c->roots, &c->big_ids, &c->big_pos, &c->big_ord, &c->loud, &c->iloud};
     for (int **q : ip) { dfree(*q); *q = nullptr; }
     dfree(c->prec);
     c->prec = nullptr;
@@ -541,7 +543,7 @@ extern "C" int imb_set_particles(imb_ctx *c, int n, const double *x, const doubl
         if (e == cudaSuccess) e = dalloc(&c->bin_ids, N);
         if (e == cudaSuccess) e = dalloc(&c->prec, N);
         const size_t Np = (N + 31) / 32 * 32;
-        int **ia[] = {&c->parent, &c->label, &c->members, &c->roots, &c->big_ids, &c->loud};
+        int **ia[] = {&c->parent, &c->label, &c->members, &c->roots, &c->big_ids, &c->big_pos, &c->big_ord, &c->loud};
         for (int **q : ia) if (e == cudaSuccess) e = dalloc(q, N);
         if (e == cudaSuccess) e = dalloc(&c->isz, Np);
         if (e == cudaSuccess) e = dalloc(&c->ifill, Np);
@@ -558,6 +560,7 @@ extern "C" int imb_set_particles(imb_ctx *c, int n, const double *x, const doubl
     }
     c->np = n;
     c->r_max = rmax;
+    if (c->p.dem_on) dem_cluster_fits();   // asked here, before any capture
     {
         const int th = (int)std::ceil(rmax) + 1, tw = 2 * th + 1;
         const size_t need = (size_t)std::max(n, 1) * tw * tw;
@@ -643,8 +646,21 @@ static int dem_cycle(imb_ctx *c, bool zero_forces) {
     CK(launch_dem_neighbours(d, c->stream), "dem neighbours");
     CK(launch_dem_islands_setup(d, c->stream), "dem islands");
     CK(launch_dem_local(d, c->stream), "dem free particles and islands");
-    CK(launch_dem_coupled(d, dem_coupled_blocks(), c->stream), "dem coupled");
-    c->launches += 7;   // neighbours, link, label, alloc, fill, free particles and islands, coupled
+    if (c->np > 32) {   // islands larger than a warp
+        // (both launches find nothing to do in a dilute suspension: 1.3 us each on this stream;
+        // on a second stream beside the free particles they cost 49 us a cycle of 20 000 disks,
+        // the cluster's shared memory and the cooperative launch waiting for idle SMs)
+        const bool cluster = dem_cluster_fits();
+        if (cluster) {
+            CK(launch_dem_cluster(d, c->stream), "dem cluster");
+            c->launches++;
+        }
+        if (!cluster || c->np > dem_cluster_capacity()) {
+            CK(launch_dem_coupled(d, dem_coupled_blocks(), c->stream), "dem coupled");
+            c->launches++;
+        }
+    }
+    c->launches += 6;   // neighbours, link, label, alloc, fill, free particles and islands
     c->nbr_cur ^= 1;
     return rebuild_table(c, c->xs, zero_forces);
 }

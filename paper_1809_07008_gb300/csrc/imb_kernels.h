@@ -111,10 +111,13 @@ struct DemArgs {
     double *wall_xi;                  // [np * 4]
     int *free_ids, *coupled_ids;      // [np]
     int *counters;                    // [0] free, [1] coupled, [2] small islands, [3] big-island
-                                      // particles, [4] member-list cursor, [5] medium islands
+                                      // particles, [4] member-list cursor, [5] medium islands, [6] set
+                                      // when k_dem_cluster stepped the big islands, [7] when a
+                                      // block's contacts don't fit its table there
     int *parent, *label;              // [np] union-find forest and island of each particle
     int *isz, *ifill, *istart;        // per root: island size, fill cursor, start in members
     int *members, *roots, *big_ids;   // [np] island members, roots of small islands, big-island particles
+    int *big_pos, *big_ord;           // [np] place of a big-island particle in the cluster, and back
     const int *bin_start, *bin_ids;   // bins of the positions at cycle start
     int *pbin;                        // [np]
     int nbx, nby;
@@ -171,6 +174,10 @@ cudaError_t launch_bin_scan(int *bin_count, int *bin_fill, int *bin_start, int n
 cudaError_t launch_bin_fill(const int *pbin, int np, int *bin_fill, const int *bin_start,
                             int *bin_ids, cudaStream_t s);
 cudaError_t launch_dem_neighbours(const DemArgs &d, cudaStream_t s);
+// islands of more than 32 particles: one cluster, then what it doesn't hold by the whole grid
+bool dem_cluster_fits();
+int dem_cluster_capacity();   // particles of large islands the cluster holds
+cudaError_t launch_dem_cluster(const DemArgs &d, cudaStream_t s);
 cudaError_t launch_dem_coupled(const DemArgs &d, int nblocks, cudaStream_t s);
 cudaError_t launch_dem_islands_setup(const DemArgs &d, cudaStream_t s);
 // free particles and islands of up to 32 particles, one launch

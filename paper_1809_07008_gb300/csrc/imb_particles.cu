@@ -11,14 +11,18 @@
 //   k_dem_local       the N_sub sub-cycles (Eq. 17) of the free particles (in registers)
 //                     and of the islands of up to 32 particles (a warp each, or eight
 //                     islands of up to four to a warp, in shared memory), in one launch;
-//   k_dem_coupled     the N_sub sub-cycles of the coupled particles, one bounded grid
-//                     barrier per sub-cycle (cooperative launch);
+//   k_dem_cluster     the N_sub sub-cycles of the islands of more than 32 particles, up to
+//                     4096 particles together, in one cluster of 16 blocks;
+//   k_dem_coupled     the same beyond that, one bounded grid barrier per sub-cycle
+//                     (cooperative launch);
 //   k_contacts        pairs in contact (Eq. 7) for readback.
 //
 // DEM arithmetic is FP64.  This file is compiled with --fmad=false so that every
 // multiply and add is rounded separately; with the contact partners summed in
 // ascending id order, particle trajectories then reproduce a plain sequential
 // FP64 evaluation of Eqs. 7-11 exactly.
+#include <cstddef>
+
 #include "imb_device.cuh"
 #include "imb_kernels.h"
 
@@ -126,7 +130,7 @@ __global__ void __launch_bounds__(256) k_bin_scan_local(int *count, int *start, 
         *reinterpret_cast<int4 *>(count + b0) = make_int4(0, 0, 0, 0);
     }
     if (threadIdx.x == 0) bsum[blockIdx.x] = total;
-    if (blockIdx.x == 0 && threadIdx.x < 6 && dem_counters) dem_counters[threadIdx.x] = 0;
+    if (blockIdx.x == 0 && threadIdx.x < 8 && dem_counters) dem_counters[threadIdx.x] = 0;
 }
 
 __global__ void __launch_bounds__(256) k_bin_scan_add(int *fill, int *start, int nbins, const int *bsum) {
@@ -583,10 +587,11 @@ __device__ __forceinline__ void particle_substep(const DemArgs &d, const int p, 
     else coast(d, kick, px, py, vx, vy, w);
 }
 
-// Particles of islands larger than a warp: all blocks step them together, one bounded
-// grid barrier per sub-cycle (cooperative launch), state exchanged through L2.
+// Particles of islands larger than a warp, when there are more than k_dem_cluster holds: all
+// blocks step them together, one bounded grid barrier per sub-cycle (cooperative launch), state
+// exchanged through L2.
 __global__ void k_dem_coupled(const DemArgs d) {
-    const int ncpl = d.counters[3];
+    const int ncpl = d.counters[6] ? 0 : d.counters[3];
     const int nb_active = min((int)gridDim.x, (ncpl + (int)blockDim.x - 1) / (int)blockDim.x);
     if (ncpl == 0 || (int)blockIdx.x >= nb_active) return;
     const int stride = nb_active * blockDim.x;
@@ -888,6 +893,360 @@ __device__ __forceinline__ void warp_islands(const DemArgs &d, WarpIslands &w, c
     __syncwarp();
 }
 
+// ------------------------------------------------------------ large islands in one cluster
+// a / b for a constant b > 0 whose correctly rounded reciprocal y = RN(1 / b) is known, rounded
+// to nearest: a faithful quotient from the reciprocal, then one step with the exact remainder
+// (Markstein 1990: with y correctly rounded and q within an ulp, q + r y rounds to a / b).
+// Five FP64 operations, 64 cycles each, instead of the ten of a division.  Zeros, infinities,
+// NaN and exponents near the ends of the range, where the remainder may not be exact, divide.
+__device__ __forceinline__ double div_by(const double a, const double b, const double y) {
+    const unsigned ea = ((unsigned)__double2hiint(a) >> 20) & 0x7ffu, eb = ((unsigned)__double2hiint(b) >> 20) & 0x7ffu;
+    if (ea - 200u < 1600u && eb - 523u < 1000u) {
+        double q = a * y;
+        q = __fma_rn(__fma_rn(-b, q, a), y, q);
+        return __fma_rn(__fma_rn(-b, q, a), y, q);
+    }
+    return a / b;
+}
+
+// Particles of islands larger than a warp, up to CL_P CL_CTAS of them together: one cluster of
+// CL_CTAS blocks holds their state in shared memory (double-buffered), each block a contiguous
+// run of the particles in Morton order of their bins, and reads the other blocks' particles
+// through the cluster.  A sub-cycle is
+//   1. the overlap test of every candidate pair and near wall of the block, a lane each; those
+//      that touch are listed,
+//   2. the listed contacts, two lanes each (the x and the y component; sums exchanged by
+//      shuffles), so that few warps run the long FP64 sequence,
+//   3. the update, three lanes a particle (x, y, spin), each summing its contacts in slot order
+//      and then the walls -- the order of a sequential evaluation,
+//   4. one hardware cluster barrier.
+// A pair across two blocks is evaluated by both, each with its own particle first: the two
+// results are each other's negatives to the bit (see warp_islands), so no forces cross blocks.
+// What bounds it: the FP64 pipe takes 64 cycles per warp instruction whatever its mask, so the
+// time is the longest chain of instructions of the three rounds plus the barrier.  The grid of
+// one-warp blocks that went through L2 with a spinning barrier and evaluated each particle's
+// candidates one after another took 12 us a sub-cycle on 1000 stacked disks; this takes 4.2 us
+// (a coupling cycle of the 2048 x 1024 collapse, 100 sub-cycles: 1.37 -> 0.56 ms).
+constexpr int CL_CTAS = 16, CL_THREADS = 256, CL_P = 256, CL_Q = 1280;
+
+struct ClusterDem {
+    double st[2][5][CL_P];               // x, y, vx, vy, w
+    double r[CL_P];                      // (at a fixed distance from st for the cluster loads)
+    double mi[2][CL_P], rmi[2][CL_P];    // mass and inertia, their reciprocals
+    double frc[3][CL_P], kick[3][CL_P];  // frozen F_x, F_y, T; contact-free velocity increments
+    double xi[CL_Q], cn[CL_Q], R[CL_Q], RR[CL_Q];
+    double f[3][CL_Q];                   // fx, fy, Ft on the contact's first particle
+    uint32_t pa[CL_Q];                   // cluster address of st[0][0] of the second particle
+    int id[CL_P];
+    unsigned short slot[CL_P][MAX_NBR + 4];   // contact of candidate j / wall, 0x8000: its second particle; 0xffff none
+    unsigned short pi[CL_Q], touch[CL_Q];
+    unsigned char nn[CL_P], kind[CL_Q], on[CL_Q];   // kind: 0 pair, 1 + wall
+    int ncon, ntouch;
+};
+
+__device__ __forceinline__ double ld_cluster(uint32_t a) {
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ double other_half(double v) { return __shfl_xor_sync(0xffffffffu, v, 1); }
+
+__device__ __forceinline__ unsigned long long morton_key(const DemArgs &d, int p) {
+    const int b = d.pbin[p];
+    unsigned long long m = 0;
+    for (int k = 0, x = b % d.nbx, y = b / d.nbx; k < 15; ++k)
+        m |= (unsigned long long)(((x >> k) & 1) | (((y >> k) & 1) << 1)) << (2 * k);
+    return (m << 32) | (unsigned)p;   // unique
+}
+
+__device__ __forceinline__ void store_cluster_state(const DemArgs &d, const ClusterDem &S, int nl) {
+    const int fin = d.N_sub & 1;
+    for (int k = threadIdx.x; k < nl; k += CL_THREADS) {
+        const int p = S.id[k];
+        d.x[2 * p] = S.st[fin][0][k];
+        d.x[2 * p + 1] = S.st[fin][1][k];
+        d.v[2 * p] = S.st[fin][2][k];
+        d.v[2 * p + 1] = S.st[fin][3][k];
+        d.w[p] = S.st[fin][4][k];
+    }
+}
+
+__global__ void __launch_bounds__(CL_THREADS) k_dem_cluster(const DemArgs d) {
+    cudaGridDependencySynchronize();   // launched as a dependent of the kernel before it
+    extern __shared__ __align__(16) unsigned char cl_smem[];
+    ClusterDem &S = *reinterpret_cast<ClusterDem *>(cl_smem);
+    const int n = d.counters[3];
+    if (n == 0 || n > CL_P * CL_CTAS) return;   // every block alike; a larger set: k_dem_coupled
+    const int tid = threadIdx.x, cta = blockIdx.x;
+    // the particles' places: rank by Morton order, block by block
+    unsigned long long *keys = reinterpret_cast<unsigned long long *>(cl_smem);
+    for (int i = tid; i < n; i += CL_THREADS) keys[i] = morton_key(d, d.big_ids[i]);
+    __syncthreads();
+    for (int i = cta * CL_THREADS + tid; i < n; i += CL_THREADS * CL_CTAS) {
+        const unsigned long long k = keys[i];
+        int rank = 0;
+        for (int j = 0; j < n; ++j) rank += keys[j] < k;
+        d.big_pos[(unsigned)k] = rank;
+        d.big_ord[rank] = (int)(unsigned)k;
+    }
+    cluster_barrier();
+    const int per = (n + CL_CTAS - 1) / CL_CTAS, base = cta * per, nl = max(0, min(per, n - base));
+    if (tid == 0) {
+        S.ncon = 0;
+        S.ntouch = 0;
+    }
+    for (int k = tid; k < nl * (MAX_NBR + 4); k += CL_THREADS) S.slot[0][k] = 0xffff;
+    __syncthreads();
+    const uint32_t st0 = smem_addr(&S.st[0][0][0]);
+    for (int k = tid; k < nl; k += CL_THREADS) {
+        const int p = __ldcg(&d.big_ord[base + k]);
+        const int nn = d.nbr_cnt[p];
+        const double rp = d.r[p], mp = d.m[p], Ip = d.I[p];
+        S.id[k] = p;
+        S.nn[k] = (unsigned char)nn;
+        S.st[0][0][k] = d.x[2 * p];
+        S.st[0][1][k] = d.x[2 * p + 1];
+        S.st[0][2][k] = d.v[2 * p];
+        S.st[0][3][k] = d.v[2 * p + 1];
+        S.st[0][4][k] = d.w[p];
+        S.r[k] = rp;
+        S.mi[0][k] = mp;
+        S.mi[1][k] = Ip;
+        S.rmi[0][k] = 1.0 / mp;
+        S.rmi[1][k] = 1.0 / Ip;
+        S.frc[0][k] = d.F[2 * p];
+        S.frc[1][k] = d.F[2 * p + 1];
+        S.frc[2][k] = d.T[p];
+        const Kick kick = free_kick(d, p);
+        S.kick[0][k] = kick.dvx;
+        S.kick[1][k] = kick.dvy;
+        S.kick[2][k] = kick.dw;
+        for (int j = 0; j < nn; ++j) {
+            const int q = d.nbr_id[p * MAX_NBR + j];
+            const int pos = __ldcg(&d.big_pos[q]);
+            if ((unsigned)pos >= (unsigned)n || __ldcg(&d.big_ord[pos]) != q) continue;   // not in a large island (lists are symmetric)
+            const int cq = pos / per, kq = pos - cq * per;
+            if (cq == cta && kq < k) continue;   // the partner leads the pair
+            const int e = atomicAdd(&S.ncon, 1);
+            if (e >= CL_Q) continue;
+            uint32_t a;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(st0 + 8u * (uint32_t)kq), "r"(cq));
+            S.pi[e] = (unsigned short)k;
+            S.pa[e] = a;
+            S.kind[e] = 0;
+            S.xi[e] = d.nbr_xi[p * MAX_NBR + j];
+            S.cn[e] = d.nbr_cn[p * MAX_NBR + j];
+            const double R = rp + d.r[q];
+            S.R[e] = R;
+            S.RR[e] = R * R;
+            S.slot[k][j] = (unsigned short)e;
+            if (cq == cta) {
+                const int nq = d.nbr_cnt[q];
+                for (int jq = 0; jq < nq; ++jq)
+                    if (d.nbr_id[q * MAX_NBR + jq] == p) S.slot[kq][jq] = (unsigned short)(e | 0x8000);
+            }
+        }
+        // walls the particle may reach within the cycle: it moves skin / 2 at most (else IMB_E_SKIN)
+        for (int wl = 0; wl < 4; ++wl) {
+            if ((wl < 2 ? d.bc_x : d.bc_y) != BC_WALL) continue;
+            const double c = wl < 2 ? d.x[2 * p] : d.x[2 * p + 1], L = wl < 2 ? (double)d.nx : (double)d.ny;
+            if (!(((wl & 1) ? L - c : c) < rp + d.skin)) continue;
+            const int e = atomicAdd(&S.ncon, 1);
+            if (e >= CL_Q) continue;
+            S.pi[e] = (unsigned short)k;
+            S.pa[e] = 0;
+            S.kind[e] = (unsigned char)(1 + wl);
+            S.xi[e] = d.wall_xi[4 * p + wl];
+            S.cn[e] = d.model == 1 ? 0.0 : damping_cn(d, mp);
+            S.R[e] = rp;
+            S.RR[e] = 0.0;
+            S.slot[k][MAX_NBR + wl] = (unsigned short)e;
+        }
+    }
+    __syncthreads();
+    const int ncon = S.ncon;
+    if (tid == 0 && ncon > CL_Q) atomicOr(&d.counters[7], 1);
+    cluster_barrier();   // the blocks' states and the flag are in place
+    if (__ldcg(&d.counters[7])) {   // a block's contacts don't fit its table: particle by particle
+        for (int s = 0; s < d.N_sub; ++s) {
+            const int cur = s & 1;
+            const double(*st)[CL_P] = S.st[cur];
+            for (int k = tid; k < nl; k += CL_THREADS) {
+                double px = st[0][k], py = st[1][k], vx = st[2][k], vy = st[3][k], w = st[4][k];
+                const Kick kick = {S.kick[0][k], S.kick[1][k], S.kick[2][k]};
+                particle_substep(d, S.id[k], kick, px, py, vx, vy, w,
+                                 [&](int, int q, double &qx, double &qy, double &qvx, double &qvy, double &qw) {
+                                     const int pos = max(__ldcg(&d.big_pos[q]), 0), cq = min(pos / per, CL_CTAS - 1);
+                                     uint32_t a;
+                                     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                                                  : "=r"(a)
+                                                  : "r"(st0 + 8u * (uint32_t)(cur * 5 * CL_P + min(pos - cq * per, CL_P - 1))),
+                                                    "r"(cq));
+                                     qx = ld_cluster(a);
+                                     qy = ld_cluster(a + CL_P * 8u);
+                                     qvx = ld_cluster(a + 2u * CL_P * 8u);
+                                     qvy = ld_cluster(a + 3u * CL_P * 8u);
+                                     qw = ld_cluster(a + 4u * CL_P * 8u);
+                                 });
+                S.st[cur ^ 1][0][k] = px;
+                S.st[cur ^ 1][1][k] = py;
+                S.st[cur ^ 1][2][k] = vx;
+                S.st[cur ^ 1][3][k] = vy;
+                S.st[cur ^ 1][4][k] = w;
+            }
+            cluster_barrier();
+        }
+        store_cluster_state(d, S, nl);
+        if (cta == 0 && tid == 0) d.counters[6] = 1;
+        return;
+    }
+    const bool perx = d.bc_x == BC_PERIODIC, pery = d.bc_y == BC_PERIODIC;
+    const uint32_t R_OFF = (uint32_t)(offsetof(ClusterDem, r) - offsetof(ClusterDem, st));
+    const double rkt = 1.0 / d.kt;
+    for (int s = 0; s < d.N_sub; ++s) {
+        const int cur = s & 1;
+        const double(*st)[CL_P] = S.st[cur];
+        const uint32_t so = (uint32_t)cur * 5u * CL_P * 8u;   // of st[cur] from st[0]
+        for (int t = tid; t < ncon; t += CL_THREADS) {
+            const int i = S.pi[t], kd = S.kind[t];
+            bool hit;
+            if (kd == 0) {
+                const uint32_t a = S.pa[t] + so;
+                const double dx = min_image(ld_cluster(a) - st[0][i], perx, d.nx);
+                const double dy = min_image(ld_cluster(a + CL_P * 8u) - st[1][i], pery, d.ny);
+                hit = dx * dx + dy * dy < S.RR[t];
+            } else {
+                const double c = kd <= 2 ? st[0][i] : st[1][i], L = kd <= 2 ? (double)d.nx : (double)d.ny;
+                hit = ((kd & 1) ? c : L - c) < S.R[t];   // kind 1 + wall: odd kinds are the walls at 0
+            }
+            S.on[t] = hit;
+            if (hit) S.touch[atomicAdd(&S.ntouch, 1)] = (unsigned short)t;
+            else S.xi[t] = 0.0;   // Eq. 7: no overlap, the spring is released
+        }
+        __syncthreads();
+        const int ntouch = S.ntouch;
+        for (int u0 = (tid & ~31) >> 1; u0 < ntouch; u0 += CL_THREADS / 2) {   // 16 contacts a warp
+            const int u = u0 + ((tid & 31) >> 1), h = tid & 1;
+            const bool act = u < ntouch;
+            const int t = S.touch[act ? u : u0], i = S.pi[t], kd = S.kind[t];
+            double xi = S.xi[t], fh, Ft;
+            if (d.model == 1) {   // Hertz-Mindlin: both lanes the whole contact
+                const double px = st[0][i], py = st[1][i], vx = st[2][i], vy = st[3][i], w = st[4][i], rp = S.r[i], mp = S.mi[0][i];
+                double fx, fy;
+                if (kd == 0) {
+                    const uint32_t a = S.pa[t] + so;
+                    const double dx = min_image(ld_cluster(a) - px, perx, d.nx);
+                    const double dy = min_image(ld_cluster(a + CL_P * 8u) - py, pery, d.ny);
+                    const double rq = ld_cluster(S.pa[t] + R_OFF), mq = ld_cluster(S.pa[t] + R_OFF + CL_P * 8u);
+                    const double dist = sqrt(dx * dx + dy * dy);
+                    const double rot = w * rp + ld_cluster(a + 4u * CL_P * 8u) * rq;
+                    contact_law_cn(d, dx / dist, dy / dist, S.R[t] - dist, ld_cluster(a + 2u * CL_P * 8u) - vx,
+                                   ld_cluster(a + 3u * CL_P * 8u) - vy, rot, S.cn[t], rp * rq / (rp + rq),
+                                   mp * mq / (mp + mq), xi, fx, fy, Ft);
+                } else {
+                    const double c = kd <= 2 ? px : py, L = kd <= 2 ? (double)d.nx : (double)d.ny;
+                    const double dist = (kd & 1) ? c : L - c, sg = (kd & 1) ? -1.0 : 1.0;
+                    contact_law_cn(d, kd <= 2 ? sg : 0.0, kd <= 2 ? 0.0 : sg, rp - dist, -vx, -vy, w * rp, S.cn[t], rp, mp,
+                                   xi, fx, fy, Ft);
+                }
+                fh = h ? fy : fx;
+            } else {   // linear law (contact_law_cn), lane h the component h
+                const double ph = st[h][i], vh = st[2 + h][i], wr = st[4][i] * S.r[i];
+                const int ax = kd <= 2 ? 0 : 1;   // of a wall
+                double dh = 0.0, dvh = -vh, rot = wr;
+                if (kd == 0) {
+                    const uint32_t a = S.pa[t] + so;
+                    dh = min_image(ld_cluster(a + (uint32_t)h * CL_P * 8u) - ph, h ? pery : perx, h ? d.ny : d.nx);
+                    dvh = ld_cluster(a + (uint32_t)(2 + h) * CL_P * 8u) - vh;
+                    rot = wr + ld_cluster(a + 4u * CL_P * 8u) * ld_cluster(S.pa[t] + R_OFF);
+                }
+                const double sq = dh * dh, d2 = sq + other_half(sq);   // the same sum on both lanes
+                double dist, nh;
+                if (kd == 0) {
+                    dist = sqrt(d2);
+                    nh = dh / dist;
+                } else {
+                    const double c = st[ax][i], L = ax ? (double)d.ny : (double)d.nx;
+                    dist = (kd & 1) ? c : L - c;
+                    nh = h == ax ? ((kd & 1) ? -1.0 : 1.0) : 0.0;
+                }
+                const double delta = S.R[t] - dist;
+                const double cn = S.cn[t], no = other_half(nh), th = h ? no : -no;
+                const double a1 = dvh * nh, vn = a1 + other_half(a1);
+                const double a2 = dvh * th, vt = (a2 + other_half(a2)) - rot;
+                xi = xi + vt * d.dt;
+                const double a3 = h ? cn * vn : d.kn * delta, o3 = other_half(a3);
+                const double Fn = h ? o3 - a3 : a3 - o3;
+                const double a4 = h ? (d.ct_ratio * cn) * vt : d.kt * xi;
+                Ft = a4 + other_half(a4);
+                const double lim = d.mu * fabs(Fn);
+                if (fabs(Ft) > lim) {
+                    Ft = copysign(lim, Ft);
+                    xi = copysign(div_by(lim, d.kt, rkt), xi);
+                }
+                fh = -Fn * nh + Ft * th;
+            }
+            if (act) {
+                S.f[h][t] = fh;
+                if (h) S.xi[t] = xi;
+                else S.f[2][t] = Ft;
+            }
+        }
+        __syncthreads();
+        if (tid == 0) S.ntouch = 0;
+        for (int u = tid; u < 3 * nl; u += CL_THREADS) {
+            const int c = u < nl ? 0 : (u < 2 * nl ? 1 : 2), k = u - c * nl;
+            double sum = 0.0;
+            bool touched = false;
+            auto add = [&](const int e) {
+                if (e == 0xffff || !S.on[e & 0x7fff]) return;
+                const double v = S.f[c][e & 0x7fff];
+                sum += c == 2 ? S.r[k] * v : ((e & 0x8000) ? -v : v);
+                touched = true;
+            };
+            for (int j = 0, nn = S.nn[k]; j < nn; ++j) add(S.slot[k][j]);
+#pragma unroll
+            for (int wl = 0; wl < 4; ++wl) add(S.slot[k][MAX_NBR + wl]);
+            double v = st[2 + c][k];
+            if (touched) {
+                const int mi = c == 2;
+                double a = div_by(sum + S.frc[c][k], S.mi[mi][k], S.rmi[mi][k]);
+                if (c < 2) a = a + (c ? d.gy_eff : d.gx_eff);
+                v = v + a * d.dt;
+            } else {
+                v = v + S.kick[c][k];
+            }
+            S.st[cur ^ 1][2 + c][k] = v;
+            if (c < 2) {   // the drift, wrapped on periodic axes
+                double x = st[c][k] + v * d.dt;
+                const double L = c ? (double)d.ny : (double)d.nx;
+                if (c ? pery : perx) {
+                    if (x >= L) x -= L;
+                    else if (x < 0.0) x += L;
+                }
+                S.st[cur ^ 1][c][k] = x;
+            }
+        }
+        cluster_barrier();
+    }
+    store_cluster_state(d, S, nl);
+    for (int k = tid; k < nl; k += CL_THREADS) {
+        const int p = S.id[k];
+        for (int j = 0, nn = S.nn[k]; j < nn; ++j) {
+            const int e = S.slot[k][j];
+            d.nbr_xi[p * MAX_NBR + j] = e == 0xffff ? 0.0 : S.xi[e & 0x7fff];
+        }
+        for (int wl = 0; wl < 4; ++wl) {
+            const int e = S.slot[k][MAX_NBR + wl];
+            d.wall_xi[4 * p + wl] = e == 0xffff ? 0.0 : S.xi[e & 0x7fff];
+        }
+    }
+    if (cta == 0 && tid == 0) d.counters[6] = 1;   // the set is done
+}
+
 // Islands of up to ISL_SMALL particles, SMALL_PER_WARP to a warp in lane groups of
 // ISL_SMALL: block blk of the role.
 __device__ __forceinline__ void dem_small_islands(const DemArgs &d, const int blk, WarpIslands (&sm)[ISL_WARPS]) {
@@ -1018,6 +1377,51 @@ cudaError_t launch_dem_coupled(const DemArgs &d, int nblocks, cudaStream_t s) {
     DemArgs copy = d;
     void *args[] = {&copy};
     return cudaLaunchCooperativeKernel((const void *)k_dem_coupled, dim3(nblocks), dim3(32), args, 0, s);
+}
+
+// Whether the device can hold the cluster (16 blocks are above the portable size of eight); asked
+// once, outside any capture.
+bool dem_cluster_fits() {
+    static const bool fits = [] {   // one device per process
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(CL_CTAS);
+        cfg.blockDim = dim3(CL_THREADS);
+        cfg.dynamicSmemBytes = sizeof(ClusterDem);
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = CL_CTAS;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int nc = 0;
+        const bool ok =
+            cudaFuncSetAttribute(k_dem_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaFuncSetAttribute(k_dem_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ClusterDem)) ==
+                cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&nc, k_dem_cluster, &cfg) == cudaSuccess && nc > 0;
+        if (!ok) cudaGetLastError();
+        return ok;
+    }();
+    return fits;
+}
+
+int dem_cluster_capacity() { return CL_P * CL_CTAS; }
+
+cudaError_t launch_dem_cluster(const DemArgs &d, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(CL_CTAS);
+    cfg.blockDim = dim3(CL_THREADS);
+    cfg.dynamicSmemBytes = sizeof(ClusterDem);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = CL_CTAS;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, k_dem_cluster, d);
 }
 
 cudaError_t launch_dem_islands_setup(const DemArgs &d, cudaStream_t s) {
