@@ -199,6 +199,16 @@ static DemArgs dem_args(imb_ctx *c) {
     d.ny = c->ny;
     d.bc_x = c->p.bc_x;
     d.bc_y = c->p.bc_y;
+    d.Lx = (double)c->nx;
+    d.Ly = (double)c->ny;
+    auto half = [](bool periodic, double L) {
+        long long b = 0x7fffffffffffffffLL;
+        const double h = 0.5 * L;
+        if (periodic) std::memcpy(&b, &h, sizeof(b));
+        return b;
+    };
+    d.half_x = half(c->p.bc_x == IMB_BC_PERIODIC, d.Lx);
+    d.half_y = half(c->p.bc_y == IMB_BC_PERIODIC, d.Ly);
     d.N_sub = c->p.N_sub;
     d.dt = 1.0 / (double)c->p.N_sub;
     d.kn = c->p.kn;
@@ -253,6 +263,7 @@ static DemArgs dem_args(imb_ctx *c) {
     d.big_ord = c->big_ord;
     d.bin_start = c->bin_start;
     d.bin_ids = c->bin_ids;
+    d.prec = c->prec;
     d.pbin = c->pbin;
     d.nbx = c->nbx;
     d.nby = c->nby;

@@ -94,6 +94,8 @@ constexpr int SMALL_UPT = 4;
 struct DemArgs {
     int np, nx, ny, bc_x, bc_y, N_sub;
     double dt, kn, kt, zeta, ct_ratio, mu, gx_eff, gy_eff, skin;
+    double Lx, Ly;              // nx, ny
+    long long half_x, half_y;   // bits of L / 2 on a periodic axis, else the largest integer
     int model;                  // 0 linear spring-dashpot, 1 simplified Hertz-Mindlin
     double hm_kn0, hm_sn0, hm_kt0, hm_c0;   // 4/3 E*, 2 E*, 8 G*, 2 sqrt(5/6) |beta|
     double *x, *v, *w;          // primary state [2np], [2np], [np]
@@ -119,6 +121,7 @@ struct DemArgs {
     int *members, *roots, *big_ids;   // [np] island members, roots of small islands, big-island particles
     int *big_pos, *big_ord;           // [np] place of a big-island particle in the cluster, and back
     const int *bin_start, *bin_ids;   // bins of the positions at cycle start
+    const PRec *prec;                 // [np] particle records of those positions
     int *pbin;                        // [np]
     int nbx, nby;
     GridBarrier *barrier;

@@ -37,6 +37,30 @@ __device__ __forceinline__ double min_image(double d, bool periodic, int L) {
     return d;
 }
 
+// The same and the wrap into [0, L) by comparisons of the bit patterns, which order non-negative
+// doubles like integers: an FP64 compare takes the FP64 pipe 64 cycles, these a few integer
+// instructions.  half: the bits of L / 2, the largest integer on an axis that is not periodic.
+// (The empty asm keeps the rare correction a branch: computed for every lane and selected, its
+// FP64 add would cost what the compare did.)
+__device__ __forceinline__ double nearest(double d, long long half, double L) {
+    if (__double_as_longlong(fabs(d)) > half) {
+        asm volatile("" : "+d"(d));
+        d -= copysign(L, d);
+    }
+    return d;
+}
+__device__ __forceinline__ double wrap_axis(double x, double L) {
+    const long long b = __double_as_longlong(x);
+    if (b >= __double_as_longlong(L)) {
+        asm volatile("" : "+d"(x));
+        x -= L;
+    } else if ((unsigned long long)b > 0x8000000000000000ull) {   // below zero, not -0
+        asm volatile("" : "+d"(x));
+        x += L;
+    }
+    return x;
+}
+
 __device__ __forceinline__ int bin_of(double px, double py, int nbx, int nby) {
     int bx = (int)floor(px / (double)TILE), by = (int)floor(py / (double)TILE);
     bx = bx < 0 ? 0 : (bx >= nbx ? nbx - 1 : bx);
@@ -226,10 +250,9 @@ __device__ __forceinline__ bool pair_force_xi(const DemArgs &d, const int p, con
                                               const double qy, const double qvx, const double qvy, const double qw,
                                               const double vx, const double vy, double &fx, double &fy,
                                               double &Ft) {
-    const bool perx = d.bc_x == BC_PERIODIC, pery = d.bc_y == BC_PERIODIC;
     const double rp = d.r[p];
-    const double dx = min_image(qx - px, perx, d.nx);
-    const double dy = min_image(qy - py, pery, d.ny);
+    const double dx = nearest(qx - px, d.half_x, d.Lx);
+    const double dy = nearest(qy - py, d.half_y, d.Ly);
     const double d2 = dx * dx + dy * dy;
     const double R = rp + d.r[q];
     if (!(d2 < R * R)) {  // Eq. 7: no overlap, the spring is released
@@ -271,9 +294,9 @@ __device__ __forceinline__ bool wall_contacts(const DemArgs &d, int p, double px
         if (!active) continue;
         double dist, nxv, nyv;
         if (wl == 0) { dist = px; nxv = -1.0; nyv = 0.0; }
-        else if (wl == 1) { dist = (double)d.nx - px; nxv = 1.0; nyv = 0.0; }
+        else if (wl == 1) { dist = d.Lx - px; nxv = 1.0; nyv = 0.0; }
         else if (wl == 2) { dist = py; nxv = 0.0; nyv = -1.0; }
-        else { dist = (double)d.ny - py; nxv = 0.0; nyv = 1.0; }
+        else { dist = d.Ly - py; nxv = 0.0; nyv = 1.0; }
         if (!(dist < rp)) {
             xiw[wl] = 0.0;
             continue;
@@ -292,14 +315,8 @@ __device__ __forceinline__ bool wall_contacts(const DemArgs &d, int p, double px
 __device__ __forceinline__ void drift(const DemArgs &d, double &px, double &py, double vx, double vy) {
     px = px + vx * d.dt;
     py = py + vy * d.dt;
-    if (d.bc_x == BC_PERIODIC) {
-        if (px >= d.nx) px -= d.nx;
-        else if (px < 0.0) px += d.nx;
-    }
-    if (d.bc_y == BC_PERIODIC) {
-        if (py >= d.ny) py -= d.ny;
-        else if (py < 0.0) py += d.ny;
-    }
+    if (d.bc_x == BC_PERIODIC) px = wrap_axis(px, d.Lx);
+    if (d.bc_y == BC_PERIODIC) py = wrap_axis(py, d.Ly);
 }
 
 // Eqs. 10-11, leapfrog kick-drift.
@@ -359,24 +376,10 @@ __device__ __forceinline__ FreeMotion free_motion(const DemArgs &d, int p, doubl
 // No wall within reach and no periodic crossing during the cycle.
 __device__ __forceinline__ bool free_of_edges(const DemArgs &d, const FreeMotion &f, double px, double py,
                                               double rp) {
-    return (d.bc_x != BC_WALL || (px - rp > f.ex && ((double)d.nx - px) - rp > f.ex)) &&
-           (d.bc_y != BC_WALL || (py - rp > f.ey && ((double)d.ny - py) - rp > f.ey)) &&
-           (d.bc_x != BC_PERIODIC || (px > f.ex && px < (double)d.nx - f.ex)) &&
-           (d.bc_y != BC_PERIODIC || (py > f.ey && py < (double)d.ny - f.ey));
-}
-
-// The N_sub sub-cycles of a particle that touches nothing: the updates of integrate().
-__device__ __forceinline__ void free_run(const DemArgs &d, const FreeMotion &f, double &px, double &py,
-                                         double &vx, double &vy, double &w) {
-    // the velocity increments a dt round to the same value every sub-cycle
-    const double dvx = f.ax * d.dt, dvy = f.ay * d.dt, dw = f.al * d.dt;
-    for (int s = 0; s < d.N_sub; ++s) {
-        vx = vx + dvx;
-        vy = vy + dvy;
-        w = w + dw;
-        px = px + vx * d.dt;
-        py = py + vy * d.dt;
-    }
+    return (d.bc_x != BC_WALL || (px - rp > f.ex && (d.Lx - px) - rp > f.ex)) &&
+           (d.bc_y != BC_WALL || (py - rp > f.ey && (d.Ly - py) - rp > f.ey)) &&
+           (d.bc_x != BC_PERIODIC || (px > f.ex && px < d.Lx - f.ex)) &&
+           (d.bc_y != BC_PERIODIC || (py > f.ey && py < d.Ly - f.ey));
 }
 
 // Candidate pair (p, q) cannot overlap within the cycle if both move freely: the gap
@@ -384,8 +387,8 @@ __device__ __forceinline__ void free_run(const DemArgs &d, const FreeMotion &f, 
 __device__ __forceinline__ bool pair_apart(const DemArgs &d, double px, double py, double rp, double exp_,
                                            double eyp, double qx, double qy, double rq, double exq,
                                            double eyq) {
-    const double dx = min_image(qx - px, d.bc_x == BC_PERIODIC, d.nx);
-    const double dy = min_image(qy - py, d.bc_y == BC_PERIODIC, d.ny);
+    const double dx = nearest(qx - px, d.half_x, d.Lx);
+    const double dy = nearest(qy - py, d.half_y, d.Ly);
     const double M = rp + rq + (exp_ + exq) + (eyp + eyq);
     return dx * dx + dy * dy > M * M;
 }
@@ -450,6 +453,8 @@ __global__ void __launch_bounds__(32 * NB_WARPS) k_dem_neighbours(const DemArgs 
     }
     const int total = __shfl_sync(FULLM, incl, 31);
     const int excl = incl - cnt;
+    const PRec P = d.prec[p];
+    const float skin_f = (float)d.skin + 0.02f;
     int nh = 0;
     for (int base = 0; base < total; base += 32) {
         const int k = base + lane;
@@ -460,10 +465,20 @@ __global__ void __launch_bounds__(32 * NB_WARPS) k_dem_neighbours(const DemArgs 
             const int g = __shfl_sync(FULLM, beg, j);
             if (k >= e && k < e + c) q = d.bin_ids[g + k - e];
         }
-        bool hit = false;
+        // in FP32 first, from the particle records and with a margin well above their rounding: few
+        // of the bins' particles are near, and the FP64 test costs a warp its full time for one lane
+        bool near = false;
         if (q >= 0 && q != p) {
-            const double dx = min_image(d.x[2 * q] - px, perx, d.nx);
-            const double dy = min_image(d.x[2 * q + 1] - py, pery, d.ny);
+            const PRec Q = d.prec[q];
+            const float dx = (float)wrap_rel(Q.ci - P.ci, d.nx, perx) + (Q.fx - P.fx);
+            const float dy = (float)wrap_rel(Q.cj - P.cj, d.ny, pery) + (Q.fy - P.fy);
+            const float R = P.r + Q.r + skin_f;
+            near = dx * dx + dy * dy < R * R;
+        }
+        bool hit = false;
+        if (near) {
+            const double dx = nearest(d.x[2 * q] - px, d.half_x, d.Lx);
+            const double dy = nearest(d.x[2 * q + 1] - py, d.half_y, d.Ly);
             const double R = rp + d.r[q] + d.skin;
             hit = dx * dx + dy * dy < R * R;
         }
@@ -515,50 +530,117 @@ __global__ void __launch_bounds__(32 * NB_WARPS) k_dem_neighbours(const DemArgs 
     }
 }
 
-// Free particles, one per thread: blocks blk of nblk.
-__device__ __forceinline__ void dem_free(const DemArgs &d, const int blk, const int nblk) {
-    const int nfree = d.counters[0];
-    for (int c = blk * blockDim.x + threadIdx.x; c < nfree; c += nblk * blockDim.x) {
-        const int p = d.free_ids[c];
-        double px = d.x[2 * p], py = d.x[2 * p + 1], vx = d.v[2 * p], vy = d.v[2 * p + 1], w = d.w[p];
-        const double rp = d.r[p], mp = d.m[p];
-        double xiw[4];
+constexpr int ISL_WARPS = 4;                    // warps of a block of k_dem_local
+constexpr int LOCAL_THREADS = 32 * ISL_WARPS;
+
+// A free particle that an edge may concern within the cycle (a wall, a periodic crossing), whole.
+__device__ __forceinline__ void free_near_edge(const DemArgs &d, const int p) {
+    double px = d.x[2 * p], py = d.x[2 * p + 1], vx = d.v[2 * p], vy = d.v[2 * p + 1], w = d.w[p];
+    const double rp = d.r[p], mp = d.m[p];
+    double xiw[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) xiw[k] = d.wall_xi[4 * p + k];
-        // candidate partners of a quiet island stay out of reach: their springs are released
-        for (int j = 0, nn = d.nbr_cnt[p]; j < nn; ++j) d.nbr_xi[p * MAX_NBR + j] = 0.0;
-        const FreeMotion f = free_motion(d, p, vx, vy);
-        const Kick kick = free_kick(d, p);
-        if (free_of_edges(d, f, px, py, rp)) {
+    for (int k = 0; k < 4; ++k) xiw[k] = d.wall_xi[4 * p + k];
+    const Kick kick = free_kick(d, p);
+    const bool walls = d.bc_x == BC_WALL || d.bc_y == BC_WALL;
+    for (int s = 0; s < d.N_sub; ++s) {
+        bool touching = false;
+        if (walls)
+            touching = (d.bc_x == BC_WALL && (px < rp || d.Lx - px < rp)) ||
+                       (d.bc_y == BC_WALL && (py < rp || d.Ly - py < rp));
+        if (touching) {
+            double Fcx = 0.0, Fcy = 0.0, Tc = 0.0;
+            wall_contacts(d, p, px, py, vx, vy, w, rp, mp, xiw, Fcx, Fcy, Tc);
+            integrate(d, p, Fcx, Fcy, Tc, px, py, vx, vy, w);
+        } else {
+            // a released wall spring (wall_contacts would zero it)
 #pragma unroll
             for (int k = 0; k < 4; ++k) xiw[k] = 0.0;
-            free_run(d, f, px, py, vx, vy, w);
-        } else {
-            const bool walls = d.bc_x == BC_WALL || d.bc_y == BC_WALL;
-            for (int s = 0; s < d.N_sub; ++s) {
-                bool touching = false;
-                if (walls)
-                    touching = (d.bc_x == BC_WALL && (px < rp || (double)d.nx - px < rp)) ||
-                               (d.bc_y == BC_WALL && (py < rp || (double)d.ny - py < rp));
-                if (touching) {
-                    double Fcx = 0.0, Fcy = 0.0, Tc = 0.0;
-                    wall_contacts(d, p, px, py, vx, vy, w, rp, mp, xiw, Fcx, Fcy, Tc);
-                    integrate(d, p, Fcx, Fcy, Tc, px, py, vx, vy, w);
-                } else {
-                    // a released wall spring (wall_contacts would zero it)
+            coast(d, kick, px, py, vx, vy, w);
+        }
+    }
+    d.x[2 * p] = px;
+    d.x[2 * p + 1] = py;
+    d.v[2 * p] = vx;
+    d.v[2 * p + 1] = vy;
+    d.w[p] = w;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) xiw[k] = 0.0;
-                    coast(d, kick, px, py, vx, vy, w);
-                }
+    for (int k = 0; k < 4; ++k) d.wall_xi[4 * p + k] = xiw[k];
+}
+
+// Free particles, FREE_GROUP to a block: three warps with a lane per particle and axis (three
+// FP64 operations a sub-cycle) and one warp with the spins (one operation each, two particles on
+// some lanes).  The FP64 pipe takes 64 cycles per warp instruction whatever its mask, and a lane
+// that walked both axes and the spin took seven of them for every sub-cycle: 22 us a coupling
+// cycle for a lone warp, against 10 us, and with 20 000 particles two such warps in a row on some
+// schedulers.  k_dem_local on the 512 x 512 suspension: 32.6 -> 16.7 us, on the 8192 x 4096 one 60 ->
+// 49 us, with the islands' chains below.  The sums are integrate()'s on zero contact sums, operation by operation.
+constexpr int FREE_GROUP = 48;
+
+__device__ __forceinline__ void dem_free(const DemArgs &d, const int blk, const int nblk,
+                                         unsigned char (&inside)[FREE_GROUP]) {
+    const int nfree = d.counters[0], tid = threadIdx.x;
+    for (int g = blk; g * FREE_GROUP < nfree; g += nblk) {
+        const int n = min(FREE_GROUP, nfree - g * FREE_GROUP);
+        const int k = tid >> 1, c = tid & 1;
+        int p = -1;
+        double x = 0.0, v = 0.0, a = 0.0;
+        bool ok = true;
+        if (k < n) {
+            p = d.free_ids[g * FREE_GROUP + k];
+            x = d.x[2 * p + c];
+            v = d.v[2 * p + c];
+            // free_motion and free_of_edges, the axis of this lane
+            a = (0.0 + d.F[2 * p + c]) / d.m[p] + (c ? d.gy_eff : d.gx_eff);
+            const double rp = d.r[p], e = fabs(v) + fabs(a) + 1e-6, L = c ? d.Ly : d.Lx;
+            const int bc = c ? d.bc_y : d.bc_x;
+            ok = (bc != BC_WALL || (x - rp > e && (L - x) - rp > e)) && (bc != BC_PERIODIC || (x > e && x < L - e));
+        }
+        const bool other = __shfl_xor_sync(0xffffffffu, (int)ok, 1) != 0;
+        ok = ok && other;
+        if (k < n && c == 0) inside[k] = ok;
+        __syncthreads();
+        if (k < n && ok) {
+            const double dv = a * d.dt;
+            for (int s = 0; s < d.N_sub; ++s) {
+                v = v + dv;
+                x = x + v * d.dt;
+            }
+            d.x[2 * p + c] = x;
+            d.v[2 * p + c] = v;
+        }
+        if (k < n && c == 0) {
+            // candidate partners of a quiet island stay out of reach: their springs are released
+            for (int j = 0, nn = d.nbr_cnt[p]; j < nn; ++j) d.nbr_xi[p * MAX_NBR + j] = 0.0;
+            if (ok) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) d.wall_xi[4 * p + q] = 0.0;
+            } else {
+                free_near_edge(d, p);
             }
         }
-        d.x[2 * p] = px;
-        d.x[2 * p + 1] = py;
-        d.v[2 * p] = vx;
-        d.v[2 * p + 1] = vy;
-        d.w[p] = w;
+        if (tid >= LOCAL_THREADS - 32) {   // the spins
+            const int l = tid & 31;
+            int q[2];
+            double w[2] = {0.0, 0.0}, dw[2] = {0.0, 0.0};
 #pragma unroll
-        for (int k = 0; k < 4; ++k) d.wall_xi[4 * p + k] = xiw[k];
+            for (int h = 0; h < 2; ++h) {
+                const int kk = l + 32 * h;
+                q[h] = kk < n && inside[kk] ? d.free_ids[g * FREE_GROUP + kk] : -1;
+                if (q[h] >= 0) {
+                    w[h] = d.w[q[h]];
+                    const double al = (0.0 + d.T[q[h]]) / d.I[q[h]];
+                    dw[h] = al * d.dt;
+                }
+            }
+            for (int s = 0; s < d.N_sub; ++s) {
+                w[0] = w[0] + dw[0];
+                w[1] = w[1] + dw[1];
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                if (q[h] >= 0) d.w[q[h]] = w[h];
+        }
+        __syncthreads();
     }
 }
 
@@ -667,8 +749,9 @@ __global__ void k_uf_link(const DemArgs d) {
         int loud = d.loud[p];
         for (int j = 0; j < n; ++j) {
             const int q = d.nbr_id[p * MAX_NBR + j];
-            loud |= !pair_apart(d, px, py, rp, exp_, eyp, d.x[2 * q], d.x[2 * q + 1], d.r[q], d.exc[2 * q],
-                                d.exc[2 * q + 1]);
+            if (!loud)
+                loud = !pair_apart(d, px, py, rp, exp_, eyp, d.x[2 * q], d.x[2 * q + 1], d.r[q], d.exc[2 * q],
+                                   d.exc[2 * q + 1]);
             if (q < p) continue;
             int a = p, b = q;
             for (;;) {
@@ -696,7 +779,6 @@ __global__ void k_uf_label(const DemArgs d) {
 }
 
 constexpr int ISL_SMALL = 4;           // islands up to this size share a warp, 8 to a warp
-constexpr int ISL_WARPS = 4;
 constexpr int ISL_PAIRS = 96;          // pairs evaluated a lane each, beyond that particle by particle
 
 // Roots reserve a contiguous range of the member list for their island.
@@ -748,6 +830,8 @@ struct WarpIslands {
     double st[2][5][32];                 // x, y, vx, vy, w
     double f[3][ISL_PAIRS];              // fx, fy, Ft on the pair's first particle
     double xi[ISL_PAIRS];                // the pair's tangential spring
+    double RR[ISL_PAIRS];                // (r_a + r_b)^2
+    float reach[32];                     // what the frozen forces add to a particle's speed in a cycle
     int id[32];
     unsigned char nn[32];                // candidates of lane l
     unsigned char nl[32][MAX_NBR];       // lane of candidate j
@@ -802,6 +886,8 @@ __device__ __forceinline__ void warp_islands(const DemArgs &d, WarpIslands &w, c
             w.slot[lane][j] = (unsigned char)k;
             if (jr < w.nn[l]) w.slot[l][jr] = (unsigned char)(k | 128);
             w.xi[k] = d.nbr_xi[p * MAX_NBR + j];   // equal to the partner's spring of the pair
+            const double R = d.r[p] + d.r[w.id[l]];
+            w.RR[k] = R * R;
             ++k;
         }
     }
@@ -816,30 +902,81 @@ __device__ __forceinline__ void warp_islands(const DemArgs &d, WarpIslands &w, c
     double xiw[4];   // wall springs, in registers on the pair-parallel path
 #pragma unroll
     for (int q = 0; q < 4; ++q) xiw[q] = act ? d.wall_xi[4 * p + q] : 0.0;
+    // a wall within reach of a lane's particle in this cycle (a particle that moves further than
+    // skin / 2 raises IMB_E_SKIN); else no wall touches and the springs are released
+    bool near_wall = false;
+    if (act) {
+        const double g = rp + d.skin, x = w.st[0][0][lane], y = w.st[0][1][lane];
+        near_wall = (d.bc_x == BC_WALL && (x < g || d.Lx - x < g)) ||
+                    (d.bc_y == BC_WALL && (y < g || d.Ly - y < g));
+    }
+    const bool walls = __any_sync(0xffffffffu, near_wall);
+    if (!walls) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) xiw[q] = 0.0;
+    }
+    // Sub-cycles without an overlap test: while nothing touches, a particle's speed along an axis
+    // stays below |v| + N_sub |kick|, so two particles close their gap by at most the sum of these
+    // bounds times dt a sub-cycle.  After a test in which no pair of the warp touched, as many
+    // sub-cycles as the narrowest gap lasts need no test (bounds in FP32, rounded outwards); any
+    // contact, with a wall too, ends the count.  The test is six of the thirteen FP64 operations
+    // of a quiet sub-cycle.
+    w.reach[lane] = act ? 1.0001f * (float)(fabs(kick.dvx) + fabs(kick.dvy)) * (float)d.N_sub : 0.0f;
+    int quiet = 0;   // sub-cycles left without a test (the same on every lane)
     __syncwarp();
     for (int s = 0; s < d.N_sub; ++s) {
         const int cur = s & 1;
         const double(*st)[32] = w.st[cur];
-        if (pairwise) {
-            for (int k = lane; k < npairs; k += 32) {
-                const int i = w.pi[k], j = w.pj[k], l = w.nl[i][j];
-                double xi = w.xi[k];
-                double fx = 0.0, fy = 0.0, Ft = 0.0;
-                w.on[k] = pair_force_xi(d, w.id[i], j, w.id[l], xi, st[0][i], st[1][i], st[4][i], st[0][l],
-                                        st[1][l], st[2][l], st[3][l], st[4][l], st[2][i], st[3][i], fx, fy, Ft);
-                w.xi[k] = xi;
-                w.f[0][k] = fx;
-                w.f[1][k] = fy;
-                w.f[2][k] = Ft;
+        const bool test = quiet == 0;
+        if (pairwise && test) {
+            bool any = false;
+            for (int k0 = 0; k0 < npairs; k0 += 32) {
+                const int k = k0 + lane;
+                bool hit = false;
+                int i = 0, l = 0;
+                double d2 = 0.0;
+                if (k < npairs) {
+                    i = w.pi[k];
+                    l = w.nl[i][w.pj[k]];
+                    const double dx = nearest(st[0][l] - st[0][i], d.half_x, d.Lx);
+                    const double dy = nearest(st[1][l] - st[1][i], d.half_y, d.Ly);
+                    d2 = dx * dx + dy * dy;
+                    hit = d2 < w.RR[k];   // Eq. 7
+                    w.on[k] = hit;
+                    if (!hit) w.xi[k] = 0.0;   // no overlap, the spring is released
+                }
+                if (hit) {
+                    double xi = w.xi[k], fx, fy, Ft;
+                    pair_force_xi(d, w.id[i], w.pj[k], w.id[l], xi, st[0][i], st[1][i], st[4][i], st[0][l], st[1][l],
+                                  st[2][l], st[3][l], st[4][l], st[2][i], st[3][i], fx, fy, Ft);
+                    w.xi[k] = xi;
+                    w.f[0][k] = fx;
+                    w.f[1][k] = fy;
+                    w.f[2][k] = Ft;
+                }
+                any |= __any_sync(0xffffffffu, hit);
+                if (!any && npairs <= 32) {   // nothing touches: how long does the narrowest gap last
+                    float last = 1.0e6f;
+                    if (k < npairs) {
+                        const float gap = 0.99999f * sqrtf((float)d2) - 1.00001f * sqrtf((float)w.RR[k]);
+                        const float speed = 1.0001f * (float)(fabs(st[2][i]) + fabs(st[3][i]) + fabs(st[2][l]) + fabs(st[3][l])) +
+                                            w.reach[i] + w.reach[l] + 1.0e-9f;
+                        last = fminf(last, gap / (speed * (float)d.dt));
+                    }
+                    // of the sub-cycles after this one, floor(last) - 1 surely show no overlap
+                    quiet = __reduce_min_sync(0xffffffffu, (int)fmaxf(last - 1.0f, 0.0f)) + 1;
+                }
             }
+            if (any || npairs > 32) quiet = 1;
             __syncwarp();
         }
+        bool contact = false;
         if (act) {
             double px = st[0][lane], py = st[1][lane], vx = st[2][lane], vy = st[3][lane], om = st[4][lane];
             if (pairwise) {
                 double Fcx = 0.0, Fcy = 0.0, Tc = 0.0;
                 bool touched = false;
-                for (int j = 0; j < nn; ++j) {
+                for (int j = 0; test && j < nn; ++j) {
                     const int e = w.slot[lane][j], k = e & 127;
                     if (!w.on[k]) continue;
                     if (e & 128) {
@@ -852,9 +989,10 @@ __device__ __forceinline__ void warp_islands(const DemArgs &d, WarpIslands &w, c
                     Tc += rp * w.f[2][k];
                     touched = true;
                 }
-                touched |= wall_contacts(d, p, px, py, vx, vy, om, rp, mp, xiw, Fcx, Fcy, Tc);
+                if (walls) touched |= wall_contacts(d, p, px, py, vx, vy, om, rp, mp, xiw, Fcx, Fcy, Tc);
                 if (touched) integrate(d, p, Fcx, Fcy, Tc, px, py, vx, vy, om);
                 else coast(d, kick, px, py, vx, vy, om);
+                contact = touched;
             } else {
                 particle_substep(d, p, kick, px, py, vx, vy, om,
                                  [&](int j, int, double &qx, double &qy, double &qvx, double &qvy, double &qw) {
@@ -872,7 +1010,8 @@ __device__ __forceinline__ void warp_islands(const DemArgs &d, WarpIslands &w, c
             w.st[cur ^ 1][3][lane] = vy;
             w.st[cur ^ 1][4][lane] = om;
         }
-        __syncwarp();
+        --quiet;
+        if (__any_sync(0xffffffffu, contact)) quiet = 0;   // speeds changed
     }
     if (act) {
         const int fin = d.N_sub & 1;
@@ -1052,7 +1191,7 @@ __global__ void __launch_bounds__(CL_THREADS) k_dem_cluster(const DemArgs d) {
         // walls the particle may reach within the cycle: it moves skin / 2 at most (else IMB_E_SKIN)
         for (int wl = 0; wl < 4; ++wl) {
             if ((wl < 2 ? d.bc_x : d.bc_y) != BC_WALL) continue;
-            const double c = wl < 2 ? d.x[2 * p] : d.x[2 * p + 1], L = wl < 2 ? (double)d.nx : (double)d.ny;
+            const double c = wl < 2 ? d.x[2 * p] : d.x[2 * p + 1], L = wl < 2 ? d.Lx : d.Ly;
             if (!(((wl & 1) ? L - c : c) < rp + d.skin)) continue;
             const int e = atomicAdd(&S.ncon, 1);
             if (e >= CL_Q) continue;
@@ -1115,11 +1254,11 @@ __global__ void __launch_bounds__(CL_THREADS) k_dem_cluster(const DemArgs d) {
             bool hit;
             if (kd == 0) {
                 const uint32_t a = S.pa[t] + so;
-                const double dx = min_image(ld_cluster(a) - st[0][i], perx, d.nx);
-                const double dy = min_image(ld_cluster(a + CL_P * 8u) - st[1][i], pery, d.ny);
+                const double dx = nearest(ld_cluster(a) - st[0][i], d.half_x, d.Lx);
+                const double dy = nearest(ld_cluster(a + CL_P * 8u) - st[1][i], d.half_y, d.Ly);
                 hit = dx * dx + dy * dy < S.RR[t];
             } else {
-                const double c = kd <= 2 ? st[0][i] : st[1][i], L = kd <= 2 ? (double)d.nx : (double)d.ny;
+                const double c = kd <= 2 ? st[0][i] : st[1][i], L = kd <= 2 ? d.Lx : d.Ly;
                 hit = ((kd & 1) ? c : L - c) < S.R[t];   // kind 1 + wall: odd kinds are the walls at 0
             }
             S.on[t] = hit;
@@ -1138,8 +1277,8 @@ __global__ void __launch_bounds__(CL_THREADS) k_dem_cluster(const DemArgs d) {
                 double fx, fy;
                 if (kd == 0) {
                     const uint32_t a = S.pa[t] + so;
-                    const double dx = min_image(ld_cluster(a) - px, perx, d.nx);
-                    const double dy = min_image(ld_cluster(a + CL_P * 8u) - py, pery, d.ny);
+                    const double dx = nearest(ld_cluster(a) - px, d.half_x, d.Lx);
+                    const double dy = nearest(ld_cluster(a + CL_P * 8u) - py, d.half_y, d.Ly);
                     const double rq = ld_cluster(S.pa[t] + R_OFF), mq = ld_cluster(S.pa[t] + R_OFF + CL_P * 8u);
                     const double dist = sqrt(dx * dx + dy * dy);
                     const double rot = w * rp + ld_cluster(a + 4u * CL_P * 8u) * rq;
@@ -1147,7 +1286,7 @@ __global__ void __launch_bounds__(CL_THREADS) k_dem_cluster(const DemArgs d) {
                                    ld_cluster(a + 3u * CL_P * 8u) - vy, rot, S.cn[t], rp * rq / (rp + rq),
                                    mp * mq / (mp + mq), xi, fx, fy, Ft);
                 } else {
-                    const double c = kd <= 2 ? px : py, L = kd <= 2 ? (double)d.nx : (double)d.ny;
+                    const double c = kd <= 2 ? px : py, L = kd <= 2 ? d.Lx : d.Ly;
                     const double dist = (kd & 1) ? c : L - c, sg = (kd & 1) ? -1.0 : 1.0;
                     contact_law_cn(d, kd <= 2 ? sg : 0.0, kd <= 2 ? 0.0 : sg, rp - dist, -vx, -vy, w * rp, S.cn[t], rp, mp,
                                    xi, fx, fy, Ft);
@@ -1159,7 +1298,7 @@ __global__ void __launch_bounds__(CL_THREADS) k_dem_cluster(const DemArgs d) {
                 double dh = 0.0, dvh = -vh, rot = wr;
                 if (kd == 0) {
                     const uint32_t a = S.pa[t] + so;
-                    dh = min_image(ld_cluster(a + (uint32_t)h * CL_P * 8u) - ph, h ? pery : perx, h ? d.ny : d.nx);
+                    dh = nearest(ld_cluster(a + (uint32_t)h * CL_P * 8u) - ph, h ? d.half_y : d.half_x, h ? d.Ly : d.Lx);
                     dvh = ld_cluster(a + (uint32_t)(2 + h) * CL_P * 8u) - vh;
                     rot = wr + ld_cluster(a + 4u * CL_P * 8u) * ld_cluster(S.pa[t] + R_OFF);
                 }
@@ -1169,7 +1308,7 @@ __global__ void __launch_bounds__(CL_THREADS) k_dem_cluster(const DemArgs d) {
                     dist = sqrt(d2);
                     nh = dh / dist;
                 } else {
-                    const double c = st[ax][i], L = ax ? (double)d.ny : (double)d.nx;
+                    const double c = st[ax][i], L = ax ? d.Ly : d.Lx;
                     dist = (kd & 1) ? c : L - c;
                     nh = h == ax ? ((kd & 1) ? -1.0 : 1.0) : 0.0;
                 }
@@ -1222,11 +1361,7 @@ __global__ void __launch_bounds__(CL_THREADS) k_dem_cluster(const DemArgs d) {
             S.st[cur ^ 1][2 + c][k] = v;
             if (c < 2) {   // the drift, wrapped on periodic axes
                 double x = st[c][k] + v * d.dt;
-                const double L = c ? (double)d.ny : (double)d.nx;
-                if (c ? pery : perx) {
-                    if (x >= L) x -= L;
-                    else if (x < 0.0) x += L;
-                }
+                if (c ? pery : perx) x = wrap_axis(x, c ? d.Ly : d.Lx);
                 S.st[cur ^ 1][c][k] = x;
             }
         }
@@ -1281,15 +1416,15 @@ __device__ __forceinline__ void dem_islands(const DemArgs &d, const int blk, con
 // ranges in that order and run side by side (the three sets of particles are disjoint), so
 // an island's chain of N_sub sub-cycles, bound by the latency of its FP64 instructions,
 // overlaps the free particles' FP64 throughput and the other islands' chains.
-constexpr int LOCAL_THREADS = 32 * ISL_WARPS;
 
 __global__ void __launch_bounds__(LOCAL_THREADS) k_dem_local(const DemArgs d, int nb_islands, int nb_small) {
     cudaGridDependencySynchronize();   // launched as a dependent of the kernel before it
     __shared__ WarpIslands sm[ISL_WARPS];
+    __shared__ unsigned char inside[FREE_GROUP];
     const int b = blockIdx.x, nb_free = (int)gridDim.x - nb_islands - nb_small;
-    if (b < nb_free) dem_free(d, b, nb_free);
-    else if (b < nb_free + nb_small) dem_small_islands(d, b - nb_free, sm);
-    else dem_islands(d, b - nb_free - nb_small, nb_islands, sm);
+    if (b < nb_small) dem_small_islands(d, b, sm);
+    else if (b < nb_small + nb_islands) dem_islands(d, b - nb_small, nb_islands, sm);
+    else dem_free(d, b - nb_small - nb_islands, nb_free, inside);
 }
 
 __global__ void k_contacts(const double *__restrict__ x, const double *__restrict__ r, int np, int nx,
@@ -1439,7 +1574,7 @@ cudaError_t launch_dem_local(const DemArgs &d, cudaStream_t s) {
     // np/2 of two or more
     const int nb_islands = blocks_for(d.np / 5 + 1, ISL_WARPS);
     const int nb_small = blocks_for(blocks_for(d.np / 2 + 1, SMALL_PER_WARP), ISL_WARPS);
-    const int nb_free = blocks_for(d.np, LOCAL_THREADS);
+    const int nb_free = blocks_for(d.np, FREE_GROUP);
     return launch_dependent(k_dem_local, nb_islands + nb_small + nb_free, LOCAL_THREADS, 0, s, true, d, nb_islands,
                             nb_small);
 }
