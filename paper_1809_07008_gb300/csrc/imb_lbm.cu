@@ -403,7 +403,7 @@ k_stream_collide(const __grid_constant__ CUtensorMap tmap_n, const __grid_consta
     const bool smag = a.smag_coef > 0.0f;
     fin += a.origin;    // node (0, 0) of plane 0
     fout += a.origin;
-    // on small lattices launched as a programmatic dependent of the previous kernel in the
+    // on lattices of one wave launched as a programmatic dependent of the previous kernel in the
     // stream: nothing that kernel writes or reads is touched before it has completed
     cudaGridDependencySynchronize();
 
@@ -617,14 +617,20 @@ k_stream_collide(const __grid_constant__ CUtensorMap tmap_n, const __grid_consta
             if (SMALL || h == UPT - 1) {   // small lattices: the partials of each unit apart
                 double *tf = tile_force + ((size_t)ti.x * (SMALL ? UPT : 1) + (SMALL ? h : 0)) * (TILE_CAND * 3);
                 for (int i = lane; i < nc * 3; i += 32) {
+                    // the warps' sums in pairs of FP32 (the rounding of every add kept: 48 bits),
+                    // to FP64 at the end: eight FP64 adds and conversions in a row, 64 cycles each,
+                    // held back the copies of the next unit
                     float *pa = acc_t + i * WARPS;
-                    double v = 0.0;
+                    float hi = pa[0], lo = 0.0f;
+                    pa[0] = 0.0f;
 #pragma unroll
-                    for (int w = 0; w < WARPS; ++w) {
-                        v += (double)pa[w];
+                    for (int w = 1; w < WARPS; ++w) {
+                        const float b = pa[w], t = __fadd_rn(hi, b), bb = __fsub_rn(t, hi);
+                        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, bb)), __fsub_rn(b, bb)));
+                        hi = t;
                         pa[w] = 0.0f;
                     }
-                    tf[i] = v;
+                    tf[i] = (double)hi + (double)lo;
                 }
             }
             __syncwarp();
@@ -656,25 +662,21 @@ k_stream_collide(const __grid_constant__ CUtensorMap tmap_n, const __grid_consta
 // Force and torque of particle p: the sum of its partial sums over the tiles whose
 // candidate lists hold it, in a fixed order (the 3 x 3 tiles around its bin, row by row), so
 // that the result does not depend on the order in which the tiles were worked.
-__device__ __forceinline__ void force_gather(const LatticeArgs &a, const double *__restrict__ tile_force, int p) {
+__device__ __forceinline__ void force_gather(const LatticeArgs &a, const double *__restrict__ tile_force, int i) {
+    const int p = i / 3, c = i - 3 * p;   // a lane per component: an FP64 add takes a warp 64 cycles
     int e[9];
 #pragma unroll
     for (int j = 0; j < 9; ++j) e[j] = a.pslot[9 * p + j];
-    double fx = 0.0, fy = 0.0, tz = 0.0;
+    double f = 0.0;
 #pragma unroll
     for (int j = 0; j < 9; ++j)
         if (e[j] >= 0) {   // entry tile * TILE_CAND + slot; tf_units partial sets per tile
             const int t = e[j] / TILE_CAND, sl = e[j] % TILE_CAND;
-            for (int v = 0; v < a.tf_units; ++v) {
-                const double *tf = tile_force + (((size_t)t * a.tf_units + v) * TILE_CAND + sl) * 3;
-                fx += tf[0];
-                fy += tf[1];
-                tz += tf[2];
-            }
+            for (int v = 0; v < a.tf_units; ++v)
+                f += tile_force[(((size_t)t * a.tf_units + v) * TILE_CAND + sl) * 3 + c];
         }
-    a.F[2 * p] = fx;
-    a.F[2 * p + 1] = fy;
-    a.T[p] = tz;
+    if (c < 2) a.F[2 * p + c] = f;
+    else a.T[p] = f;
 }
 
 // Per-tile candidate lists: one warp per tile gathers the particles of the 3 x 3
@@ -979,11 +981,11 @@ __device__ __forceinline__ void fill_ghosts(S *f, const LatticeArgs &a, int i) {
 template <typename S>
 __global__ void __launch_bounds__(256) k_step_tail(const LatticeArgs a, const double *__restrict__ tile_force,
                                                    S *f, int nbf) {
-    cudaGridDependencySynchronize();   // on small lattices a programmatic dependent of the stream-collide launch
+    cudaGridDependencySynchronize();   // on lattices of one wave a programmatic dependent of the stream-collide launch
     cudaTriggerProgrammaticLaunchCompletion();
     if ((int)blockIdx.x < nbf) {
-        const int p = blockIdx.x * blockDim.x + threadIdx.x;
-        if (p < a.np) force_gather(a, tile_force, p);
+        const int i = blockIdx.x * blockDim.x + threadIdx.x;
+        if (i < 3 * a.np) force_gather(a, tile_force, i);
     } else {
         const int i = (blockIdx.x - nbf) * blockDim.x + threadIdx.x;
         if (i < edge_nodes(a.nx, a.ny)) fill_ghosts(f, a, i);
@@ -1009,24 +1011,6 @@ cudaError_t launch_init_populations(void *f, int storage, const LatticeArgs &a, 
         k_init<S><<<grid, 256, 0, s>>>((S *)f, a, rho0, ux0, uy0);
         return cudaGetLastError();
     });
-}
-
-static cudaError_t step_tail(void *f, int storage, const LatticeArgs &a, const double *tile_force, int nbf,
-                             cudaStream_t s) {
-    return by_storage(storage, [&](auto tag) {
-        using S = std::remove_pointer_t<decltype(tag)>;
-        const int nbg = (edge_nodes(a.nx, a.ny) + 255) / 256;
-        return launch_dependent(k_step_tail<S>, nbf + nbg, 256, 0, s, a.tf_units == SMALL_UPT, a, tile_force, (S *)f,
-                                nbf);
-    });
-}
-
-cudaError_t launch_fill_ghosts(void *f, int storage, const LatticeArgs &a, cudaStream_t s) {
-    return step_tail(f, storage, a, nullptr, 0, s);
-}
-
-cudaError_t launch_step_tail(void *f, int storage, const LatticeArgs &a, const double *tile_force, cudaStream_t s) {
-    return step_tail(f, storage, a, tile_force, (a.np + 255) / 256, s);
 }
 
 template <typename S, bool FORCED, bool SMALL>
@@ -1058,6 +1042,31 @@ int stream_collide_resident_blocks(int storage) {
     return per_sm * device_sms();
 }
 
+// Whether all blocks of a lattice's stream-collide are resident at once (eight-row units, or no
+// more tiles than the persistent grid has blocks).  Then it and k_step_tail are launched as
+// programmatic dependents: a step is a few microseconds, of which the launches are a good part
+// beside them.  On lattices of several waves the dependent launch cost 0.7 to 4 %.
+static bool one_wave(int storage, const LatticeArgs &a) {
+    return a.tf_units == SMALL_UPT || a.nbx * a.nby <= stream_collide_resident_blocks(storage);
+}
+
+static cudaError_t step_tail(void *f, int storage, const LatticeArgs &a, const double *tile_force, int nbf,
+                             cudaStream_t s) {
+    return by_storage(storage, [&](auto tag) {
+        using S = std::remove_pointer_t<decltype(tag)>;
+        const int nbg = (edge_nodes(a.nx, a.ny) + 255) / 256;
+        return launch_dependent(k_step_tail<S>, nbf + nbg, 256, 0, s, one_wave(storage, a), a, tile_force, (S *)f, nbf);
+    });
+}
+
+cudaError_t launch_fill_ghosts(void *f, int storage, const LatticeArgs &a, cudaStream_t s) {
+    return step_tail(f, storage, a, nullptr, 0, s);
+}
+
+cudaError_t launch_step_tail(void *f, int storage, const LatticeArgs &a, const double *tile_force, cudaStream_t s) {
+    return step_tail(f, storage, a, tile_force, (3 * a.np + 255) / 256, s);
+}
+
 cudaError_t launch_stream_collide(const void *fin, void *fout, int storage, const LatticeArgs &a,
                                   const CUtensorMap *tmap_narrow, const CUtensorMap *tmap_wide,
                                   const TileCand *tiles, double *tile_force, bool small, cudaStream_t s) {
@@ -1070,7 +1079,7 @@ cudaError_t launch_stream_collide(const void *fin, void *fout, int storage, cons
             const int grid = SM ? ntiles * Box<S, true>::UPT
                                 : std::min(ntiles, stream_collide_per_sm<S, F, false>() * device_sms());
             if (SM) stream_collide_per_sm<S, F, true>();   // sets the shared-memory attribute
-            return launch_dependent(k_stream_collide<S, F, SM>, grid, BLOCK, Box<S, SM>::SMEM_BYTES, s, SM,
+            return launch_dependent(k_stream_collide<S, F, SM>, grid, BLOCK, Box<S, SM>::SMEM_BYTES, s, one_wave(storage, a),
                                     *tmap_narrow, *tmap_wide, (const S *)fin, (S *)fout, a, tiles, ntiles, tile_force);
         };
         const bool forced = a.Fx != 0.0f || a.Fy != 0.0f;
