@@ -188,6 +188,7 @@ static LatticeArgs lattice_args(const imb_ctx *c) {
     a.pbin = c->pbin;
     a.pslot = c->pslot;
     a.pivl = c->pivl;
+    a.Jsum = nullptr;
     a.tf_units = c->small ? SMALL_UPT : 1;
     return a;
 }
@@ -676,9 +677,12 @@ static int dem_cycle(imb_ctx *c, bool zero_forces) {
     return rebuild_table(c, c->xs, zero_forces);
 }
 
-static int lattice_step(imb_ctx *c) {
+// from the populations in `in` (tensor maps tm) to `out`; forces: the particles' forces too, their
+// drag added to Jsum when given
+static int lattice_step_to(imb_ctx *c, const void *in, const CUtensorMap *tm, void *out, bool forces, double *Jsum) {
     // every particle's force and torque are written whole by the force gather below
     LatticeArgs a = lattice_args(c);
+    a.Jsum = Jsum;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (c->timing) {
         while (c->events.size() < c->ev_used + 2) {
@@ -693,16 +697,21 @@ static int lattice_step(imb_ctx *c) {
         CK(cudaEventRecordWithFlags(e0, c->stream, c->capturing ? cudaEventRecordExternal : cudaEventRecordDefault),
            "event record");
     }
-    CK(launch_stream_collide(c->fbuf[c->cur], c->fbuf[c->cur ^ 1], c->p.storage, a, &c->tmap[c->cur][0],
-                             &c->tmap[c->cur][1], c->tiles, c->tile_force, c->small, c->stream),
+    CK(launch_stream_collide(in, out, c->p.storage, a, &tm[0], &tm[1], c->tiles, c->tile_force, c->small, c->stream),
        "stream-collide");
-    CK(launch_step_tail(c->fbuf[c->cur ^ 1], c->p.storage, a, c->tile_force, c->stream), "forces and ghosts");
+    if (forces) CK(launch_step_tail(out, c->p.storage, a, c->tile_force, c->stream), "forces and ghosts");
+    else CK(launch_fill_ghosts(out, c->p.storage, a, c->stream), "ghosts");
     c->launches += 2;
     if (c->timing)
         CK(cudaEventRecordWithFlags(e1, c->stream, c->capturing ? cudaEventRecordExternal : cudaEventRecordDefault),
            "event record");
-    c->cur ^= 1;
     return IMB_OK;
+}
+
+static int lattice_step(imb_ctx *c) {
+    const int rc = lattice_step_to(c, c->fbuf[c->cur], c->tmap[c->cur], c->fbuf[c->cur ^ 1], true, nullptr);
+    if (!rc) c->cur ^= 1;
+    return rc;
 }
 
 // Steps from a CUDA graph: `dem` one coupling cycle with the DEM (DEM, particle map,
@@ -1091,15 +1100,41 @@ extern "C" const char *imb_last_error(imb_ctx *c) {
 // time) or binomial (a fixed number of snapshots placed by the recursive binomial schedule).
 namespace {
 
+// a state: the post-collision populations a step starts from, with their tensor maps
+struct GradState {
+    void *p = nullptr;
+    CUtensorMap tm[2];
+};
+
 struct GradBufs {
     size_t ncell = 0, state = 0, sb = 0;   // cells, floats per state, bytes per state
-    DevTmp<float> lam, Eb, fin;
-    DevTmp<double> acc, gE, gx, Fsave;
+    DevTmp<float> lam, Eb, states;
+    DevTmp<double> acc, gE, gx, Fsave, Jsum;
     DevTmp<int> cnt, ids;
     DevTmp<float> epsb;
     float *lam1 = nullptr, *lam0 = nullptr;   // d J / d f(t+1), d J / d f(t)
     float inv_T = 0.0f;
+    GradState work[2], fin;          // the context's two buffers, the state after the T steps
+    std::vector<GradState> kept;     // checkpoints, segment states or snapshots
 };
+
+// n states of the call's own, each stepped from and into in place (no copies between them); the
+// padding of their frames is cleared once, as the context's buffers are
+int grad_states(imb_ctx *c, GradBufs &g, size_t n) {
+    CK(dalloc(&g.states.p, g.state * (n + 1)), "states");
+    CK(cudaMemsetAsync(g.states.p, 0, g.sb * (n + 1), c->stream), "clear");
+    g.kept.resize(n);
+    for (size_t k = 0; k <= n; ++k) {
+        GradState &st = k < n ? g.kept[k] : g.fin;
+        st.p = g.states.p + g.state * k;
+        for (int wide = 0; wide < 2; ++wide) CK(make_tensor_map(c, st.p, &st.tm[wide], wide), "TMA descriptor");
+    }
+    for (int b = 0; b < 2; ++b) {
+        g.work[b].p = c->fbuf[b];
+        for (int wide = 0; wide < 2; ++wide) g.work[b].tm[wide] = c->tmap[b][wide];
+    }
+    return IMB_OK;
+}
 
 int grad_prepare(imb_ctx *c, int T, GradBufs &g) {
     if (c->p.dem_on || c->C_smag != 0.0 || c->p.Fx != 0.0 || c->p.Fy != 0.0 || c->p.eps_mode != IMB_EPS_EXACT ||
@@ -1123,17 +1158,18 @@ int grad_prepare(imb_ctx *c, int T, GradBufs &g) {
     g.sb = g.state * sizeof(float);
     g.inv_T = 1.0f / (float)T;
     CK(dalloc(&g.lam.p, 2 * g.state), "adjoint buffers");
-    CK(dalloc(&g.fin.p, g.state), "final state");
     CK(dalloc(&g.Eb.p, g.ncell), "solid ratio");
     CK(dalloc(&g.gE.p, g.ncell), "solid-ratio gradient");
     CK(dalloc(&g.acc.p, 4), "accumulators");
     CK(dalloc(&g.gx.p, 2 * (size_t)std::max(np, 1)), "position gradient");
     CK(dalloc(&g.Fsave.p, 3 * (size_t)std::max(np, 1)), "force copy");
+    CK(dalloc(&g.Jsum.p, (size_t)std::max(np, 1)), "drag sums");
     CK(dalloc(&g.cnt.p, g.ncell), "cell map");
     CK(dalloc(&g.ids.p, g.ncell * MAX_SLOTS), "cell map");
     CK(dalloc(&g.epsb.p, g.ncell * MAX_SLOTS), "cell map");
     cudaStream_t s = c->stream;
     CK(cudaMemsetAsync(g.acc.p, 0, 4 * sizeof(double), s), "clear");
+    CK(cudaMemsetAsync(g.Jsum.p, 0, (size_t)std::max(np, 1) * sizeof(double), s), "clear");
     CK(cudaMemsetAsync(g.gE.p, 0, g.ncell * sizeof(double), s), "clear");
     CK(cudaMemsetAsync(g.gx.p, 0, 2 * (size_t)std::max(np, 1) * sizeof(double), s), "clear");
     CK(cudaMemsetAsync(g.lam.p, 0, 2 * g.sb, s), "clear");
@@ -1149,21 +1185,9 @@ int grad_prepare(imb_ctx *c, int T, GradBufs &g) {
     return IMB_OK;
 }
 
-// one forward step whose drag enters J
-int grad_forward_step(imb_ctx *c, GradBufs &g) {
-    int rc = lattice_step(c);
-    if (rc) return rc;
-    if (c->np > 0) {
-        CK(launch_drag_sum(c->F, c->np, g.acc.p, c->stream), "drag");
-        c->launches++;
-    }
-    return IMB_OK;
-}
-
-// the state after the T steps and its forces, kept for the end of the call
-int grad_keep_final(imb_ctx *c, GradBufs &g) {
+// the forces of the last step, kept to the end of the call
+int grad_keep_forces(imb_ctx *c, GradBufs &g) {
     cudaStream_t s = c->stream;
-    CK(cudaMemcpyAsync(g.fin.p, c->fbuf[c->cur], g.sb, cudaMemcpyDeviceToDevice, s), "final state");
     if (c->np > 0) {
         CK(cudaMemcpyAsync(g.Fsave.p, c->F, 16 * (size_t)c->np, cudaMemcpyDeviceToDevice, s), "forces");
         CK(cudaMemcpyAsync(g.Fsave.p + 2 * (size_t)c->np, c->T, 8 * (size_t)c->np, cudaMemcpyDeviceToDevice, s),
@@ -1176,24 +1200,22 @@ int grad_keep_final(imb_ctx *c, GradBufs &g) {
 // solid-ratio terms; then, for t >= 1, the transpose of the inlet/outlet rule that produced
 // f(t) from state t (it adds the inlet-velocity term), so that the next unit starts from the
 // full d J / d f(t).
-int grad_unit(imb_ctx *c, GradBufs &g, int t, const float *S0) {
-    LatticeArgs a = lattice_args(c);
-    cudaStream_t s = c->stream;
-    CK(launch_adjoint_step(g.lam1, S0, g.lam0, a, g.Eb.p, g.gE.p, g.inv_T, g.acc.p + 1, s), "adjoint step");
+int grad_unit(imb_ctx *c, GradBufs &g, int t, const GradState &st) {
+    CK(launch_adjoint_step(g.lam1, (const float *)st.p, g.lam0, lattice_args(c), g.Eb.p, g.gE.p, g.inv_T, g.acc.p + 1,
+                           t >= 1 && c->p.bc_x == IMB_BC_INLET_OUTLET, g.acc.p + 2, c->stream),
+       "adjoint step");
     c->launches++;
     std::swap(g.lam1, g.lam0);
-    if (t >= 1 && c->p.bc_x == IMB_BC_INLET_OUTLET) {
-        CK(launch_adjoint_inlet(g.lam1, S0, a, g.acc.p + 2, s), "adjoint inlet");
-        c->launches++;
-    }
     return IMB_OK;
 }
 
 int grad_finish(imb_ctx *c, GradBufs &g, int T, double *J, double *dJ_duin, double *dJ_dtau, double *dJ_dx) {
     cudaStream_t s = c->stream;
     const int np = c->np;
-    CK(cudaMemcpyAsync(c->fbuf[c->cur], g.fin.p, g.sb, cudaMemcpyDeviceToDevice, s), "restore final state");
+    CK(cudaMemcpyAsync(c->fbuf[c->cur], g.fin.p, g.sb, cudaMemcpyDeviceToDevice, s), "final state");
     if (np > 0) {
+        CK(launch_drag_sum(g.Jsum.p, np, g.acc.p, s), "drag");
+        c->launches++;
         CK(cudaMemcpyAsync(c->F, g.Fsave.p, 16 * (size_t)np, cudaMemcpyDeviceToDevice, s), "forces");
         CK(cudaMemcpyAsync(c->T, g.Fsave.p + 2 * (size_t)np, 8 * (size_t)np, cudaMemcpyDeviceToDevice, s), "torques");
         CK(launch_position_grad(g.cnt.p, g.ids.p, g.gE.p, c->x, c->r, c->nx, c->ny, c->p.bc_x, c->p.bc_y, g.gx.p, s),
@@ -1311,29 +1333,33 @@ extern "C" int imb_drag_gradient(imb_ctx *c, int T, int checkpoint_every, double
     GradBufs g;
     int rc = grad_prepare(c, T, g);
     if (rc) return rc;
-    const int K = checkpoint_every, nck = (T + K - 1) / K;
-    const size_t state = g.state, sb = g.sb;
-    DevTmp<float> ck, seg;
-    CK(dalloc(&ck.p, state * nck), "checkpoints");
-    CK(dalloc(&seg.p, state * (size_t)std::min(K, T)), "segment states");
+    const int K = checkpoint_every, nck = (T + K - 1) / K, last0 = (nck - 1) * K;
+    // states: the checkpoints 0, K, 2K ..., then the states between two checkpoints; every step
+    // reads and writes them where they are kept, so nothing is copied between the first state and
+    // the last, and the states of the last segment are kept on the way forward
+    const int nseg = std::min(K, T) - 1;
+    if ((rc = grad_states(c, g, (size_t)nck + nseg))) return rc;
     cudaStream_t s = c->stream;
-    // forward: every K-th state kept, the drag of every step summed
+    double *Jsum = c->np > 0 ? g.Jsum.p : nullptr;
+    auto between = [&](int t, int t0) -> GradState & { return t == t0 ? g.kept[t0 / K] : g.kept[nck + (t - t0 - 1)]; };
+    CK(cudaMemcpyAsync(g.kept[0].p, c->fbuf[c->cur], g.sb, cudaMemcpyDeviceToDevice, s), "checkpoint");
+    const GradState *at = &g.kept[0];
     for (int t = 0; t < T; ++t) {
-        if (t % K == 0)
-            CK(cudaMemcpyAsync(ck.p + state * (t / K), c->fbuf[c->cur], sb, cudaMemcpyDeviceToDevice, s), "checkpoint");
-        if ((rc = grad_forward_step(c, g))) return rc;
+        const GradState *to = t + 1 == T         ? &g.fin
+                              : (t + 1) % K == 0 ? &g.kept[(t + 1) / K]
+                              : t >= last0       ? &between(t + 1, last0)
+                                                 : &g.work[(t + 1) & 1];
+        if ((rc = lattice_step_to(c, at->p, at->tm, to->p, true, Jsum))) return rc;
+        at = to;
     }
-    if ((rc = grad_keep_final(c, g))) return rc;
+    if ((rc = grad_keep_forces(c, g))) return rc;
     // backward, one checkpoint segment at a time: recompute its states, then walk back
     for (int j = nck - 1; j >= 0; --j) {
         const int t0 = j * K, t1 = std::min(T, t0 + K);
-        CK(cudaMemcpyAsync(c->fbuf[c->cur], ck.p + state * j, sb, cudaMemcpyDeviceToDevice, s), "restore");
-        for (int t = t0; t < t1; ++t) {
-            CK(cudaMemcpyAsync(seg.p + state * (t - t0), c->fbuf[c->cur], sb, cudaMemcpyDeviceToDevice, s), "segment");
-            if (t + 1 < t1 && (rc = lattice_step(c))) return rc;
-        }
+        for (int t = t0; t + 1 < t1 && t0 != last0; ++t)
+            if ((rc = lattice_step_to(c, between(t, t0).p, between(t, t0).tm, between(t + 1, t0).p, false, nullptr))) return rc;
         for (int t = t1 - 1; t >= t0; --t)
-            if ((rc = grad_unit(c, g, t, seg.p + state * (t - t0)))) return rc;
+            if ((rc = grad_unit(c, g, t, between(t, t0)))) return rc;
     }
     return grad_finish(c, g, T, J, dJ_duin, dJ_dtau, dJ_dx);
 }
@@ -1347,39 +1373,40 @@ extern "C" int imb_drag_gradient_binomial(imb_ctx *c, int T, int snapshots, doub
     if (rc) return rc;
     Sched sc;
     binomial_schedule(T, snapshots, sc);
-    const size_t state = g.state, sb = g.sb;
-    DevTmp<float> snap;
-    CK(dalloc(&snap.p, state * sc.slot_t.size()), "snapshots");
+    if ((rc = grad_states(c, g, sc.slot_t.size()))) return rc;
     std::vector<int> slot_t(sc.slot_t.size(), -1);
     cudaStream_t s = c->stream;
+    double *Jsum = c->np > 0 ? g.Jsum.p : nullptr;
     int cur_t = 0, done = 0;   // time of the working state; steps whose drag is in J
+    const GradState *at = &g.work[c->cur];
     for (size_t k = 0; k < sc.ops.size(); k += 2) {
         const int kind = sc.ops[k], v = sc.ops[k + 1];
         if (kind == IMB_CK_ADVANCE) {
             for (int n = 0; n < v; ++n, ++cur_t) {
-                if (cur_t == done) {   // first pass over this step: its drag enters J
-                    if ((rc = grad_forward_step(c, g))) return rc;
-                    ++done;
-                } else if ((rc = lattice_step(c))) {
-                    return rc;
-                }
+                // the step before a snapshot is taken writes it in place
+                const bool store = n + 1 == v && k + 2 < sc.ops.size() && sc.ops[k + 2] == IMB_CK_STORE;
+                const GradState *to = store ? &g.kept[sc.ops[k + 3]] : at == &g.work[0] ? &g.work[1] : &g.work[0];
+                const bool first = cur_t == done;   // first pass over this step: its drag enters J
+                if ((rc = lattice_step_to(c, at->p, at->tm, to->p, first, first ? Jsum : nullptr))) return rc;
+                done += first;
+                at = to;
             }
         } else if (kind == IMB_CK_STORE) {
-            CK(cudaMemcpyAsync(snap.p + state * v, c->fbuf[c->cur], sb, cudaMemcpyDeviceToDevice, s), "snapshot");
+            if (at != &g.kept[v])
+                CK(cudaMemcpyAsync(g.kept[v].p, at->p, g.sb, cudaMemcpyDeviceToDevice, s), "snapshot");
             slot_t[v] = cur_t;
         } else if (kind == IMB_CK_RESTORE) {
-            CK(cudaMemcpyAsync(c->fbuf[c->cur], snap.p + state * v, sb, cudaMemcpyDeviceToDevice, s), "restore");
+            at = &g.kept[v];
             cur_t = slot_t[v];
         } else {   // IMB_CK_ADJOINT of step v from the working state
             if (v != cur_t) return fail(c, IMB_E_CUDA, "internal: checkpoint schedule out of order");
             if (v == T - 1) {   // the first adjoint: the last forward step completes J and the final state
                 if (done != T - 1) return fail(c, IMB_E_CUDA, "internal: checkpoint schedule skipped a step");
-                if ((rc = grad_forward_step(c, g))) return rc;
+                if ((rc = lattice_step_to(c, at->p, at->tm, g.fin.p, true, Jsum))) return rc;
                 ++done;
-                if ((rc = grad_keep_final(c, g))) return rc;
-                c->cur ^= 1;   // the step wrote the other buffer: state T - 1 is still in this one
+                if ((rc = grad_keep_forces(c, g))) return rc;
             }
-            if ((rc = grad_unit(c, g, v, (const float *)c->fbuf[c->cur]))) return rc;
+            if ((rc = grad_unit(c, g, v, *at))) return rc;
         }
     }
     return grad_finish(c, g, T, J, dJ_duin, dJ_dtau, dJ_dx);

@@ -84,6 +84,7 @@ struct LatticeArgs {
                                // reaches into, [x, y], and covers whole, [z, w] (exact-area mode)
     int *pslot;                // [np][9] tile * TILE_CAND + slot of the particle in the candidate lists of the
                                // 3 x 3 tiles around its bin (row by row), -1 where it is not a candidate
+    double *Jsum;              // [np] NULL, or each particle's F_x is added to it (the drag gradient's J)
     int tf_units;              // force partials per tile: 1, or SMALL_UPT when each work unit keeps its own
 };
 
@@ -156,12 +157,12 @@ cudaError_t launch_gather(const void *fin, int storage, const LatticeArgs &a, do
                           double *rho, double *ux, double *uy, cudaStream_t s);
 cudaError_t launch_cell_map(const LatticeArgs &a, int *count, int *ids, float *eps, cudaStream_t s);
 // drag gradient (imb_adjoint.cu)
-cudaError_t launch_drag_sum(const double *F, int np, double *acc, cudaStream_t s);
+cudaError_t launch_drag_sum(const double *Jsum, int np, double *acc, cudaStream_t s);
 cudaError_t launch_cell_E(const int *count, const float *eps, size_t ncell, float *E, cudaStream_t s);
-cudaError_t launch_adjoint_inlet(float *lam, const float *S1, const LatticeArgs &a, double *g_uin,
-                                 cudaStream_t s);
+// inlet: followed by the transpose of the inlet and outlet columns of the pull from S0
 cudaError_t launch_adjoint_step(const float *lam1, const float *S0, float *lam0, const LatticeArgs &a,
-                                const float *E, double *gE, float inv_T, double *g_tau, cudaStream_t s);
+                                const float *E, double *gE, float inv_T, double *g_tau, bool inlet, double *g_uin,
+                                cudaStream_t s);
 cudaError_t launch_position_grad(const int *count, const int *ids, const double *gE, const double *x,
                                  const double *r, int nx, int ny, int bc_x, int bc_y, double *dJ_dx,
                                  cudaStream_t s);

@@ -677,6 +677,7 @@ __device__ __forceinline__ void force_gather(const LatticeArgs &a, const double 
         }
     if (c < 2) a.F[2 * p + c] = f;
     else a.T[p] = f;
+    if (c == 0 && a.Jsum) a.Jsum[p] += f;
 }
 
 // Per-tile candidate lists: one warp per tile gathers the particles of the 3 x 3
