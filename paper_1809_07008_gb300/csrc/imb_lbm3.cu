@@ -176,14 +176,16 @@ __device__ __forceinline__ float f32_of(float v) { return v; }
 __device__ __forceinline__ float f32_of(__half v) { return __half2float(v); }
 __device__ __forceinline__ float f32_of(__nv_bfloat16 v) { return __bfloat162float(v); }
 
-// the 19 stored values a cell pulls (Eq. 1), as stored: interior cells by the per-direction
-// offsets, edge cells with the wrap and wall rules
+// the 19 stored values a cell pulls (Eq. 1), as stored: rows inside the y and z edges (the same
+// for a whole warp) by the per-direction offsets, the periodic wrap in x by the base of each c_x;
+// the other rows with the wrap and wall rules
 template <typename S>
 __device__ __forceinline__ void fetch3(const S *__restrict__ fin, const Args3 &a, int x, int y, int z, S (&r)[19]) {
     const size_t cell = ((size_t)z * a.ny + y) * a.nx + x;
-    if (x > 0 && x < a.nx - 1 && y > 0 && y < a.ny - 1 && z > 0 && z < a.nz - 1) {
+    if (y > 0 && y < a.ny - 1 && z > 0 && z < a.nz - 1) {
+        const S *p0 = fin + cell, *pm = x == 0 ? p0 + a.nx : p0, *pp = x == a.nx - 1 ? p0 - a.nx : p0;
 #pragma unroll
-        for (int q = 0; q < 19; ++q) r[q] = ld_raw3(fin + (cell + a.off[q]));
+        for (int q = 0; q < 19; ++q) r[q] = ld_raw3((cx3(q) == 0 ? p0 : cx3(q) > 0 ? pm : pp) + a.off[q]);
         return;
     }
 #pragma unroll
@@ -300,34 +302,52 @@ __device__ __forceinline__ void sphere_force(float Bp, float rho, float jx, floa
     fo[5] = r[0] * fo[1] - r[1] * fo[0];
 }
 
-// the plain variant of collide3_gen below (one sphere per cell, tau fixed), written out on its
-// own: folding the general function down to this case compiled to a 3 % slower FP32 kernel
-template <typename S>
-__device__ __forceinline__ int collide3_plain(const float (&d)[19], const Args3 &a, int x, int y, int z, size_t cell,
-                                        const unsigned *__restrict__ map, const Sph3 *__restrict__ sph,
-                                        S *__restrict__ fout, float (&fo)[6], bool &unstable) {
-    // the 18 moving directions as nine pairs (q, q + 1) = (q, -q), q odd, computed with FP32x2
-    // instructions: their terms differ only in the sign of the odd parts
+// Collision of one cell from its pulled values d: moments (Eqs. 3-4, Guo half-force shift), BGK with
+// Guo forcing, Eqs. 12-14 where a sphere covers the cell, the 19 stores; returns the covering sphere
+// of lower index (-1: none) with its force and torque contribution in fo (Eqs. 15-16).  word: the
+// cell's first map word, fetched with the populations.  GEN: the general variant, with a second
+// covering sphere (its share goes to the thread's column sums) and the Smagorinsky relaxation time;
+// the host launches it only when some cell holds two spheres or C_smag > 0.
+//
+// The kernel issues more than it waits for memory (half the cycles in FP32, more in 16 bits), so
+// the algebra is arranged for few instructions.  The 18 moving directions are nine pairs (q, -q),
+// q odd, in FP32x2 operations.  A fluid cell needs no non-equilibrium parts: its update is
+//   d*_{+-q} = (1 - omega) d_{+-q} + w_q [T0 + c.u (4.5 omega rho c.u + 9 s c.F) +- c.J],
+//   T0 = omega (drho - 1.5 rho u^2) - 3 s u.F,  J = 3 (omega j + s F),  s = 1 - omega / 2;
+// a covered cell is (1 - B) times that plus B (n_{-q} + f^eq_q(rho, u_s) - w_q), and the
+// closure's momentum flux comes from the second moments, Pi = sum c c d - (drho / 3 + rho u u).
+// Kernel time on 16 M cells with one sphere 505 -> 453 us FP32 (5.4 TB/s), 446 -> 337 us FP16; the
+// 240 x 100 x 100 packed bed (GEN) 172 -> 105 us.  Three blocks an SM (80 registers, spills): 499,
+// 397 and 182 us; columns of 16 cells: 457, 347 and 111 us.
+template <bool GEN, typename S>
+__device__ __forceinline__ int collide3(const float (&d)[19], const Args3 &a, int x, int y, int z, size_t cell,
+                                        const unsigned word, const unsigned *__restrict__ map2,
+                                        const Sph3 *__restrict__ sph, S *__restrict__ fout, double *FT,
+                                        ForceSums &fs, float (&fo)[6], bool &unstable) {
     float2 P[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) P[k] = make_float2(d[2 * k + 1], d[2 * k + 2]);
-    float2 Sp[9];
+    float drho, s[9];
+    if constexpr (GEN) {
+        drho = d[0];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) Sp[k] = P[k];
-#pragma unroll
-    for (int h = 1; h < 9; h <<= 1)
-#pragma unroll
-        for (int k = 0; k + h < 9; k += 2 * h) Sp[k] = __fadd2_rn(Sp[k], Sp[k + h]);
-    const float drho = d[0] + (Sp[0].x + Sp[0].y);
-    float mx = 0.0f, my = 0.0f, mz = 0.0f;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {   // c_{-q} = -c_q: first moments from d_q - d_-q
-        const int q = 2 * k + 1;
-        const float Dk = P[k].x - P[k].y;
-        if (cx3(q)) mx += cx3(q) * Dk;
-        if (cy3(q)) my += cy3(q) * Dk;
-        if (cz3(q)) mz += cz3(q) * Dk;
+        for (int k = 0; k < 9; ++k) {
+            s[k] = P[k].x + P[k].y;
+            drho += s[k];
+        }
+    } else {
+        const float2 t = __fadd2_rn(__fadd2_rn(__fadd2_rn(P[0], P[1]), __fadd2_rn(P[2], P[3])),
+                                    __fadd2_rn(__fadd2_rn(P[4], P[5]), __fadd2_rn(P[6], P[7])));
+        const float2 u = __fadd2_rn(t, P[8]);
+        drho = d[0] + (u.x + u.y);
     }
+    float D[9];   // c_{-q} = -c_q: first moments from d_q - d_-q
+#pragma unroll
+    for (int k = 0; k < 9; ++k) D[k] = P[k].x - P[k].y;
+    // pairs: x, y, z, x+y, x-y, x+z, x-z, y+z, y-z
+    const float mx = D[0] + ((D[3] + D[4]) + (D[5] + D[6]));
+    const float my = D[1] + ((D[3] - D[4]) + (D[7] + D[8]));
+    const float mz = D[2] + ((D[5] - D[6]) + (D[7] - D[8]));
     const float rho = 1.0f + drho;
     const float jx = fmaf(0.5f, a.Fx, mx), jy = fmaf(0.5f, a.Fy, my), jz = fmaf(0.5f, a.Fz, mz);
     const float inv = __fdividef(1.0f, rho);
@@ -335,140 +355,46 @@ __device__ __forceinline__ int collide3_plain(const float (&d)[19], const Args3 
     const float uu = ux * ux + uy * uy + uz * uz;
     if (!(uu < 0.09f)) unstable = true;   // Mach guard, also catches NaN
     const float t = fmaf(-1.5f * rho, uu, drho);
-    const float2 t2 = make_float2(t, t);
-    // non-equilibrium parts (Eq. 2), shifted by w: n_{+-q} = d_{+-q} - w_q (t +- rho c.u (3 +- 4.5 c.u))
-    const float n0 = d[0] - w3(0) * t;
-    float2 N[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        const int q = 2 * k + 1;
-        const float cu = cdot3(q, ux, uy, uz), rcu = rho * cu;
-        const float2 X = __ffma2_rn(make_float2(rcu, -rcu), make_float2(fmaf(4.5f, cu, 3.0f), fmaf(-4.5f, cu, 3.0f)), t2);
-        N[k] = __ffma2_rn(make_float2(-w3(q), -w3(q)), X, P[k]);
-    }
-    const unsigned word = map[cell];
-    int sid = -1;
-    float B = 0.0f, usx = 0.0f, usy = 0.0f, usz = 0.0f, rx = 0.0f, ry = 0.0f, rz = 0.0f;
-    if (word) {   // Eq. 14 with the sub-cell solid ratio; u_s = v + w x r at the node
-        sid = (int)(word & ID_MASK) - 1;
-        const float eps = (float)(word >> ID_BITS) * a.inv_nsub3;
-        const float tm = a.tau - 0.5f;
-        B = __fdividef(eps * tm, (1.0f - eps) + tm);
-        const Sph3 Ps = sph[sid];
-        rx = (float)min_image(x - Ps.ci, a.nx) + 0.5f - Ps.fx;
-        ry = (float)(a.wall_y ? y - Ps.cj : min_image(y - Ps.cj, a.ny)) + 0.5f - Ps.fy;
-        rz = (float)min_image(z - Ps.ck, a.nz) + 0.5f - Ps.fz;
-        usx = Ps.vx + (Ps.wy * rz - Ps.wz * ry);
-        usy = Ps.vy + (Ps.wz * rx - Ps.wx * rz);
-        usz = Ps.vz + (Ps.wx * ry - Ps.wy * rx);
-    }
-    const float fl = 1.0f - B, sf = 1.0f - 0.5f * a.omega;
-    const float uF = ux * a.Fx + uy * a.Fy + uz * a.Fz;
-    // BGK with Guo forcing (its source divided by 1 - 1/(2 tau)), weighted by 1 - B:
-    // -omega n_q + sf w_q (3 (c_q.F - u.F) + 9 (c_q.u)(c_q.F)), for the pair (q, -q)
-    const float f0 = fmaf(-a.omega, n0, sf * (w3(0) * (-3.0f * uF)));
-    const float2 mo2 = make_float2(-a.omega, -a.omega), muF2 = make_float2(-uF, -uF);
-    auto fluid2 = [&](int k) {
-        const int q = 2 * k + 1;
-        const float cu = cdot3(q, ux, uy, uz), cF = cdot3(q, a.Fx, a.Fy, a.Fz);
-        const float e9 = 9.0f * cu * cF;
-        const float2 A = __fadd2_rn(make_float2(cF, -cF), muF2);
-        const float2 G = __ffma2_rn(make_float2(3.0f, 3.0f), A, make_float2(e9, e9));
-        const float sw = sf * w3(q);
-        return __ffma2_rn(mo2, N[k], __fmul2_rn(make_float2(sw, sw), G));
-    };
-    if (word) {   // Eq. 12 in shifted form: n_{-q} + (f^eq_q(u_s) - w_q) - d_q, weighted by B
-        const float uss = usx * usx + usy * usy + usz * usz;
-        const float ts = fmaf(-1.5f * rho, uss, drho);
-        const float2 ts2 = make_float2(ts, ts), B2 = make_float2(B, B), fl2 = make_float2(fl, fl);
-        Store<S>::st(fout + cell, d[0] + fmaf(B, n0 + w3(0) * ts - d[0], fl * f0));
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            const int q = 2 * k + 1;
-            const float cs = cdot3(q, usx, usy, usz), rcs = rho * cs;
-            const float2 Xs = __ffma2_rn(make_float2(rcs, -rcs), make_float2(fmaf(4.5f, cs, 3.0f), fmaf(-4.5f, cs, 3.0f)), ts2);
-            // n_{-q} + w_q Xs - d_q for q and -q
-            const float2 T = __fadd2_rn(__ffma2_rn(make_float2(w3(q), w3(q)), Xs, make_float2(N[k].y, N[k].x)),
-                                        make_float2(-P[k].x, -P[k].y));
-            const float2 v = __ffma2_rn(B2, T, __fmul2_rn(fl2, fluid2(k)));
-            const float2 o = __fadd2_rn(P[k], v);
-            Store<S>::st(fout + (size_t)q * a.plane + cell, o.x);
-            Store<S>::st(fout + (size_t)(q + 1) * a.plane + cell, o.y);
-        }
-    } else {      // no sphere: the fluid operator alone
-        Store<S>::st(fout + cell, d[0] + f0);
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            const int q = 2 * k + 1;
-            const float2 o = __fadd2_rn(P[k], fluid2(k));
-            Store<S>::st(fout + (size_t)q * a.plane + cell, o.x);
-            Store<S>::st(fout + (size_t)(q + 1) * a.plane + cell, o.y);
-        }
-    }
-    if (word) {   // Eqs. 15-16: force on the sphere B (rho u - rho u_s - F), torque r x force
-        fo[0] = B * (jx - rho * usx - a.Fx);
-        fo[1] = B * (jy - rho * usy - a.Fy);
-        fo[2] = B * (jz - rho * usz - a.Fz);
-        fo[3] = ry * fo[2] - rz * fo[1];
-        fo[4] = rz * fo[0] - rx * fo[2];
-        fo[5] = rx * fo[1] - ry * fo[0];
-    }
-    return sid;
-}
-
-// collision of one cell from its pulled values d, general variant: moments (Eqs. 3-4, Guo
-// half-force shift), the Smagorinsky relaxation time (when smag_coef > 0), BGK with Guo
-// forcing, Eqs. 12-14 where one or two spheres cover the cell, the 19 stores; returns the
-// covering sphere of lower index (-1: none) with its force and torque contribution in fo
-// (Eqs. 15-16); a second covering sphere's share goes to the thread's column sums.  The kernel runs it
-// only when some cell holds two spheres or C_smag > 0: its code in every cell's schedule
-// slowed the plain case by 9-13 %
-template <typename S>
-__device__ __forceinline__ int collide3_gen(const float (&d)[19], const Args3 &a, int x, int y, int z, size_t cell,
-                                        const unsigned *__restrict__ map, const unsigned *__restrict__ map2,
-                                        const Sph3 *__restrict__ sph, S *__restrict__ fout, double *FT,
-                                        ForceSums &fs, float (&fo)[6], bool &unstable) {
-    float drho = 0.0f, mx = 0.0f, my = 0.0f, mz = 0.0f;
-#pragma unroll
-    for (int q = 0; q < 19; ++q) {
-        drho += d[q];
-        if (cx3(q)) mx += cx3(q) * d[q];
-        if (cy3(q)) my += cy3(q) * d[q];
-        if (cz3(q)) mz += cz3(q) * d[q];
-    }
-    const float rho = 1.0f + drho;
-    const float jx = fmaf(0.5f, a.Fx, mx), jy = fmaf(0.5f, a.Fy, my), jz = fmaf(0.5f, a.Fz, mz);
-    const float inv = __fdividef(1.0f, rho);
-    const float ux = jx * inv, uy = jy * inv, uz = jz * inv;
-    const float uu = ux * ux + uy * uy + uz * uz;
-    if (!(uu < 0.09f)) unstable = true;   // Mach guard, also catches NaN
-    const float t = fmaf(-1.5f * rho, uu, drho);
-    float n[19];
-#pragma unroll
-    for (int q = 0; q < 19; ++q) {   // non-equilibrium parts (Eq. 2), shifted by w
-        const float cu = cdot3(q, ux, uy, uz);
-        n[q] = d[q] - w3(q) * fmaf(rho * cu, fmaf(4.5f, cu, 3.0f), t);
-    }
     float te = a.tau, omega = a.omega;
-    if (a.smag_coef > 0.0f) {   // tau_eff = (tau + sqrt(tau^2 + 18 sqrt(2) C^2 sqrt(Pi : Pi) / rho)) / 2
-        float pxx = 0.0f, pyy = 0.0f, pzz = 0.0f, pxy = 0.0f, pxz = 0.0f, pyz = 0.0f;
-#pragma unroll
-        for (int q = 1; q < 19; ++q) {   // Pi = sum_q c_q c_q n_q
-            if (cx3(q)) pxx += n[q];
-            if (cy3(q)) pyy += n[q];
-            if (cz3(q)) pzz += n[q];
-            if (cx3(q) && cy3(q)) pxy += cx3(q) * cy3(q) > 0 ? n[q] : -n[q];
-            if (cx3(q) && cz3(q)) pxz += cx3(q) * cz3(q) > 0 ? n[q] : -n[q];
-            if (cy3(q) && cz3(q)) pyz += cy3(q) * cz3(q) > 0 ? n[q] : -n[q];
-        }
+    if (GEN && a.smag_coef > 0.0f) {   // tau_eff = (tau + sqrt(tau^2 + 18 sqrt(2) C^2 sqrt(Pi : Pi) / rho)) / 2
+        const float sxy = s[3] + s[4], sxz = s[5] + s[6], syz = s[7] + s[8], th = drho * (1.0f / 3.0f);
+        const float pxx = fmaf(-jx, ux, (s[0] + (sxy + sxz)) - th);
+        const float pyy = fmaf(-jy, uy, (s[1] + (sxy + syz)) - th);
+        const float pzz = fmaf(-jz, uz, (s[2] + (sxz + syz)) - th);
+        const float pxy = fmaf(-jx, uy, s[3] - s[4]), pxz = fmaf(-jx, uz, s[5] - s[6]), pyz = fmaf(-jy, uz, s[7] - s[8]);
         const float Q = fmaf(pxx, pxx, fmaf(pyy, pyy, pzz * pzz)) + 2.0f * fmaf(pxy, pxy, fmaf(pxz, pxz, pyz * pyz));
         const float sq = Q > 0.0f ? Q * rsqrtf(Q) : 0.0f;   // sqrt(Q)
         const float disc = fmaf(a.smag_coef * sq, inv, a.tau * a.tau);
         te = 0.5f * (a.tau + disc * rsqrtf(disc));
         omega = __fdividef(1.0f, te);
     }
-    unsigned w1 = map[cell], w2 = 0u;
-    if (w1 && a.two_slots) {
+    const float sf = 1.0f - 0.5f * omega, om1 = 1.0f - omega;
+    const float uF = ux * a.Fx + uy * a.Fy + uz * a.Fz;
+    const float T0 = fmaf(omega, t, -3.0f * sf * uF), K = 4.5f * omega * rho, o3 = 3.0f * omega, s3 = 3.0f * sf;
+    const float Jx = fmaf(o3, jx, s3 * a.Fx), Jy = fmaf(o3, jy, s3 * a.Fy), Jz = fmaf(o3, jz, s3 * a.Fz);
+    const float s9x = 9.0f * sf * a.Fx, s9y = 9.0f * sf * a.Fy, s9z = 9.0f * sf * a.Fz;
+    const float2 om2 = make_float2(om1, om1);
+    // the fluid's d*_q and d*_-q
+    auto fluid2 = [&](int k) {
+        const int q = 2 * k + 1;
+        const float cu = cdot3(q, ux, uy, uz), cJ = cdot3(q, Jx, Jy, Jz);
+        const float ev = fmaf(cu, fmaf(K, cu, cdot3(q, s9x, s9y, s9z)), T0);
+        return __ffma2_rn(make_float2(w3(q), w3(q)), make_float2(ev + cJ, ev - cJ), __fmul2_rn(om2, P[k]));
+    };
+    const float f0 = fmaf(om1, d[0], w3(0) * T0);
+    if (!word) {
+        Store<S>::st(fout + cell, f0);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            const int q = 2 * k + 1;
+            const float2 o = fluid2(k);
+            Store<S>::st(fout + (size_t)q * a.plane + cell, o.x);
+            Store<S>::st(fout + (size_t)(q + 1) * a.plane + cell, o.y);
+        }
+        return -1;
+    }
+    unsigned w1 = word, w2 = 0u;
+    if (GEN && a.two_slots) {
         w2 = map2[cell];
         if (w2 && (w2 & ID_MASK) < (w1 & ID_MASK)) {   // the sphere of lower index first
             const unsigned tw = w1;
@@ -476,59 +402,61 @@ __device__ __forceinline__ int collide3_gen(const float (&d)[19], const Args3 &a
             w2 = tw;
         }
     }
-    int sid = -1;
-    float B = 0.0f, B1 = 0.0f, B2 = 0.0f;
-    float r1[3] = {0.0f, 0.0f, 0.0f}, u1[3] = {0.0f, 0.0f, 0.0f}, r2[3] = {0.0f, 0.0f, 0.0f}, u2[3] = {0.0f, 0.0f, 0.0f};
-    if (w1) {   // Eq. 14 with the summed sub-cell solid ratio, shared by the spheres' own ratios
-        sid = (int)(w1 & ID_MASK) - 1;
-        const unsigned c1 = w1 >> ID_BITS, c2 = w2 >> ID_BITS;
-        const float eps = fminf(1.0f, (float)(c1 + c2) * a.inv_nsub3);   // two spheres may overlap
-        const float tm = te - 0.5f;
-        B = __fdividef(eps * tm, (1.0f - eps) + tm);
-        B1 = B;
-        surface_velocity(sph[sid], a, x, y, z, r1, u1);
-        if (w2) {
-            const float inv_c = __fdividef(1.0f, (float)(c1 + c2));
-            B1 = B * ((float)c1 * inv_c);
-            B2 = B * ((float)c2 * inv_c);
-            surface_velocity(sph[(w2 & ID_MASK) - 1], a, x, y, z, r2, u2);
-        }
+    // Eq. 14 with the (summed) sub-cell solid ratio, shared by the spheres' own ratios
+    const int sid = (int)(w1 & ID_MASK) - 1;
+    const unsigned c1 = w1 >> ID_BITS, c2 = GEN ? w2 >> ID_BITS : 0u;
+    const float eps = GEN ? fminf(1.0f, (float)(c1 + c2) * a.inv_nsub3) : (float)c1 * a.inv_nsub3;   // two may overlap
+    const float tm = te - 0.5f;
+    const float B = __fdividef(eps * tm, (1.0f - eps) + tm), fl = 1.0f - B;
+    float B1 = B, B2 = 0.0f, r1[3], u1[3], r2[3] = {0.0f, 0.0f, 0.0f}, u2[3] = {0.0f, 0.0f, 0.0f};
+    surface_velocity(sph[sid], a, x, y, z, r1, u1);
+    if (GEN && w2) {
+        const float inv_c = __fdividef(1.0f, (float)(c1 + c2));
+        B1 = B * ((float)c1 * inv_c);
+        B2 = B * ((float)c2 * inv_c);
+        surface_velocity(sph[(w2 & ID_MASK) - 1], a, x, y, z, r2, u2);
     }
-    const float fl = 1.0f - B, sf = 1.0f - 0.5f * omega;
-    const float uF = ux * a.Fx + uy * a.Fy + uz * a.Fz;
-    // BGK with Guo forcing (its source divided by 1 - 1/(2 tau)), weighted by 1 - B
-    auto fluid = [&](int q) {
-        const float cu = cdot3(q, ux, uy, uz);
-        const float cF = cdot3(q, a.Fx, a.Fy, a.Fz);
-        const float Sg = w3(q) * (3.0f * (cF - uF) + 9.0f * cu * cF);
-        return fmaf(-omega, n[q], sf * Sg);
+    const float r45 = 4.5f * rho, r30 = 3.0f * rho;
+    // n_{-q} and n_q (Eq. 2), in that order, weighted by B
+    auto back2 = [&](int k) {
+        const int q = 2 * k + 1;
+        const float cu = cdot3(q, ux, uy, uz), e = fmaf(r45 * cu, cu, t), cj = r30 * cu;
+        const float2 X = make_float2(e - cj, e + cj);
+        return __ffma2_rn(make_float2(-w3(q), -w3(q)), X, make_float2(P[k].y, P[k].x));
     };
-    // f^eq_q(rho, u_s) - w_q
-    auto eq_solid = [&](int q, const float (&us)[3], float ts) {
-        const float cs = cdot3(q, us[0], us[1], us[2]);
-        return w3(q) * fmaf(rho * cs, fmaf(4.5f, cs, 3.0f), ts);
+    // f^eq_q(rho, u_s) - w_q over w_q, and its opposite's
+    auto solid2 = [&](int k, const float (&us)[3], float ts) {
+        const float cs = cdot3(2 * k + 1, us[0], us[1], us[2]), e = fmaf(r45 * cs, cs, ts), cj = r30 * cs;
+        return make_float2(e + cj, e - cj);
     };
-    if (w2) {     // Eq. 12 summed over both spheres: B (n_{-q} - d_q) + sum_p B_p (f^eq_q(u_s,p) - w_q)
-        const float ts1 = fmaf(-1.5f * rho, u1[0] * u1[0] + u1[1] * u1[1] + u1[2] * u1[2], drho);
+    const float ts1 = fmaf(-1.5f * rho, u1[0] * u1[0] + u1[1] * u1[1] + u1[2] * u1[2], drho);
+    const float n0 = fmaf(-w3(0), t, d[0]);
+    const float2 fl2 = make_float2(fl, fl), Bb = make_float2(B, B);
+    if (GEN && w2) {   // both spheres' Omega^s by their shares: B n_{-q} + sum_p B_p (f^eq_q(u_s,p) - w_q)
         const float ts2 = fmaf(-1.5f * rho, u2[0] * u2[0] + u2[1] * u2[1] + u2[2] * u2[2], drho);
+        Store<S>::st(fout + cell, fmaf(fl, f0, fmaf(B, n0, w3(0) * fmaf(B1, ts1, B2 * ts2))));
 #pragma unroll
-        for (int q = 0; q < 19; ++q) {
-            const float v = fmaf(B, n[opp3(q)] - d[q], fl * fluid(q)) + fmaf(B1, eq_solid(q, u1, ts1), B2 * eq_solid(q, u2, ts2));
-            Store<S>::st(fout + (size_t)q * a.plane + cell, d[q] + v);
+        for (int k = 0; k < 9; ++k) {
+            const int q = 2 * k + 1;
+            const float2 v = __ffma2_rn(make_float2(B1, B1), solid2(k, u1, ts1), __fmul2_rn(make_float2(B2, B2), solid2(k, u2, ts2)));
+            const float2 w = __ffma2_rn(make_float2(w3(q), w3(q)), v, __fmul2_rn(Bb, back2(k)));
+            const float2 o = __ffma2_rn(fl2, fluid2(k), w);
+            Store<S>::st(fout + (size_t)q * a.plane + cell, o.x);
+            Store<S>::st(fout + (size_t)(q + 1) * a.plane + cell, o.y);
         }
-    } else if (w1) {   // Eq. 12 in shifted form: n_{-q} + (f^eq_q(u_s) - w_q) - d_q, weighted by B
-        const float ts = fmaf(-1.5f * rho, u1[0] * u1[0] + u1[1] * u1[1] + u1[2] * u1[2], drho);
+    } else {
+        Store<S>::st(fout + cell, fmaf(fl, f0, B * fmaf(w3(0), ts1, n0)));
 #pragma unroll
-        for (int q = 0; q < 19; ++q) {
-            const float v = fmaf(B, n[opp3(q)] + eq_solid(q, u1, ts) - d[q], fl * fluid(q));
-            Store<S>::st(fout + (size_t)q * a.plane + cell, d[q] + v);
+        for (int k = 0; k < 9; ++k) {
+            const int q = 2 * k + 1;
+            const float2 v = __ffma2_rn(make_float2(w3(q), w3(q)), solid2(k, u1, ts1), back2(k));
+            const float2 o = __ffma2_rn(fl2, fluid2(k), __fmul2_rn(Bb, v));
+            Store<S>::st(fout + (size_t)q * a.plane + cell, o.x);
+            Store<S>::st(fout + (size_t)(q + 1) * a.plane + cell, o.y);
         }
-    } else {      // no sphere: the fluid operator alone
-#pragma unroll
-        for (int q = 0; q < 19; ++q) Store<S>::st(fout + (size_t)q * a.plane + cell, d[q] + fluid(q));
     }
-    if (w1) sphere_force(B1, rho, jx, jy, jz, u1, r1, a, fo);
-    if (w2) {     // the second sphere's share
+    sphere_force(B1, rho, jx, jy, jz, u1, r1, a, fo);
+    if (GEN && w2) {   // the second sphere's share
         float f2[6];
         sphere_force(B2, rho, jx, jy, jz, u2, r2, a, f2);
         add_force3(fs, FT, (int)(w2 & ID_MASK) - 1, f2);
@@ -554,10 +482,13 @@ __global__ void __launch_bounds__(256, 2) k3_stream_collide(const S *__restrict_
 #pragma unroll
     for (int k = 0; k < FSLOTS; ++k) sm.id[k][t] = -1;   // each thread reads its own entries only
     S r[19];
-    if (in) fetch3(fin, a, x, y, z0, r);
+    unsigned word = 0u;
+    if (in) {
+        fetch3(fin, a, x, y, z0, r);
+        word = __ldg(map + ((size_t)z0 * a.ny + y) * a.nx + x);
+    }
     for (int z = z0; z < z1; ++z) {
         if (in) {
-            int sid = -1;
             float fo[6];
             float d[19];
 #pragma unroll
@@ -568,12 +499,13 @@ __global__ void __launch_bounds__(256, 2) k3_stream_collide(const S *__restrict_
                     if (cx3(q) != 0 && ((y == 0 && cy3(q) == 1) || (y == a.ny - 1 && cy3(q) == -1)))
                         d[q] += 6.0f * w3(q) * (float)cx3(q) * (y == 0 ? a.uw_bot : a.uw_top);
             }
-            if (z + 1 < z1) fetch3(fin, a, x, y, z + 1, r);   // in flight during this cell's arithmetic
             const size_t cell = ((size_t)z * a.ny + y) * a.nx + x;
-            if constexpr (GEN)
-                sid = collide3_gen(d, a, x, y, z, cell, map, map2, sph, fout, FT, sm, fo, unstable);
-            else
-                sid = collide3_plain(d, a, x, y, z, cell, map, sph, fout, fo, unstable);
+            const unsigned wz = word;
+            if (z + 1 < z1) {   // in flight during this cell's arithmetic
+                fetch3(fin, a, x, y, z + 1, r);
+                word = __ldg(map + cell + (size_t)a.ny * a.nx);
+            }
+            const int sid = collide3<GEN>(d, a, x, y, z, cell, wz, map2, sph, fout, FT, sm, fo, unstable);
             if (sid >= 0) {
                 add_force3(sm, FT, sid, fo);
                 met = true;
