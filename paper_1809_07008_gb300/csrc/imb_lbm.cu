@@ -589,19 +589,6 @@ k_stream_collide(const __grid_constant__ CUtensorMap tmap_n, const __grid_consta
                     const SolidMoments none = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
                     node_collide_store<S, false, FORCED>(d, c, none, fout + (size_t)y * a.pitch + x, a);
                 }
-            } else if (!FORCED && !(rowc & (rowc - 1u))) {
-                // one candidate s in the row: a lane's node is covered by s alone or not at all
-                // (e0 = 0, hence B = 0 and no terms)
-                const int s = __ffs(rowc) - 1;
-                const PRec &P = tc->p[s];
-                const float eps = fminf(e0, 1.0f), tm = c.te - 0.5f;
-                const float B = e0 > 0.0f ? __fdividef(eps * tm, (1.0f - eps) + tm) : 0.0f;   // Eq. 14
-                const float rx = __fsub_rn((float)(lane - P.ci), P.fx) + 0.5f, ry = __fsub_rn((float)(yy - P.cj), P.fy) + 0.5f;
-                const float usx = P.vx - P.w * ry, usy = P.vy + P.w * rx;   // u_s = v + w z x r
-                // Eqs. 15-16
-                const float vx = B * fmaf(-c.rho, usx, c.jx), vy = B * fmaf(-c.rho, usy, c.jy);
-                add_terms(s, vx, vy, rx * vy - ry * vx, ka, kb, fa, fb, acc_t + warp);
-                if (xin) node_collide_store1<S>(d, c, B, usx, usy, fout + (size_t)y * a.pitch + x, a);
             } else {
                 SolidMoments sm;
                 row_imb<FORCED>(c, lane, yy, cm, rowc, e0, tc->p, tc->eoff, ka, kb, fa, fb, acc_t + warp, a, sm);

@@ -42,17 +42,19 @@ __device__ __forceinline__ void node_state(const float (&d)[9], const LatticeArg
     c.ux = c.jx * inv;
     c.uy = c.jy * inv;
     c.usq = c.ux * c.ux + c.uy * c.uy;
-    // ---- non-equilibrium parts (Eq. 2): n_{+-q} = d_{+-q} - w_q (t + (3 c.j) (1.5 c.u) +- 3 c.j),
-    // t = drho - 1.5 rho u^2
-    const float t = fmaf(-1.5f * c.rho, c.usq, c.drho);
-    c.n[0] = fmaf(-w_of(0), t, d[0]);
-    const float jx3 = 3.0f * c.jx, jy3 = 3.0f * c.jy, ux15 = 1.5f * c.ux, uy15 = 1.5f * c.uy;
+    // ---- non-equilibrium parts (Eq. 2)
+    const float m15 = -1.5f * c.usq;
+    c.n[0] = d[0] - w_of(0) * fmaf(c.rho, m15, c.drho);
     float2 N[4];
+    const float2 rho2 = make_float2(c.rho, c.rho), drho2 = make_float2(c.drho, c.drho);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
+        // n_{+-q} = d_{+-q} - w_q (drho + rho (4.5 (c.u)^2 - 1.5 u^2 +- 3 c.u)), each rounded once
         const int q = pair_q(k);
-        const float cj = cdot(q, jx3, jy3), e = fmaf(cj, cdot(q, ux15, uy15), t);
-        N[k] = __ffma2_rn(make_float2(-w_of(q), -w_of(q)), make_float2(e + cj, e - cj), P[k]);
+        const float cu = cdot(q, c.ux, c.uy);
+        const float e = fmaf(4.5f * cu, cu, m15), o3 = 3.0f * cu;
+        const float2 X = __ffma2_rn(rho2, make_float2(e + o3, e - o3), drho2);
+        N[k] = __ffma2_rn(make_float2(-w_of(q), -w_of(q)), X, P[k]);
         c.n[q] = N[k].x;
         c.n[opp_of(q)] = N[k].y;
     }
@@ -71,34 +73,6 @@ __device__ __forceinline__ void node_state(const float (&d)[9], const LatticeArg
         const float disc = fmaf(a.smag_coef * sq, inv, a.tau * a.tau);
         c.te = 0.5f * (a.tau + disc * rsqrtf(disc));                // (tau + sqrt(disc)) / 2
         c.omega = __fdividef(1.0f, c.te);
-    }
-}
-
-// Collision and store of a node covered by one particle of surface velocity (usx, usy), or by none
-// (B = 0): in the shifted variables Eq. 13 is
-//   d*_q = (1 - B) (d_q - omega n_q) + B (n_{-q} + f^eq_q(rho, u_s) - w_q),
-// four FP32x2 operations for a pair, without the moments that several particles need: with the
-// equilibrium of node_state in j and u, 103.2 -> 99.6 M warp instructions on a 4096 x 2048 suspension
-// (16 bits 108.0 -> 102.5 M); with the tail on 8192 x 4096 516 -> 508 us FP32, 486 -> 473 us FP16.
-template <typename S>
-__device__ __forceinline__ void node_collide_store1(const float (&d)[9], const NodeState &c, const float B,
-                                                    const float usx, const float usy, S *__restrict__ outp,
-                                                    const LatticeArgs &a) {
-    const float fl = 1.0f - B, mo = -fl * c.omega;
-    const float ts = fmaf(-1.5f * c.rho, usx * usx + usy * usy, c.drho);
-    Store<S>::st(outp, fmaf(fl, d[0], fmaf(mo, c.n[0], B * fmaf(w_of(0), ts, c.n[0]))));
-    const float r3 = 3.0f * c.rho, jx3 = r3 * usx, jy3 = r3 * usy, ux15 = 1.5f * usx, uy15 = 1.5f * usy;
-    const float2 fl2 = make_float2(fl, fl), mo2 = make_float2(mo, mo), B2 = make_float2(B, B);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int q = pair_q(k), o = opp_of(q);
-        const float cj = cdot(q, jx3, jy3), e = fmaf(cj, cdot(q, ux15, uy15), ts);
-        // n_{-q} + f^eq_q(u_s) - w_q, for q and -q
-        float2 v = __ffma2_rn(make_float2(w_of(q), w_of(q)), make_float2(e + cj, e - cj), make_float2(c.n[o], c.n[q]));
-        v = __ffma2_rn(B2, v, __fmul2_rn(mo2, make_float2(c.n[q], c.n[o])));
-        v = __ffma2_rn(fl2, make_float2(d[q], d[o]), v);
-        Store<S>::st(outp + (size_t)q * a.plane, v.x);
-        Store<S>::st(outp + (size_t)o * a.plane, v.y);
     }
 }
 
