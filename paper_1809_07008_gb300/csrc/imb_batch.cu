@@ -27,243 +27,308 @@ namespace imb {
 
 struct BatchDomain {
     int nx, ny;
-    int item0[2];       // first work item of the domain: row segments of 32 / 64 cells
-    size_t off;         // element offset of the domain's plane 0 in the population buffers
-    size_t plane;       // nx * ny
-    size_t e_off;       // offset of the domain's solid ratios (cells)
+    int item0[2];       // first work item of the domain, with one and with two cells per lane
+    size_t off;         // element offset of the domain in the population buffers
+    size_t row;         // elements from one row to the next
+    size_t e_off;       // offset of the domain's solid ratios, rows of 2 ceil(nx / 2) (even)
     float tau, omega0, Fx, Fy;
     float smag_coef;    // 18 sqrt(2) C^2 of the Smagorinsky closure (0: plain BGK)
     float pad2;
 };
 
-// One node of a domain whose disks are at rest.  With u_s = 0 the solid operator of Eq. 12
+// Layout of the populations: rows of blocks of 128 bytes per plane, the nine planes of a block one
+// after another ([y][x / SEGB][slot][x % SEGB]), so that one pointer and compile-time offsets
+// reach every plane: with whole planes one after another a node's nine loads and nine stores took
+// some 40 of its 330 instructions for addresses.  The planes that a node pulls from the same row
+// (c_y = 0, 1, -1) are neighbours: slots 3 g, 3 g + 1, 3 g + 2 hold c_x = 0, 1, -1.
+template <typename S> __host__ __device__ constexpr int segb() { return 128 / (int)sizeof(S); }
+__host__ __device__ constexpr int group_q(int g, int k) { return (g == 0 ? 0x310 : g == 1 ? 0x652 : 0x784) >> (4 * k) & 15; }
+__host__ __device__ constexpr int slot_of(int q) {
+    for (int i = 0; i < 9; ++i)
+        if (group_q(i / 3, i % 3) == q) return i;
+    return -1;
+}
+static_assert(cy_of(2) == 1 && cy_of(5) == 1 && cy_of(6) == 1 && cy_of(4) == -1 && cy_of(8) == -1 && cy_of(7) == -1 &&
+                  cx_of(1) == 1 && cx_of(5) == 1 && cx_of(8) == 1 && cx_of(3) == -1 && cx_of(6) == -1 && cx_of(7) == -1,
+              "groups of the planes by source row");
+// element offset of cell x in a row, slot 0
+template <typename S> __host__ __device__ __forceinline__ int col_of(int x) {
+    return x / segb<S>() * 9 * segb<S>() + x % segb<S>();
+}
+
+// The node of a domain whose disks are at rest.  With u_s = 0 the solid operator of Eq. 12
 // summed over the covering disks is B (f_{-q} - f^eq_{-q}(u) + f^eq_q(0) - f_q); in the
 // shifted variables d_q = f_q - w_q and n_q = d_q - (f^eq_q(u) - w_q) this is
 // B (n_{-q} - d_q + w_q drho), and Eq. 13 becomes
-//   d*_q = d_q + (1 - B) [-omega n_q + (1 - omega / 2) w_q S_q] + B (n_{-q} - d_q + w_q drho)
+//   d*_q = (1 - B) [d_q - omega n_q + (1 - omega / 2) w_q S_q] + B (n_{-q} + w_q drho)
 // with S_q / w_q = 3 (c_q - u).F + 9 (c_q.u)(c_q.F) (Guo forcing).  The same algebra as the
 // general collision with every solid-velocity moment zero, with fewer operations.
-struct RestNode {
-    float B, jx, jy;      // drag weight of the node (Eq. 14); jx, jy include the half-force shift
-    bool ok;              // |u|^2 below the Mach guard (false for NaN)
+struct Cells1 {           // one cell per lane
+    using T = float;
+    static __device__ __forceinline__ T all(float a) { return a; }
+    static __device__ __forceinline__ T add(T a, T b) { return a + b; }
+    static __device__ __forceinline__ T mul(T a, T b) { return a * b; }
+    static __device__ __forceinline__ T fma(T a, T b, T c) { return fmaf(a, b, c); }
+    template <typename F> static __device__ __forceinline__ T each(T a, F f) { return f(a); }
+    static __device__ __forceinline__ bool below(T a, float lim) { return a < lim; }
+    static __device__ __forceinline__ float sum(T a) { return a; }
 };
+struct Cells2 {           // two neighbouring cells per lane, FP32x2 instructions throughout
+    using T = float2;
+    static __device__ __forceinline__ T all(float a) { return make_float2(a, a); }
+    static __device__ __forceinline__ T add(T a, T b) { return __fadd2_rn(a, b); }
+    static __device__ __forceinline__ T mul(T a, T b) { return __fmul2_rn(a, b); }
+    static __device__ __forceinline__ T fma(T a, T b, T c) { return __ffma2_rn(a, b, c); }
+    template <typename F> static __device__ __forceinline__ T each(T a, F f) { return make_float2(f(a.x), f(a.y)); }
+    static __device__ __forceinline__ bool below(T a, float lim) { return a.x < lim && a.y < lim; }
+    static __device__ __forceinline__ float sum(T a) { return a.x + a.y; }
+};
+template <int CPL> using CellsOf = std::conditional_t<CPL == 2, Cells2, Cells1>;
 
 // The eight moving directions as four pairs (q, -q), q = 1, 2, 5, 6, whose terms differ only in
-// the sign of their odd parts: computed with FP32x2 instructions where the operations line up.
+// the sign of their odd parts.
 __host__ __device__ constexpr int bpair_q(int k) { return k < 2 ? k + 1 : k + 3; }
 
-template <typename S>
-__device__ __forceinline__ RestNode rest_node(const float (&d)[9], float e, const BatchDomain &D, S *__restrict__ outp) {
-    RestNode r;
-    float2 P[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) P[k] = make_float2(d[bpair_q(k)], d[opp_of(bpair_q(k))]);
-    const float2 Sm = __fadd2_rn(__fadd2_rn(P[0], P[1]), __fadd2_rn(P[2], P[3]));
-    const float drho = d[0] + (Sm.x + Sm.y);
-    const float rho = 1.0f + drho;
-    float Dq[4];   // d_q - d_-q
-#pragma unroll
-    for (int k = 0; k < 4; ++k) Dq[k] = P[k].x - P[k].y;
-    const float jx = fmaf(0.5f, D.Fx, (Dq[0] + Dq[2]) - Dq[3]);   // Eqs. 3-4
-    const float jy = fmaf(0.5f, D.Fy, (Dq[1] + Dq[2]) + Dq[3]);
-    const float inv = __fdividef(1.0f, rho);
-    const float ux = jx * inv, uy = jy * inv;
-    const float usq = ux * ux + uy * uy;
-    const float t = fmaf(-1.5f * rho, usq, drho);
-    // non-equilibrium parts (Eq. 2): n_{+-q} = d_{+-q} - w_q (t + 4.5 rho (c.u)^2 +- 3 rho c.u)
-    const float n0 = d[0] - w_of(0) * t;
-    float2 N[4];
+// d -> post-collision d, in place; the lane's drag (Eq. 15 with u_s = 0) is added to fx, fy.  Returns
+// whether |u|^2 lies below the Mach guard (false for NaN).
+template <class V>
+__device__ __forceinline__ bool rest_node(typename V::T (&d)[9], const typename V::T e, const BatchDomain &D,
+                                          typename V::T &fx, typename V::T &fy) {
+    using T = typename V::T;
+    const T one = V::all(1.0f), neg = V::all(-1.0f);
+    auto sub = [&](T a, T b) { return V::fma(b, neg, a); };
+    T P[4], M[4];   // d_q + d_-q, d_q - d_-q
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int q = bpair_q(k);
-        const float cu = cdot(q, ux, uy);
-        const float rcu = rho * cu;
-        const float ev = fmaf(4.5f * rcu, cu, t), od = 3.0f * rcu;
-        N[k] = __ffma2_rn(make_float2(-w_of(q), -w_of(q)), make_float2(ev + od, ev - od), P[k]);
+        P[k] = V::add(d[q], d[opp_of(q)]);
+        M[k] = sub(d[q], d[opp_of(q)]);
     }
-    float omega = D.omega0, te = D.tau;
-    if (D.smag_coef > 0.0f) {       // Smagorinsky closure, as in the single-lattice path
-        const float2 Ep = __fadd2_rn(N[2], N[3]);                            // (n5 + n6, n7 + n8)
-        const float2 Fp = __fadd2_rn(N[2], make_float2(-N[3].x, -N[3].y));   // (n5 - n6, n7 - n8)
-        const float ee = Ep.x + Ep.y;
-        const float pxx = (N[0].x + N[0].y) + ee;
-        const float pyy = (N[1].x + N[1].y) + ee;
-        const float pxy = Fp.x + Fp.y;
-        const float Q = pxx * pxx + pyy * pyy + 2.0f * pxy * pxy;
-        const float sq = Q > 0.0f ? Q * rsqrtf(Q) : 0.0f;
-        const float disc = fmaf(D.smag_coef * sq, inv, D.tau * D.tau);
-        te = 0.5f * (D.tau + disc * rsqrtf(disc));
-        omega = __fdividef(1.0f, te);
+    const T diag = V::add(P[2], P[3]);
+    const T drho = V::add(d[0], V::add(V::add(P[0], P[1]), diag));
+    const T inv = V::each(V::add(one, drho), [](float r) { return __fdividef(1.0f, r); });
+    const T mx = sub(V::add(M[0], M[2]), M[3]), my = V::add(V::add(M[1], M[2]), M[3]);
+    const T jx = V::fma(V::all(0.5f), V::all(D.Fx), mx), jy = V::fma(V::all(0.5f), V::all(D.Fy), my);   // Eqs. 3-4
+    const T ux = V::mul(jx, inv), uy = V::mul(jy, inv);
+    const T jxx = V::mul(jx, ux), juu = V::fma(jy, uy, jxx);
+    const T t = V::fma(V::all(-1.5f), juu, drho);   // f^eq_{+-q} - w_q = w_q (t + (3 c.j) (1.5 c.u) +- 3 c.j)
+    T omega = V::all(D.omega0), te = V::all(D.tau);
+    if (D.smag_coef > 0.0f) {       // Smagorinsky closure; Pi = sum c c f - (drho / 3 + j u) on the diagonal
+        const T third = V::fma(V::all(1.0f / 3.0f), drho, jxx), thirdy = V::fma(V::all(1.0f / 3.0f), drho, V::mul(jy, uy));
+        const T pxx = sub(V::add(P[0], diag), third), pyy = sub(V::add(P[1], diag), thirdy);
+        const T pxy = V::fma(V::mul(jx, neg), uy, sub(P[2], P[3]));
+        const T Q = V::fma(pxx, pxx, V::fma(pyy, pyy, V::mul(V::add(pxy, pxy), pxy)));
+        const T sq = V::each(Q, [](float v) { return v > 0.0f ? v * rsqrtf(v) : 0.0f; });
+        const T disc = V::fma(V::mul(V::all(D.smag_coef), sq), inv, V::all(D.tau * D.tau));
+        const T root = V::each(disc, [](float v) { return v * rsqrtf(v); });
+        te = V::mul(V::all(0.5f), V::add(V::all(D.tau), root));
+        omega = V::each(te, [](float v) { return __fdividef(1.0f, v); });
     }
-    const float ec = fminf(e, 1.0f), tm = te - 0.5f;
-    const float B = __fdividef(ec * tm, (1.0f - ec) + tm);   // Eq. 14 (0 in uncovered cells)
-    const float fl = 1.0f - B, flw = -fl * omega, fls = fl * (1.0f - 0.5f * omega), Bd = B * drho;
-    const float g = -3.0f * (ux * D.Fx + uy * D.Fy);
-    // d*_q = (1 - B) d_q - (1 - B) omega n_q + B n_{-q} + w_q [(1 - B)(1 - omega/2) S_q + B drho]
-    // with S_q / w_q = cF (3 + 9 cu) - 3 u.F (cF = c_q.F); both halves of a pair: cu, cF -> -cu, -cF
-    Store<S>::st(outp, fmaf(fl, d[0], fmaf(flw, n0, fmaf(B, n0, fmaf(w_of(0) * fls, g, w_of(0) * Bd)))));
-    const float2 fl2 = make_float2(fl, fl), flw2 = make_float2(flw, flw), B2 = make_float2(B, B);
+    const T ec = V::each(e, [](float v) { return fminf(v, 1.0f); });
+    const T tm = V::add(te, V::all(-0.5f));
+    const T den = V::each(V::add(sub(one, ec), tm), [](float v) { return __fdividef(1.0f, v); });
+    const T B = V::mul(V::mul(ec, tm), den);   // Eq. 14 (0 in uncovered cells)
+    // d*_q = (1 - B) [d_q - omega (d_q - w_q (even + odd))] + B [d_-q - w_q (back even - back odd)],
+    //   even = t + 4.5 rho (c.u)^2 + m (9 (c.u)(c.F) - 3 u.F),  odd = 3 c.j + m 3 c.F,  m = tau_eff - 1/2:
+    // the forcing (1 - omega / 2) S_q = omega m S_q goes into the equilibrium that is relaxed to;
+    //   back even = t - drho + 4.5 rho (c.u)^2,  back odd = 3 c.j
+    const T fl = sub(one, B), mo = V::mul(omega, neg), m3 = V::mul(V::all(3.0f), tm), m9 = V::mul(V::all(9.0f), tm);
+    const T g = V::mul(V::all(-3.0f), V::fma(ux, V::all(D.Fx), V::mul(uy, V::all(D.Fy))));
+    const T jx3 = V::mul(V::all(3.0f), jx), jy3 = V::mul(V::all(3.0f), jy);
+    const T ux15 = V::mul(V::all(1.5f), ux), uy15 = V::mul(V::all(1.5f), uy);
+    const T base = V::fma(tm, g, t), back = V::mul(V::all(-1.5f), juu);
+    const T ox = V::fma(m3, V::all(D.Fx), jx3), oy = V::fma(m3, V::all(D.Fy), jy3);
+    const T hx = V::fma(m9, V::all(D.Fx), V::mul(V::all(1.5f), jx3)), hy = V::fma(m9, V::all(D.Fy), V::mul(V::all(1.5f), jy3));
+    const T f0 = V::fma(mo, V::fma(V::all(-w_of(0)), base, d[0]), d[0]);
+    d[0] = V::fma(fl, f0, V::mul(B, V::fma(V::all(-w_of(0)), back, d[0])));
+    const T u4[4] = {ux, uy, V::add(ux, uy), sub(uy, ux)}, h4[4] = {hx, hy, V::add(hx, hy), sub(hy, hx)};
+    const T v4[4] = {ux15, uy15, V::add(ux15, uy15), sub(uy15, ux15)}, j4[4] = {jx3, jy3, V::add(jx3, jy3), sub(jy3, jx3)};
+    const T o4[4] = {ox, oy, V::add(ox, oy), sub(oy, ox)};
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int q = bpair_q(k), o = opp_of(q);
-        const float cu = cdot(q, ux, uy), cF = cdot(q, D.Fx, D.Fy);
-        const float kq = w_of(q) * fls, bq = w_of(q) * Bd;
-        const float2 Sq = __ffma2_rn(make_float2(cF, -cF), make_float2(fmaf(9.0f, cu, 3.0f), fmaf(-9.0f, cu, 3.0f)),
-                                     make_float2(g, g));
-        float2 v = __ffma2_rn(make_float2(kq, kq), Sq, make_float2(bq, bq));
-        v = __ffma2_rn(B2, make_float2(N[k].y, N[k].x), v);
-        v = __ffma2_rn(flw2, N[k], v);
-        v = __ffma2_rn(fl2, P[k], v);
-        Store<S>::st(outp + (size_t)q * D.plane, v.x);
-        Store<S>::st(outp + (size_t)o * D.plane, v.y);
+        const T w = V::all(-w_of(q));
+        const T ev = V::fma(u4[k], h4[k], base), bk = V::fma(j4[k], v4[k], back);
+        const T fq = V::fma(mo, V::fma(w, V::add(ev, o4[k]), d[q]), d[q]);
+        const T fo = V::fma(mo, V::fma(w, sub(ev, o4[k]), d[o]), d[o]);
+        const T sq = V::fma(w, sub(bk, j4[k]), d[o]), so = V::fma(w, V::add(bk, j4[k]), d[q]);
+        d[q] = V::fma(fl, fq, V::mul(B, sq));
+        d[o] = V::fma(fl, fo, V::mul(B, so));
     }
-    r.B = B;
-    r.jx = jx;
-    r.jy = jy;
-    r.ok = usq < 0.09f;
-    return r;
+    fx = V::fma(B, V::add(jx, V::all(-D.Fx)), fx);
+    fy = V::fma(B, V::add(jy, V::all(-D.Fy)), fy);
+    const T usq = V::mul(juu, inv);
+    return V::below(usq, 0.09f);
 }
 
-// stored value as loaded (converted to FP32 where it is used)
-template <typename S> __device__ __forceinline__ S ld_raw(const S *p) { return __ldg(p); }
+// stored values as loaded (converted to FP32 where they are used), one or two cells
 __device__ __forceinline__ float to_f32(float v) { return v; }
 __device__ __forceinline__ float to_f32(__half v) { return __half2float(v); }
 __device__ __forceinline__ float to_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
+template <typename S> struct Pair;
+template <> struct Pair<float> {
+    using T = float2;
+    static __device__ __forceinline__ float2 f32(T v) { return v; }
+    static __device__ __forceinline__ T of(float2 v) { return v; }
+};
+template <> struct Pair<__half> {
+    using T = __half2;
+    static __device__ __forceinline__ float2 f32(T v) { return __half22float2(v); }
+    static __device__ __forceinline__ T of(float2 v) { return __float22half2_rn(v); }
+};
+template <> struct Pair<__nv_bfloat16> {
+    using T = __nv_bfloat162;
+    static __device__ __forceinline__ float2 f32(T v) { return __bfloat1622float2(v); }
+    static __device__ __forceinline__ T of(float2 v) { return __float22bfloat162_rn(v); }
+};
 
-// A work item is a segment of 32 CPL cells of one row (the last segment of a row may be
-// shorter); items are numbered domain by domain, row by row.  Each warp takes an equal run of
-// consecutive items, so the warps finish together whatever the domain sizes, the rows a warp
-// visits one after another share their neighbour rows in L1, and the drag of a domain is
-// summed in registers until the warp leaves the domain.  With one cell per lane the loads of
-// the next item of the same domain are issued before the arithmetic of the current one.
+// the pulled values of a lane (Eq. 1, periodic wrap) from the rows y, y - 1 and y + 1 of a domain
+template <typename S, int CPL> struct Pulled;
+template <typename S> struct Pulled<S, 1> {
+    S r[9];
+    float e;
+    __device__ __forceinline__ void fetch(const S *const (&R)[3], const float *Er, int x, int nx) {
+        const int c = col_of<S>(x), cl = col_of<S>(x == 0 ? nx - 1 : x - 1), cr = col_of<S>(x == nx - 1 ? 0 : x + 1);
+#pragma unroll
+        for (int g = 0; g < 3; ++g) {
+            r[3 * g] = __ldg(R[g] + c + 3 * g * segb<S>());
+            r[3 * g + 1] = __ldg(R[g] + cl + (3 * g + 1) * segb<S>());
+            r[3 * g + 2] = __ldg(R[g] + cr + (3 * g + 2) * segb<S>());
+        }
+        e = __ldg(Er + x);
+    }
+    __device__ __forceinline__ void values(float (&d)[9], bool) const {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) d[group_q(i / 3, i % 3)] = to_f32(r[i]);
+    }
+    static __device__ __forceinline__ void store(S *p, const float (&d)[9]) {
+#pragma unroll
+        for (int q = 0; q < 9; ++q) Store<S>::st(p + slot_of(q) * segb<S>(), d[q]);
+    }
+};
+// The cells x (even) and x + 1.  A plane with c_x = 0 is one load of both; the others' sources
+// straddle the pairs and are loaded one by one (x - 1 and x, x + 1 and x + 2): no exchange between
+// lanes, whose rows may differ.
+template <typename S> struct Pulled<S, 2> {
+    typename Pair<S>::T c2[3];
+    S l0[3], l1[3], r0[3], r1[3];
+    float2 e;
+    __device__ __forceinline__ void fetch(const S *const (&R)[3], const float *Er, int x, int nx) {
+        constexpr int G = segb<S>();
+        const int in = x % G, c = x / G * 9 * G + in;
+        const int cl = x == 0 ? col_of<S>(nx - 1) : (in == 0 ? c - 8 * G - 1 : c - 1);
+        const int ca = x + 1 == nx ? 0 : c + 1;
+        const int cb = x + 2 >= nx ? 0 : (in == G - 2 ? c + 8 * G + 2 : c + 2);
+#pragma unroll
+        for (int g = 0; g < 3; ++g) {
+            c2[g] = __ldg(reinterpret_cast<const typename Pair<S>::T *>(R[g] + c + 3 * g * G));
+            l0[g] = __ldg(R[g] + cl + (3 * g + 1) * G);
+            l1[g] = __ldg(R[g] + c + (3 * g + 1) * G);
+            r0[g] = __ldg(R[g] + ca + (3 * g + 2) * G);
+            r1[g] = __ldg(R[g] + cb + (3 * g + 2) * G);
+        }
+        e = __ldg(reinterpret_cast<const float2 *>(Er + x));
+    }
+    // tail: x is the last cell of a row of odd length, and the lane's second cell no cell of the
+    // domain.  It takes the first one's values (its solid ratio is 0: no drag).
+    __device__ __forceinline__ void values(float2 (&d)[9], bool tail) const {
+#pragma unroll
+        for (int g = 0; g < 3; ++g) {
+            d[group_q(g, 0)] = Pair<S>::f32(c2[g]);
+            d[group_q(g, 1)] = make_float2(to_f32(l0[g]), to_f32(l1[g]));
+            d[group_q(g, 2)] = make_float2(to_f32(r0[g]), to_f32(r1[g]));
+        }
+        if (tail) {
+#pragma unroll
+            for (int q = 0; q < 9; ++q) d[q].y = d[q].x;
+        }
+    }
+    static __device__ __forceinline__ void store(S *p, const float2 (&d)[9]) {
+#pragma unroll
+        for (int q = 0; q < 9; ++q)
+            *reinterpret_cast<typename Pair<S>::T *>(p + slot_of(q) * segb<S>()) = Pair<S>::of(d[q]);
+    }
+};
+
+// A work item is 32 CPL cells of a domain, row after row without regard to the rows' ends (with two
+// cells per lane, of rows rounded up to even length); only a domain's last item leaves lanes idle.
+// Each warp takes an equal run of consecutive items, so the warps finish together whatever the
+// domain sizes, and the drag of a domain is summed in registers until the warp leaves it.  The
+// loads of the next item of the same domain are issued before the arithmetic of the current one.
+//
+// What bounds it: with two cells a lane the registers (120, two blocks an SM: 16 warps) and the latency
+// of the loads; the schedulers issue on half the cycles and DRAM moves 44 B a cell of the 40 it must
+// (16 bits), at 4.5 TB/s.  256 domains, 15.5 M cells, FP16: 198 us a step with whole planes one after
+// another and one cell a lane, 158 us now; 12 domains of 0.28 M cells together, FP32: 11.6 -> 9.7 us.
+// With the collision as a sum of d_q + d_-q and d_q - d_-q (half the operations) 156 us and twice
+// the FP32 error; two items ahead 148 us with that form, 176 us (spills) with this one; three
+// blocks an SM (80 registers, spills) 187 us; five of 128 threads 151 us.
 template <typename S, int CPL>
-__global__ void __launch_bounds__(256, 3) k_batch_step(const S *__restrict__ fin, S *__restrict__ fout, const BatchDomain *__restrict__ dom,
-                             int ndom, int nitems, const float *__restrict__ E, double *drag, unsigned *err) {
-    constexpr int SEG = 32 * CPL;
+__global__ void __launch_bounds__(256, CPL == 2 ? 2 : 3)
+k_batch_step(const S *__restrict__ fin, S *__restrict__ fout, const BatchDomain *__restrict__ dom,
+             int ndom, int nitems, const float *__restrict__ E, double *drag, unsigned *err) {
+    using V = CellsOf<CPL>;
     const int lane = threadIdx.x & 31;
     const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int nw = (int)((gridDim.x * blockDim.x) >> 5);
     const int per = nitems / nw, rem = nitems % nw;
-    int it = gw * per + min(gw, rem);
-    const int end = it + per + (gw < rem ? 1 : 0);
-    if (it >= end) return;   // the whole warp: gw is the same on every lane
+    const int it0 = gw * per + min(gw, rem);
+    int left = per + (gw < rem ? 1 : 0);   // items of the warp
+    if (left <= 0) return;   // the whole warp: gw is the same on every lane
     int lo = 0, hi = ndom - 1;   // the domain of the first item
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (dom[mid].item0[CPL - 1] <= it) lo = mid;
+        if (dom[mid].item0[CPL - 1] <= it0) lo = mid;
         else hi = mid - 1;
     }
-    int dd = lo;
-    BatchDomain D = dom[dd];
-    int nseg = (D.nx + SEG - 1) / SEG;
-    int y = (it - D.item0[CPL - 1]) / nseg;
-    int sg = it - D.item0[CPL - 1] - y * nseg;
     bool unstable = false;
-    float fx_acc = 0.0f, fy_acc = 0.0f;
-    if constexpr (CPL == 1) {
-        S r[9];
-        float e = 0.0f;
-        auto fetch = [&](const BatchDomain &Dc, int yc, int sgc) {   // pull (Eq. 1), periodic wrap
-            const int x = sgc * 32 + lane, nx = Dc.nx, ny = Dc.ny, plane = (int)Dc.plane;
-            if (x >= nx) return;
-            const S *src = fin + Dc.off;
-            const int rm = (yc == 0 ? ny - 1 : yc - 1) * nx, r0 = yc * nx, rp = (yc == ny - 1 ? 0 : yc + 1) * nx;
-            const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
-#pragma unroll
-            for (int q = 0; q < 9; ++q) {
-                const int xs = cx_of(q) == 0 ? x : (cx_of(q) == 1 ? xm : xp);
-                const int ys = cy_of(q) == 0 ? r0 : (cy_of(q) == 1 ? rm : rp);
-                r[q] = ld_raw(src + (q * plane + ys + xs));
-            }
-            e = __ldg(E + Dc.e_off + (size_t)yc * nx + x);
+    for (int dd = lo, first = it0; left > 0; ++dd) {   // domains of the warp
+        const BatchDomain D = dom[dd];
+        const int nx = D.nx, ny = D.ny, width = (nx + CPL - 1) / CPL;
+        first -= dd == lo ? D.item0[CPL - 1] : first;   // item within the domain
+        int n = min(left, (int)(((long long)width * ny + 31) / 32) - first);   // items of this domain
+        left -= n;
+        const int p = first * 32 + lane;
+        int y = p / width, x = (p - y * width) * CPL;
+        Pulled<S, CPL> r;
+        const S *src = fin + D.off;
+        S *out = fout + D.off;
+        const float *Ed = E + D.e_off;
+        const int e_row = (nx + 1) / 2 * 2;
+        auto fetch = [&] {
+            if (y >= ny) return;   // past the end of the domain's last item
+            const S *R[3] = {src + (size_t)y * D.row, src + (size_t)(y == 0 ? ny - 1 : y - 1) * D.row,
+                             src + (size_t)(y == ny - 1 ? 0 : y + 1) * D.row};
+            r.fetch(R, Ed + (size_t)y * e_row, x, nx);
         };
-        fetch(D, y, sg);
-        for (;;) {
-            float d[9];
-#pragma unroll
-            for (int q = 0; q < 9; ++q) d[q] = to_f32(r[q]);
-            const float ec = e;
-            const int x = sg * 32 + lane;
-            const bool act = x < D.nx;
-            S *dst = fout + D.off + (size_t)y * D.nx + x;
-            ++it;
-            if (++sg == nseg) {
-                sg = 0;
+        fetch();
+        typename V::T fx = V::all(0.0f), fy = V::all(0.0f);
+        while (n > 0) {
+            typename V::T d[9];
+            r.values(d, CPL == 2 && x + 1 == nx);
+            const auto ec = r.e;
+            const bool act = y < ny;
+            S *dst = out + (size_t)y * D.row + col_of<S>(x);
+            x += 32 * CPL;
+            while (x >= nx) {   // rows of fewer than 32 CPL cells: several at once
+                x -= width * CPL;
                 ++y;
             }
-            const bool last = it == end, leave = last || y == D.ny;
-            if (!leave) fetch(D, y, sg);   // in flight during this item's arithmetic
+            if (--n > 0) fetch();   // in flight during this item's arithmetic
             if (act) {
-                const RestNode c = rest_node(d, ec, D, dst);
-                if (!c.ok) unstable = true;   // Mach guard, also catches NaN
-                fx_acc = fmaf(c.B, c.jx - D.Fx, fx_acc);   // Eq. 15 with u_s = 0
-                fy_acc = fmaf(c.B, c.jy - D.Fy, fy_acc);
-            }
-            if (leave) {   // leaving the domain: add its drag
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    fx_acc += __shfl_xor_sync(0xffffffffu, fx_acc, o);
-                    fy_acc += __shfl_xor_sync(0xffffffffu, fy_acc, o);
-                }
-                if (lane == 0 && (fx_acc != 0.0f || fy_acc != 0.0f)) {
-                    atomicAdd(&drag[2 * dd], (double)fx_acc);
-                    atomicAdd(&drag[2 * dd + 1], (double)fy_acc);
-                }
-                fx_acc = fy_acc = 0.0f;
-                if (last) break;
-                D = dom[++dd];
-                nseg = (D.nx + SEG - 1) / SEG;
-                y = 0;
-                fetch(D, y, sg);
+                if (!rest_node<V>(d, ec, D, fx, fy)) unstable = true;   // Mach guard, also catches NaN
+                Pulled<S, CPL>::store(dst, d);
             }
         }
-        if (__any_sync(0xffffffffu, unstable) && lane == 0) set_err(err, ERR_UNSTABLE);
-        return;
-    }
-    for (;;) {
-        const int nx = D.nx, ny = D.ny, plane = (int)D.plane;
-        const S *src = fin + D.off;
-        const float *Er = E + D.e_off + (size_t)y * nx;
-        S *dst = fout + D.off + (size_t)y * nx;
-        const int rm = (y == 0 ? ny - 1 : y - 1) * nx, r0 = y * nx, rp = (y == ny - 1 ? 0 : y + 1) * nx;
+        float sx = V::sum(fx), sy = V::sum(fy);   // leaving the domain: add its drag
 #pragma unroll
-        for (int k = 0; k < CPL; ++k) {
-            const int x = sg * SEG + 32 * k + lane;
-            if (x >= nx) continue;
-            const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
-            float d[9];
-#pragma unroll
-            for (int q = 0; q < 9; ++q) {   // pull from x - c_q with the periodic wrap (Eq. 1)
-                const int xs = cx_of(q) == 0 ? x : (cx_of(q) == 1 ? xm : xp);
-                const int ys = cy_of(q) == 0 ? r0 : (cy_of(q) == 1 ? rm : rp);
-                d[q] = Store<S>::ld(src + (q * plane + ys + xs));
-            }
-            const RestNode c = rest_node(d, Er[x], D, dst + x);
-            if (!c.ok) unstable = true;   // Mach guard, also catches NaN
-            fx_acc = fmaf(c.B, c.jx - D.Fx, fx_acc);   // Eq. 15 with u_s = 0
-            fy_acc = fmaf(c.B, c.jy - D.Fy, fy_acc);
+        for (int o = 16; o > 0; o >>= 1) {
+            sx += __shfl_xor_sync(0xffffffffu, sx, o);
+            sy += __shfl_xor_sync(0xffffffffu, sy, o);
         }
-        ++it;
-        if (++sg == nseg) {
-            sg = 0;
-            ++y;
-        }
-        const bool last = it == end;
-        if (last || y == ny) {   // leaving the domain: add its drag
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                fx_acc += __shfl_xor_sync(0xffffffffu, fx_acc, o);
-                fy_acc += __shfl_xor_sync(0xffffffffu, fy_acc, o);
-            }
-            if (lane == 0 && (fx_acc != 0.0f || fy_acc != 0.0f)) {
-                atomicAdd(&drag[2 * dd], (double)fx_acc);
-                atomicAdd(&drag[2 * dd + 1], (double)fy_acc);
-            }
-            fx_acc = fy_acc = 0.0f;
-            if (last) break;
-            D = dom[++dd];
-            nseg = (D.nx + SEG - 1) / SEG;
-            y = 0;
+        if (lane == 0 && (sx != 0.0f || sy != 0.0f)) {
+            atomicAdd(&drag[2 * dd], (double)sx);
+            atomicAdd(&drag[2 * dd + 1], (double)sy);
         }
     }
     if (__any_sync(0xffffffffu, unstable) && lane == 0) set_err(err, ERR_UNSTABLE);
@@ -285,7 +350,7 @@ __global__ void k_batch_solid(const BatchDomain *__restrict__ dom, const int *__
     const float lox = __fsub_rn((float)di, fx), loy = __fsub_rn((float)dk, fy);
     if (!covers(lox, loy, rf)) return;
     const int i = ((ci + di) % D.nx + D.nx) % D.nx, k = ((cj + dk) % D.ny + D.ny) % D.ny;
-    atomicAdd(&E[D.e_off + (size_t)k * D.nx + i], cell_disk_area(lox, loy, rf));
+    atomicAdd(&E[D.e_off + (size_t)k * ((D.nx + 1) / 2 * 2) + i], cell_disk_area(lox, loy, rf));
 }
 
 // f(x, t) of one domain (the pull of its post-collision field), as FP64 f = w + (f - w)
@@ -294,13 +359,14 @@ __global__ void k_batch_gather(const S *__restrict__ fin, const BatchDomain *__r
                                double *out) {
     const BatchDomain D = dom[d];
     const size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= D.plane) return;
+    const size_t cells = (size_t)D.nx * D.ny;
+    if (c >= cells) return;
     const int x = (int)(c % D.nx), y = (int)(c / D.nx);
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
         const int xs = (x - cx_of(q) + D.nx) % D.nx, ys = (y - cy_of(q) + D.ny) % D.ny;
-        out[(size_t)q * D.plane + c] =
-            (double)w_of(q) + (double)Store<S>::ld(fin + D.off + (size_t)q * D.plane + (size_t)ys * D.nx + xs);
+        out[(size_t)q * cells + c] =
+            (double)w_of(q) + (double)Store<S>::ld(fin + D.off + (size_t)ys * D.row + col_of<S>(xs) + slot_of(q) * segb<S>());
     }
 }
 
@@ -311,6 +377,7 @@ using namespace imb;
 struct imb_batch {
     int device = 0, storage = 0, elem = 4, ndom = 0, nitems[2] = {0, 0}, ndisk = 0;
     size_t total = 0;          // elements per population buffer
+    size_t cells = 0;
     void *buf[2] = {nullptr, nullptr};
     int cur = 0;               // buffer holding the current post-collision field
     BatchDomain *dom = nullptr;
@@ -422,8 +489,9 @@ extern "C" int imb_batch_create(imb_batch **out, int n_domains, const int *nx, c
     b->elem = storage == IMB_STORE_FP32 ? 4 : 2;
     b->ndom = n_domains;
     double rmax = 0.0;
-    size_t cells = 0;
-    long long items = 0, items2 = 0;   // row segments of 32 and of 64 cells
+    size_t cells = 0, e_cells = 0;
+    long long items = 0, items2 = 0;   // work items of 32 and of 64 cells
+    const size_t G = storage == IMB_STORE_FP32 ? segb<float>() : segb<__half>();
     int ndisk = 0;
     for (int d = 0; d < n_domains; ++d) {
         if (nx[d] < 3 || ny[d] < 3 || 9.0 * nx[d] * ny[d] > 2147483647.0 || !(tau[d] > 0.5) ||
@@ -436,18 +504,20 @@ extern "C" int imb_batch_create(imb_batch **out, int n_domains, const int *nx, c
         D.ny = ny[d];
         D.item0[0] = (int)items;
         D.item0[1] = (int)items2;
-        D.plane = (size_t)nx[d] * ny[d];
-        D.off = 9 * cells;
-        D.e_off = cells;
+        D.off = b->total;
+        D.row = (nx[d] + G - 1) / G * 9 * G;
+        D.e_off = e_cells;
         D.tau = (float)tau[d];
         D.omega0 = (float)(1.0 / tau[d]);
         D.Fx = (float)Fx[d];
         D.Fy = (float)Fy[d];
         D.smag_coef = (float)(18.0 * std::sqrt(2.0) * C_smag[d] * C_smag[d]);
         b->hdom.push_back(D);
-        cells += D.plane;
-        items += (long long)ny[d] * ((nx[d] + 31) / 32);
-        items2 += (long long)ny[d] * ((nx[d] + 63) / 64);
+        cells += (size_t)nx[d] * ny[d];
+        e_cells += (size_t)(nx[d] + 1) / 2 * 2 * ny[d];
+        b->total += D.row * ny[d];
+        items += ((long long)ny[d] * nx[d] + 31) / 32;
+        items2 += ((long long)ny[d] * ((nx[d] + 1) / 2) + 31) / 32;
         ndisk += n_disks[d];
     }
     if (ndisk > 0 && (!disk_xy || !disk_r)) {
@@ -473,14 +543,14 @@ extern "C" int imb_batch_create(imb_batch **out, int n_domains, const int *nx, c
     b->nitems[0] = (int)items;
     b->nitems[1] = (int)items2;
     b->ndisk = ndisk;
-    b->total = 9 * cells;
+    b->cells = cells;
     cudaGetDevice(&b->device);
     cudaError_t e;
     if ((e = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking)) != cudaSuccess ||
         (e = cudaMalloc(&b->buf[0], b->total * b->elem)) != cudaSuccess ||
         (e = cudaMalloc(&b->buf[1], b->total * b->elem)) != cudaSuccess ||
         (e = cudaMalloc(&b->dom, sizeof(BatchDomain) * n_domains)) != cudaSuccess ||
-        (e = cudaMalloc(&b->E, sizeof(float) * std::max(cells, (size_t)1))) != cudaSuccess ||
+        (e = cudaMalloc(&b->E, sizeof(float) * e_cells)) != cudaSuccess ||
         (e = cudaMalloc(&b->drag, sizeof(double) * 2 * n_domains)) != cudaSuccess ||
         (e = cudaMalloc(&b->err, sizeof(unsigned))) != cudaSuccess) {
         *out = b;
@@ -490,7 +560,7 @@ extern "C" int imb_batch_create(imb_batch **out, int n_domains, const int *nx, c
     // fluid at rest with rho = 1: f = w, i.e. zero shifted populations
     BCK(cudaMemsetAsync(b->buf[0], 0, b->total * b->elem, b->stream), "clear");
     BCK(cudaMemsetAsync(b->buf[1], 0, b->total * b->elem, b->stream), "clear");
-    BCK(cudaMemsetAsync(b->E, 0, sizeof(float) * cells, b->stream), "clear");
+    BCK(cudaMemsetAsync(b->E, 0, sizeof(float) * e_cells, b->stream), "clear");
     BCK(cudaMemsetAsync(b->drag, 0, sizeof(double) * 2 * n_domains, b->stream), "clear");
     BCK(cudaMemsetAsync(b->err, 0, sizeof(unsigned), b->stream), "clear");
     BCK(cudaMemcpyAsync(b->dom, b->hdom.data(), sizeof(BatchDomain) * n_domains, cudaMemcpyHostToDevice, b->stream),
@@ -648,12 +718,12 @@ extern "C" int imb_batch_get_populations(imb_batch *b, int domain, double *f) {
     if (!b || !f || domain < 0 || domain >= b->ndom) return IMB_E_INVALID_ARG;
     int rc = batch_wait(b);
     if (rc) return rc;
-    const size_t n = 9 * b->hdom[domain].plane;
+    const size_t cells = (size_t)b->hdom[domain].nx * b->hdom[domain].ny, n = 9 * cells;
     double *t = nullptr;
     BCK(cudaMalloc(&t, sizeof(double) * n), "readback buffer");
     cudaError_t e = by_storage_b(b->storage, [&](auto tag) {
         using S = std::remove_pointer_t<decltype(tag)>;
-        k_batch_gather<S><<<(unsigned)((b->hdom[domain].plane + 255) / 256), 256, 0, b->stream>>>(
+        k_batch_gather<S><<<(unsigned)((cells + 255) / 256), 256, 0, b->stream>>>(
             (const S *)b->buf[b->cur], b->dom, domain, t);
         return cudaGetLastError();
     });
@@ -665,7 +735,7 @@ extern "C" int imb_batch_get_populations(imb_batch *b, int domain, double *f) {
 }
 
 extern "C" long long imb_batch_cells(const imb_batch *b) {
-    return b ? (long long)(b->total / 9) : 0;
+    return b ? (long long)b->cells : 0;
 }
 
 extern "C" const char *imb_batch_last_error(const imb_batch *b) {
