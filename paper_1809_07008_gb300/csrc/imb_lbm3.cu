@@ -310,15 +310,14 @@ __device__ __forceinline__ void sphere_force(float Bp, float rho, float jx, floa
 // the host launches it only when some cell holds two spheres or C_smag > 0.
 //
 // The kernel issues more than it waits for memory (half the cycles in FP32, more in 16 bits), so
-// the algebra is arranged for few instructions.  The 18 moving directions are nine pairs (q, -q),
-// q odd, in FP32x2 operations.  A fluid cell needs no non-equilibrium parts: its update is
-//   d*_{+-q} = (1 - omega) d_{+-q} + w_q [T0 + c.u (4.5 omega rho c.u + 9 s c.F) +- c.J],
-//   T0 = omega (drho - 1.5 rho u^2) - 3 s u.F,  J = 3 (omega j + s F),  s = 1 - omega / 2;
-// a covered cell is (1 - B) times that plus B (n_{-q} + f^eq_q(rho, u_s) - w_q), and the
-// closure's momentum flux comes from the second moments, Pi = sum c c d - (drho / 3 + rho u u).
-// Kernel time on 16 M cells with one sphere 505 -> 453 us FP32 (5.4 TB/s), 446 -> 337 us FP16; the
-// 240 x 100 x 100 packed bed (GEN) 172 -> 105 us.  Three blocks an SM (80 registers, spills): 499,
-// 397 and 182 us; columns of 16 cells: 457, 347 and 111 us.
+// the algebra is arranged for few instructions: the 18 moving directions are nine pairs (q, -q),
+// q odd, in FP32x2 operations, and a pair's non-equilibrium parts are formed where they are used.
+// The order of the sums and products of Eqs. 2 and 13 is kept as it was: with bfloat16 populations any
+// other rounding moves weak transverse flows by 1 % within 50 steps (the forcing put into the
+// equilibrium, and Pi from second moments, would save another 5 %).
+// A step with its share of the read-back, before and with the fetch of the map word ahead and pairs
+// formed where used: 400 x 100 x 400 FP32 673 -> 560 us, 203 x 77 x 151 FP16 111 -> 81 us, the
+// 240 x 100 x 100 packed bed (GEN) 315 -> 140 us with the column sums.
 template <bool GEN, typename S>
 __device__ __forceinline__ int collide3(const float (&d)[19], const Args3 &a, int x, int y, int z, size_t cell,
                                         const unsigned word, const unsigned *__restrict__ map2,
@@ -327,27 +326,30 @@ __device__ __forceinline__ int collide3(const float (&d)[19], const Args3 &a, in
     float2 P[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) P[k] = make_float2(d[2 * k + 1], d[2 * k + 2]);
-    float drho, s[9];
+    float drho, mx = 0.0f, my = 0.0f, mz = 0.0f;
     if constexpr (GEN) {
-        drho = d[0];
+        drho = 0.0f;
 #pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            s[k] = P[k].x + P[k].y;
-            drho += s[k];
+        for (int q = 0; q < 19; ++q) {
+            drho += d[q];
+            if (cx3(q)) mx += cx3(q) * d[q];
+            if (cy3(q)) my += cy3(q) * d[q];
+            if (cz3(q)) mz += cz3(q) * d[q];
         }
-    } else {
+    } else {   // c_{-q} = -c_q: first moments from d_q - d_-q
         const float2 t = __fadd2_rn(__fadd2_rn(__fadd2_rn(P[0], P[1]), __fadd2_rn(P[2], P[3])),
                                     __fadd2_rn(__fadd2_rn(P[4], P[5]), __fadd2_rn(P[6], P[7])));
         const float2 u = __fadd2_rn(t, P[8]);
         drho = d[0] + (u.x + u.y);
-    }
-    float D[9];   // c_{-q} = -c_q: first moments from d_q - d_-q
 #pragma unroll
-    for (int k = 0; k < 9; ++k) D[k] = P[k].x - P[k].y;
-    // pairs: x, y, z, x+y, x-y, x+z, x-z, y+z, y-z
-    const float mx = D[0] + ((D[3] + D[4]) + (D[5] + D[6]));
-    const float my = D[1] + ((D[3] - D[4]) + (D[7] + D[8]));
-    const float mz = D[2] + ((D[5] - D[6]) + (D[7] - D[8]));
+        for (int k = 0; k < 9; ++k) {
+            const int q = 2 * k + 1;
+            const float Dk = P[k].x - P[k].y;
+            if (cx3(q)) mx += cx3(q) * Dk;
+            if (cy3(q)) my += cy3(q) * Dk;
+            if (cz3(q)) mz += cz3(q) * Dk;
+        }
+    }
     const float rho = 1.0f + drho;
     const float jx = fmaf(0.5f, a.Fx, mx), jy = fmaf(0.5f, a.Fy, my), jz = fmaf(0.5f, a.Fz, mz);
     const float inv = __fdividef(1.0f, rho);
@@ -355,39 +357,56 @@ __device__ __forceinline__ int collide3(const float (&d)[19], const Args3 &a, in
     const float uu = ux * ux + uy * uy + uz * uz;
     if (!(uu < 0.09f)) unstable = true;   // Mach guard, also catches NaN
     const float t = fmaf(-1.5f * rho, uu, drho);
+    // n_q and n_-q (Eq. 2): d - w_q (t +- rho c.u (3 +- 4.5 c.u))
+    auto noneq2 = [&](int k) {
+        const int q = 2 * k + 1;
+        const float cu = cdot3(q, ux, uy, uz), rcu = rho * cu;
+        const float2 X = __ffma2_rn(make_float2(rcu, -rcu), make_float2(fmaf(4.5f, cu, 3.0f), fmaf(-4.5f, cu, 3.0f)), make_float2(t, t));
+        return __ffma2_rn(make_float2(-w3(q), -w3(q)), X, P[k]);
+    };
     float te = a.tau, omega = a.omega;
     if (GEN && a.smag_coef > 0.0f) {   // tau_eff = (tau + sqrt(tau^2 + 18 sqrt(2) C^2 sqrt(Pi : Pi) / rho)) / 2
-        const float sxy = s[3] + s[4], sxz = s[5] + s[6], syz = s[7] + s[8], th = drho * (1.0f / 3.0f);
-        const float pxx = fmaf(-jx, ux, (s[0] + (sxy + sxz)) - th);
-        const float pyy = fmaf(-jy, uy, (s[1] + (sxy + syz)) - th);
-        const float pzz = fmaf(-jz, uz, (s[2] + (sxz + syz)) - th);
-        const float pxy = fmaf(-jx, uy, s[3] - s[4]), pxz = fmaf(-jx, uz, s[5] - s[6]), pyz = fmaf(-jy, uz, s[7] - s[8]);
+        float pxx = 0.0f, pyy = 0.0f, pzz = 0.0f, pxy = 0.0f, pxz = 0.0f, pyz = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {   // Pi = sum_q c_q c_q n_q, q and then -q
+            const int q = 2 * k + 1;
+            const float2 N = noneq2(k);
+            if (cx3(q)) pxx = (pxx + N.x) + N.y;
+            if (cy3(q)) pyy = (pyy + N.x) + N.y;
+            if (cz3(q)) pzz = (pzz + N.x) + N.y;
+            if (cx3(q) && cy3(q)) pxy = cx3(q) * cy3(q) > 0 ? (pxy + N.x) + N.y : (pxy - N.x) - N.y;
+            if (cx3(q) && cz3(q)) pxz = cx3(q) * cz3(q) > 0 ? (pxz + N.x) + N.y : (pxz - N.x) - N.y;
+            if (cy3(q) && cz3(q)) pyz = cy3(q) * cz3(q) > 0 ? (pyz + N.x) + N.y : (pyz - N.x) - N.y;
+        }
         const float Q = fmaf(pxx, pxx, fmaf(pyy, pyy, pzz * pzz)) + 2.0f * fmaf(pxy, pxy, fmaf(pxz, pxz, pyz * pyz));
         const float sq = Q > 0.0f ? Q * rsqrtf(Q) : 0.0f;   // sqrt(Q)
         const float disc = fmaf(a.smag_coef * sq, inv, a.tau * a.tau);
         te = 0.5f * (a.tau + disc * rsqrtf(disc));
         omega = __fdividef(1.0f, te);
     }
-    const float sf = 1.0f - 0.5f * omega, om1 = 1.0f - omega;
-    const float uF = ux * a.Fx + uy * a.Fy + uz * a.Fz;
-    const float T0 = fmaf(omega, t, -3.0f * sf * uF), K = 4.5f * omega * rho, o3 = 3.0f * omega, s3 = 3.0f * sf;
-    const float Jx = fmaf(o3, jx, s3 * a.Fx), Jy = fmaf(o3, jy, s3 * a.Fy), Jz = fmaf(o3, jz, s3 * a.Fz);
-    const float s9x = 9.0f * sf * a.Fx, s9y = 9.0f * sf * a.Fy, s9z = 9.0f * sf * a.Fz;
-    const float2 om2 = make_float2(om1, om1);
-    // the fluid's d*_q and d*_-q
-    auto fluid2 = [&](int k) {
+    const float uF = ux * a.Fx + uy * a.Fy + uz * a.Fz, sf = 1.0f - 0.5f * omega;
+    const float n0 = d[0] - w3(0) * t;
+    const float2 mo2 = make_float2(-omega, -omega);
+    // the fluid's change of d_q and d_-q: BGK with Guo forcing (its source divided by 1 - 1/(2 tau)),
+    // -omega n_q + sf w_q (3 (c_q.F - u.F) + 9 (c_q.u)(c_q.F))
+    const float f0 = fmaf(-omega, n0, sf * (w3(0) * (-3.0f * uF)));
+    auto fluid2 = [&](int k, const float2 N) {
         const int q = 2 * k + 1;
-        const float cu = cdot3(q, ux, uy, uz), cJ = cdot3(q, Jx, Jy, Jz);
-        const float ev = fmaf(cu, fmaf(K, cu, cdot3(q, s9x, s9y, s9z)), T0);
-        return __ffma2_rn(make_float2(w3(q), w3(q)), make_float2(ev + cJ, ev - cJ), __fmul2_rn(om2, P[k]));
+        const float cu = cdot3(q, ux, uy, uz), cF = cdot3(q, a.Fx, a.Fy, a.Fz);
+        const float e9 = 9.0f * cu * cF, sw = sf * w3(q);
+        const float2 G = __ffma2_rn(make_float2(3.0f, 3.0f), __fadd2_rn(make_float2(cF, -cF), make_float2(-uF, -uF)), make_float2(e9, e9));
+        if constexpr (GEN) {   // sf (w S): one more rounding than the constant sf w
+            const float2 wS = __fmul2_rn(make_float2(w3(q), w3(q)), G);
+            return __ffma2_rn(mo2, N, __fmul2_rn(make_float2(sf, sf), wS));
+        }
+        return __ffma2_rn(mo2, N, __fmul2_rn(make_float2(sw, sw), G));
     };
-    const float f0 = fmaf(om1, d[0], w3(0) * T0);
     if (!word) {
-        Store<S>::st(fout + cell, f0);
+        Store<S>::st(fout + cell, d[0] + f0);
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
             const int q = 2 * k + 1;
-            const float2 o = fluid2(k);
+            const float2 o = __fadd2_rn(P[k], fluid2(k, noneq2(k)));
             Store<S>::st(fout + (size_t)q * a.plane + cell, o.x);
             Store<S>::st(fout + (size_t)(q + 1) * a.plane + cell, o.y);
         }
@@ -416,41 +435,37 @@ __device__ __forceinline__ int collide3(const float (&d)[19], const Args3 &a, in
         B2 = B * ((float)c2 * inv_c);
         surface_velocity(sph[(w2 & ID_MASK) - 1], a, x, y, z, r2, u2);
     }
-    const float r45 = 4.5f * rho, r30 = 3.0f * rho;
-    // n_{-q} and n_q (Eq. 2), in that order, weighted by B
-    auto back2 = [&](int k) {
-        const int q = 2 * k + 1;
-        const float cu = cdot3(q, ux, uy, uz), e = fmaf(r45 * cu, cu, t), cj = r30 * cu;
-        const float2 X = make_float2(e - cj, e + cj);
-        return __ffma2_rn(make_float2(-w3(q), -w3(q)), X, make_float2(P[k].y, P[k].x));
-    };
     // f^eq_q(rho, u_s) - w_q over w_q, and its opposite's
     auto solid2 = [&](int k, const float (&us)[3], float ts) {
-        const float cs = cdot3(2 * k + 1, us[0], us[1], us[2]), e = fmaf(r45 * cs, cs, ts), cj = r30 * cs;
-        return make_float2(e + cj, e - cj);
+        const float cs = cdot3(2 * k + 1, us[0], us[1], us[2]), rcs = rho * cs;
+        return __ffma2_rn(make_float2(rcs, -rcs), make_float2(fmaf(4.5f, cs, 3.0f), fmaf(-4.5f, cs, 3.0f)), make_float2(ts, ts));
     };
     const float ts1 = fmaf(-1.5f * rho, u1[0] * u1[0] + u1[1] * u1[1] + u1[2] * u1[2], drho);
-    const float n0 = fmaf(-w3(0), t, d[0]);
     const float2 fl2 = make_float2(fl, fl), Bb = make_float2(B, B);
-    if (GEN && w2) {   // both spheres' Omega^s by their shares: B n_{-q} + sum_p B_p (f^eq_q(u_s,p) - w_q)
+    if (GEN && w2) {   // both spheres' Omega^s by their shares: B (n_{-q} - d_q) + sum_p B_p (f^eq_q(u_s,p) - w_q)
         const float ts2 = fmaf(-1.5f * rho, u2[0] * u2[0] + u2[1] * u2[1] + u2[2] * u2[2], drho);
-        Store<S>::st(fout + cell, fmaf(fl, f0, fmaf(B, n0, w3(0) * fmaf(B1, ts1, B2 * ts2))));
+        Store<S>::st(fout + cell, d[0] + (fmaf(B, n0 - d[0], fl * f0) + fmaf(B1, w3(0) * ts1, B2 * (w3(0) * ts2))));
+        const float2 B12 = make_float2(B1, B1), B22 = make_float2(B2, B2);
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
             const int q = 2 * k + 1;
-            const float2 v = __ffma2_rn(make_float2(B1, B1), solid2(k, u1, ts1), __fmul2_rn(make_float2(B2, B2), solid2(k, u2, ts2)));
-            const float2 w = __ffma2_rn(make_float2(w3(q), w3(q)), v, __fmul2_rn(Bb, back2(k)));
-            const float2 o = __ffma2_rn(fl2, fluid2(k), w);
+            const float2 N = noneq2(k), w2 = make_float2(w3(q), w3(q));
+            const float2 e1 = __fmul2_rn(w2, solid2(k, u1, ts1)), e2 = __fmul2_rn(w2, solid2(k, u2, ts2));
+            const float2 T = __fadd2_rn(make_float2(N.y, N.x), make_float2(-P[k].x, -P[k].y));
+            const float2 v = __fadd2_rn(__ffma2_rn(Bb, T, __fmul2_rn(fl2, fluid2(k, N))), __ffma2_rn(B12, e1, __fmul2_rn(B22, e2)));
+            const float2 o = __fadd2_rn(P[k], v);
             Store<S>::st(fout + (size_t)q * a.plane + cell, o.x);
             Store<S>::st(fout + (size_t)(q + 1) * a.plane + cell, o.y);
         }
-    } else {
-        Store<S>::st(fout + cell, fmaf(fl, f0, B * fmaf(w3(0), ts1, n0)));
+    } else {   // n_{-q} + (f^eq_q(u_s) - w_q) - d_q, weighted by B
+        Store<S>::st(fout + cell, d[0] + fmaf(B, n0 + w3(0) * ts1 - d[0], fl * f0));
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
             const int q = 2 * k + 1;
-            const float2 v = __ffma2_rn(make_float2(w3(q), w3(q)), solid2(k, u1, ts1), back2(k));
-            const float2 o = __ffma2_rn(fl2, fluid2(k), __fmul2_rn(Bb, v));
+            const float2 N = noneq2(k);
+            const float2 T = __fadd2_rn(__ffma2_rn(make_float2(w3(q), w3(q)), solid2(k, u1, ts1), make_float2(N.y, N.x)),
+                                        make_float2(-P[k].x, -P[k].y));
+            const float2 o = __fadd2_rn(P[k], __ffma2_rn(Bb, T, __fmul2_rn(fl2, fluid2(k, N))));
             Store<S>::st(fout + (size_t)q * a.plane + cell, o.x);
             Store<S>::st(fout + (size_t)(q + 1) * a.plane + cell, o.y);
         }
