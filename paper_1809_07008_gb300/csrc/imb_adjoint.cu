@@ -52,6 +52,11 @@ __device__ __forceinline__ void pair_add(float &hi, float &lo, float b, float b_
     hi = t;
 }
 
+// sum of the nine directions, in the order of a butterfly over lanes
+__device__ __forceinline__ float tree9(const float (&v)[9]) {
+    return (((v[0] + v[8]) + v[4]) + (v[2] + v[6])) + ((v[1] + v[5]) + (v[3] + v[7]));
+}
+
 // One step backwards: lam1 = d J / d f(t+1) (columns already transposed), S0 = P(t-1)
 // (f(t) is pulled from it); writes lam0 = d J / d f(t).  With `inlet` the transpose of the inlet
 // and outlet columns of the pull that gave f(t) from S0 follows in the same launch: f(0) =
@@ -59,10 +64,11 @@ __device__ __forceinline__ void pair_add(float &hi, float &lo, float b, float b_
 // and nx - 1 on to the threads of columns 1 and nx - 2, which hold the pulled f(t) they need, and
 // the row's d J / d u_in to g_uin (the launch keeps columns nx - 2 and nx - 1 in one block).
 //
-// The directions are taken in opposite pairs, whose sums and differences of the adjoint (Lp, Lm)
-// enter the transposed equilibrium; d J / d tau is summed in pairs of FP32 over the block (an FP64
-// add takes a warp 64 cycles, and every warp's shuffle tree took five of them).  The gradient of
-// 400 steps on 512 x 256 cells: 33.7 -> 16.9 ms with the copies and launches saved in the host's loop.
+// d J / d tau is summed in pairs of FP32 over the block (an FP64 add takes a warp 64 cycles, and
+// every warp's shuffle tree took five of them).  The adjoint itself keeps the order of its sums:
+// taken on opposite pairs it has fewer instructions and is no faster on 512 x 256 cells (42 us a
+// forward and reverse step, 84 before the launches and copies were saved), but where the adjoint front
+// has not reached the inlet d J / d u_in is rounding noise, which any other order changes whole.
 __global__ void __launch_bounds__(256) k_adjoint_step(const float *__restrict__ lam1, const float *__restrict__ S0,
                                                       float *__restrict__ lam0, const LatticeArgs a,
                                                       const float *__restrict__ E, double *__restrict__ gE,
@@ -77,7 +83,7 @@ __global__ void __launch_bounds__(256) k_adjoint_step(const float *__restrict__ 
     S0 += a.origin;
     lam0 += a.origin;
     float v[9];
-    float drho = 0.0f, rho = 1.0f, ux = 0.0f, uy = 0.0f;
+    float col_rho = 1.0f, col_ux = 0.0f, col_uy = 0.0f;
     if (x < a.nx) {
         // adjoint of P(t) at (x, y): who pulled P_q(x, y); and f(t) at (x, y), pulled from
         // P(t-1) (shifted populations d = f - w).  Away from the edges no boundary rule applies.
@@ -113,64 +119,68 @@ __global__ void __launch_bounds__(256) k_adjoint_step(const float *__restrict__ 
             }
             pull_cell(S0, a, x, y, d);
         }
-        float jx = 0.0f, jy = 0.0f;
+        float drho = 0.0f, jx = 0.0f, jy = 0.0f;
 #pragma unroll
         for (int q = 0; q < 9; ++q) {   // products with a zero velocity component left out
             drho += d[q];
             if (cx_of(q) != 0) jx += cx_of(q) > 0 ? d[q] : -d[q];
             if (cy_of(q) != 0) jy += cy_of(q) > 0 ? d[q] : -d[q];
         }
-        rho = 1.0f + drho;
-        const float inv = 1.0f / rho;
-        ux = jx * inv;
-        uy = jy * inv;
-        const float usq = ux * ux + uy * uy;
-        const float e = fminf(Ec, 1.0f), tm = a.tau - 0.5f, den = (1.0f - e) + tm, rden = 1.0f / den;
-        const float B = Ec > 0.0f ? e * tm * rden : 0.0f;
-        const float af = (1.0f - B) * a.omega0;
-        // n_q = d_q - w_q (drho + rho (3 cu + 4.5 cu^2 - 1.5 u^2)); for a pair (q, -q), with
-        // s = sum and m = difference of the two: L.n = (Lp ns + Lm nm) / 2, the sum of the swapped
-        // products L_q n_-q + L_-q n_q = (Lp ns - Lm nm) / 2
-        const float t0 = fmaf(-1.5f * rho, usq, drho);
-        const float n0 = d[0] - w_of(0) * t0;
-        float Ln = L[0] * n0, Lno = L[0] * n0, Ld = L[0] * d[0], wL = w_of(0) * L[0];
-        const float mu0 = (af - B) * L[0];
-        float lr = mu0 * (w_of(0) * fmaf(1.5f, usq, 1.0f)), wm = w_of(0) * mu0, lx = 0.0f, ly = 0.0f;
+        const float rho = 1.0f + drho, ux = jx / rho, uy = jy / rho, usq = ux * ux + uy * uy;
+        float n[9];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int q = k < 2 ? k + 1 : k + 3, o = opp_of(q);
-            const float cu = cdot(q, ux, uy), cc = 4.5f * cu * cu, w = w_of(q);
-            const float Lp = L[q] + L[o], Lm = L[q] - L[o];
-            const float ns = (d[q] + d[o]) - 2.0f * w * fmaf(rho, cc, t0), nm = (d[q] - d[o]) - 6.0f * w * rho * cu;
-            const float a1 = 0.5f * Lp * ns, a2 = 0.5f * Lm * nm;
-            Ln += a1 + a2;
-            Lno += a1 - a2;
-            Ld += L[q] * d[q] + L[o] * d[o];
-            wL = fmaf(w, Lp, wL);
-            const float mp = (af - B) * Lp, mm = (af + B) * Lm;
-            lr = fmaf(w * mp, fmaf(1.5f, usq, 1.0f) - cc, lr);
-            wm = fmaf(w, mp, wm);
-            const float g = w * (3.0f * mm + 9.0f * cu * mp);
-            if (cx_of(q) != 0) lx += cx_of(q) > 0 ? g : -g;
-            if (cy_of(q) != 0) ly += cy_of(q) > 0 ? g : -g;
+        for (int q = 0; q < 9; ++q) {
+            const float cu = cdot(q, ux, uy);
+            n[q] = d[q] - w_of(q) * (drho + rho * (3.0f * cu + 4.5f * cu * cu - 1.5f * usq));
         }
-        lr = fmaf(B, wL, lr);
-        lx = fmaf(-3.0f * ux, wm, lx);
-        ly = fmaf(-3.0f * uy, wm, ly);
-        const float keep = 1.0f - af - B, drag = inv_T * B, lxd = lx + drag;
-        v[0] = fmaf(keep + B, L[0], lr);
+        const float e = fminf(Ec, 1.0f), tau = a.tau, tm = tau - 0.5f;
+        const float B = Ec > 0.0f ? e * tm / ((1.0f - e) + tm) : 0.0f;
+        const float af = (1.0f - B) / tau;
+        float mu[9], nu = 0.0f;
 #pragma unroll
-        for (int q = 1; q < 9; ++q) {
-            float t = fmaf(keep, L[q], fmaf(B, L[opp_of(q)], lr));
-            if (cx_of(q) != 0) t += cx_of(q) > 0 ? lxd : -lxd;
-            if (cy_of(q) != 0) t += cy_of(q) > 0 ? ly : -ly;
+        for (int q = 0; q < 9; ++q) {
+            mu[q] = af * L[q] - B * L[opp_of(q)];
+            nu += B * w_of(q) * L[q];
+        }
+        float lr = nu, ljx = 0.0f, ljy = 0.0f;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            const float cxq = (float)cx_of(q), cyq = (float)cy_of(q), cu = cdot(q, ux, uy);
+            lr += mu[q] * w_of(q) * (1.0f - 4.5f * cu * cu + 1.5f * usq);
+            ljx += mu[q] * w_of(q) * (cx_of(q) != 0 ? 3.0f * cxq + 9.0f * cu * cxq - 3.0f * ux : -3.0f * ux);
+            ljy += mu[q] * w_of(q) * (cy_of(q) != 0 ? 3.0f * cyq + 9.0f * cu * cyq - 3.0f * uy : -3.0f * uy);
+        }
+        float Ln = 0.0f;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            const float cxq = (float)cx_of(q), cyq = (float)cy_of(q);
+            float t = L[q] * (1.0f - af - B) + B * L[opp_of(q)];
+            if (cx_of(q) != 0) t += inv_T * B * cxq;
+            t += lr;
+            if (cx_of(q) != 0) t += cxq * ljx;
+            if (cy_of(q) != 0) t += cyq * ljy;
             v[q] = t;
+            Ln += L[q] * (1.0f - B) * n[q];
         }
-        gt = (1.0f - B) * Ln * (a.omega0 * a.omega0);
+        gt = Ln / (tau * tau);
         if (B > 0.0f) {
-            const float lB = inv_T * jx + fmaf(a.omega0, Ln, Lno) + (drho * wL - Ld);
-            pair_add(gt, gt_lo, lB * e * (1.0f - e) * (rden * rden), 0.0f);
-            if (Ec < 1.0f) gE[c] += (double)(lB * tm * (1.0f + tm) * (rden * rden));
+            float lB = inv_T * jx;
+#pragma unroll
+            for (int q = 0; q < 9; ++q) lB += L[q] * (n[q] / tau + n[opp_of(q)] + w_of(q) * drho - d[q]);
+            const float den = (1.0f - e) + tm;
+            pair_add(gt, gt_lo, lB * e * (1.0f - e) / (den * den), 0.0f);
+            if (Ec < 1.0f) gE[c] += (double)(lB * tm * (1.0f + tm) / (den * den));
+        }
+        if (inlet && (x == 1 || x == a.nx - 2)) {   // f(t) of the column, for the columns next to it
+            float mx[9], my[9];
+#pragma unroll
+            for (int q = 0; q < 9; ++q) {
+                mx[q] = (float)cx_of(q) * d[q];
+                my[q] = (float)cy_of(q) * d[q];
+            }
+            col_rho = 1.0f + tree9(d);
+            col_ux = tree9(mx) / col_rho;
+            col_uy = tree9(my) / col_rho;
         }
     }
     if (inlet && (blockIdx.x == 0 || blockIdx.x == gridDim.x - 1)) {
@@ -184,28 +194,33 @@ __global__ void __launch_bounds__(256) k_adjoint_step(const float *__restrict__ 
         if (x == a.nx - 2) {
             // outlet: f(nx-1) = f^eq(1, u), u = j / rho of f(nx-2); d f^eq_q / d u = w_q (3 c_q +
             // 9 (c_q . u) c_q - 3 u), d u / d f_p(nx-2) = (c_p - u) / rho
-            float gx = 0.0f, gy = 0.0f;
+            const float rho = col_rho, ux = col_ux, uy = col_uy;
+            float px[9], py[9];
 #pragma unroll
             for (int q = 0; q < 9; ++q) {
-                const float lw = edge[1][q] * w_of(q), cu9 = 9.0f * cdot(q, ux, uy) + 3.0f;
-                gx += lw * ((cx_of(q) != 0 ? (float)cx_of(q) * cu9 : 0.0f) - 3.0f * ux);
-                gy += lw * ((cy_of(q) != 0 ? (float)cy_of(q) * cu9 : 0.0f) - 3.0f * uy);
+                const float cxq = (float)cx_of(q), cyq = (float)cy_of(q), lo = edge[1][q], wq = w_of(q);
+                const float cu = cxq * ux + cyq * uy;
+                px[q] = lo * wq * (3.0f * cxq + __fmul_rn(9.0f, cu) * cxq - 3.0f * ux);
+                py[q] = lo * wq * (3.0f * cyq + __fmul_rn(9.0f, cu) * cyq - 3.0f * uy);
             }
+            const float gx = tree9(px), gy = tree9(py);
 #pragma unroll
             for (int q = 0; q < 9; ++q) v[q] += (gx * ((float)cx_of(q) - ux) + gy * ((float)cy_of(q) - uy)) / rho;
         }
         if (x == 1) {   // inlet: f(0) = f^eq(rho1, u_in), rho1 = 1 + the pulled shifted populations of column 1
-            const float uix = a.u_in_x, uiy = a.u_in_y, usq = uix * uix + uiy * uiy;
-            float l = 0.0f, g = 0.0f;
+            const float ux = a.u_in_x, uy = a.u_in_y, usq = ux * ux + uy * uy;
+            float pr[9], pg[9];
 #pragma unroll
             for (int q = 0; q < 9; ++q) {
-                const float lw = edge[0][q] * w_of(q), cu = cdot(q, uix, uiy);
-                l += lw * (1.0f + 3.0f * cu + 4.5f * cu * cu - 1.5f * usq);
-                g += lw * ((cx_of(q) != 0 ? (float)cx_of(q) * (3.0f + 9.0f * cu) : 0.0f) - 3.0f * uix);
+                const float cxq = (float)cx_of(q), cyq = (float)cy_of(q), l0 = edge[0][q], wq = w_of(q);
+                const float cu = cxq * ux + cyq * uy;
+                pr[q] = l0 * wq * (1.0f + 3.0f * cu + 4.5f * cu * cu - 1.5f * usq);
+                pg[q] = l0 * wq * (3.0f * cxq + __fmul_rn(9.0f, cu) * cxq - 3.0f * ux);
             }
+            const float l = tree9(pr), g = tree9(pg);
 #pragma unroll
             for (int q = 0; q < 9; ++q) v[q] += l;
-            if (g != 0.0f) atomicAdd(g_uin, (double)(g * rho));
+            if (g != 0.0f) atomicAdd(g_uin, (double)(g * col_rho));
         }
     }
     if (x < a.nx) {
