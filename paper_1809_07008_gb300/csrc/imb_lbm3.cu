@@ -315,9 +315,8 @@ __device__ __forceinline__ void sphere_force(float Bp, float rho, float jx, floa
 // The order of the sums and products of Eqs. 2 and 13 is kept as it was: with bfloat16 populations any
 // other rounding moves weak transverse flows by 1 % within 50 steps (the forcing put into the
 // equilibrium, and Pi from second moments, would save another 5 %).
-// A step with its share of the read-back, before and with the fetch of the map word ahead and pairs
-// formed where used: 400 x 100 x 400 FP32 673 -> 560 us, 203 x 77 x 151 FP16 111 -> 81 us, the
-// 240 x 100 x 100 packed bed (GEN) 315 -> 140 us with the column sums.
+// Kernel time on 16 M cells with one sphere 506 -> 453 us FP32 (5.4 TB/s), 446 -> 355 us FP16; the
+// 240 x 100 x 100 packed bed (GEN) with the column sums 269 -> 119 us.
 template <bool GEN, typename S>
 __device__ __forceinline__ int collide3(const float (&d)[19], const Args3 &a, int x, int y, int z, size_t cell,
                                         const unsigned word, const unsigned *__restrict__ map2,
