@@ -1012,6 +1012,7 @@ __device__ __forceinline__ void warp_islands(const DemArgs &d, WarpIslands &w, c
         }
         --quiet;
         if (__any_sync(0xffffffffu, contact)) quiet = 0;   // speeds changed
+        __syncwarp();   // the vote orders no memory: the states are read, on, f and xi overwritten by other lanes
     }
     if (act) {
         const int fin = d.N_sub & 1;
