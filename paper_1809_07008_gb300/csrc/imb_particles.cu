@@ -1329,6 +1329,7 @@ __global__ void __launch_bounds__(CL_THREADS) k_dem_cluster(const DemArgs d) {
                 }
                 fh = -Fn * nh + Ft * th;
             }
+            __syncwarp();   // xi is read by both lanes, and by the lanes past the list, before it is overwritten
             if (act) {
                 S.f[h][t] = fh;
                 if (h) S.xi[t] = xi;

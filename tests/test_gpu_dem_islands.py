@@ -1,7 +1,8 @@
 """Islands of 2 to 32 particles, whose lanes hand their particles' state to each other in every
 sub-cycle, bit for bit against the sequential FP64 evaluation: two lanes, the largest island that
 shares a warp, one more, a whole warp, walls beside the island, several islands to a warp, and an
-island of more pairs than are evaluated a lane each (stepped particle by particle)."""
+island of more pairs than are evaluated a lane each (stepped particle by particle).  Two islands above
+a warp, whose contacts two lanes share, stand beside them."""
 import numpy as np
 import pytest
 
@@ -38,6 +39,10 @@ CASES = {
     "warp at a wall": (block(32, 8, 5.0, 0.02, 7, at=(5.01, 5.01)), 1.0),
     "hertz-mindlin": (block(32, 8, 5.0, 0.02, 8, contact_model=1, E_young=2.0e4, nu_poisson=0.3), 1.0),
     "particle by particle": (block(32, 8, 3.0, 0.05, 9), 6.5),   # twelve candidates a disk inside, over 96 pairs
+    # above a warp, two lanes a contact that share its spring (the last lanes of the list idle)
+    "cluster at a wall": (block(45, 9, 5.0, 0.02, 10, at=(5.01, 5.01)), 1.0),
+    "cluster, hertz-mindlin at a wall": (block(45, 9, 5.0, 0.02, 11, at=(5.01, 5.01), contact_model=1, E_young=2.0e4,
+                                               nu_poisson=0.3), 1.0),
 }
 
 
