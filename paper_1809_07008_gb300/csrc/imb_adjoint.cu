@@ -15,6 +15,7 @@
 //     f(nx-1) = f^eq(1, u of column nx-2)), adding d J / d u_in.
 // d E / d (disk centre) is the difference of the chord lengths on opposite cell edges.
 #include "imb_device.cuh"
+#include "imb_host.h"
 #include "imb_kernels.h"
 #include "imb_pull.cuh"
 
@@ -62,29 +63,30 @@ __device__ __forceinline__ float tree9(const float (&v)[9]) {
 // and outlet columns of the pull that gave f(t) from S0 follows in the same launch: f(0) =
 // f^eq(rho of column 1, u_in) and f(nx-1) = f^eq(1, u of column nx-2) hand the adjoint of columns 0
 // and nx - 1 on to the threads of columns 1 and nx - 2, which hold the pulled f(t) they need, and
-// the row's d J / d u_in to g_uin (the launch keeps columns nx - 2 and nx - 1 in one block).
+// the row's d J / d u_in to g_uin (columns 0 and 1, and nx - 2 and nx - 1, share a block: adjoint_grid).
 //
 // d J / d tau is summed in pairs of FP32 over the block (an FP64 add takes a warp 64 cycles, and
 // every warp's shuffle tree took five of them).  The adjoint itself keeps the order of its sums:
 // taken on opposite pairs it has fewer instructions and is no faster on 512 x 256 cells (42 us a
 // forward and reverse step, 84 before the launches and copies were saved), but where the adjoint front
 // has not reached the inlet d J / d u_in is rounding noise, which any other order changes whole.
-__global__ void __launch_bounds__(256) k_adjoint_step(const float *__restrict__ lam1, const float *__restrict__ S0,
+__global__ void __launch_bounds__(ADJ_BLOCK) k_adjoint_step(const float *__restrict__ lam1, const float *__restrict__ S0,
                                                       float *__restrict__ lam0, const LatticeArgs a,
                                                       const float *__restrict__ E, double *__restrict__ gE,
-                                                      float inv_T, double *g_tau, int inlet, double *g_uin) {
+                                                      float inv_T, double *g_tau, int inlet, double *g_uin, int shift) {
     cudaGridDependencySynchronize();   // launched as a dependent of the kernel before it
     cudaTriggerProgrammaticLaunchCompletion();
     __shared__ float edge[2][9];
     __shared__ float2 part[8];
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
+    const int x = (int)(blockIdx.x * blockDim.x + threadIdx.x) - shift, y = blockIdx.y;
+    const bool in = x >= 0 && x < a.nx;
     float gt = 0.0f, gt_lo = 0.0f;
     lam1 += a.origin;   // node (0, 0) of plane 0 in the frame
     S0 += a.origin;
     lam0 += a.origin;
     float v[9];
     float col_rho = 1.0f, col_ux = 0.0f, col_uy = 0.0f;
-    if (x < a.nx) {
+    if (in) {
         // adjoint of P(t) at (x, y): who pulled P_q(x, y); and f(t) at (x, y), pulled from
         // P(t-1) (shifted populations d = f - w).  Away from the edges no boundary rule applies.
         float L[9], d[9];
@@ -223,7 +225,7 @@ __global__ void __launch_bounds__(256) k_adjoint_step(const float *__restrict__ 
             if (g != 0.0f) atomicAdd(g_uin, (double)(g * col_rho));
         }
     }
-    if (x < a.nx) {
+    if (in) {
 #pragma unroll
         for (int q = 0; q < 9; ++q) lam0[(size_t)q * a.plane + (size_t)y * a.pitch + x] = v[q];
     }
@@ -288,18 +290,17 @@ cudaError_t launch_cell_E(const int *count, const float *eps, size_t ncell, floa
 cudaError_t launch_adjoint_step(const float *lam1, const float *S0, float *lam0, const LatticeArgs &a,
                                 const float *E, double *gE, float inv_T, double *g_tau, bool inlet, double *g_uin,
                                 cudaStream_t s) {
-    int block = 256;   // columns nx - 2 and nx - 1 in one block
-    while (inlet && a.nx % block == 1) block -= 32;
+    const AdjointGrid g = adjoint_grid(a.nx, inlet);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((a.nx + block - 1) / block, a.ny);
-    cfg.blockDim = dim3(block);
+    cfg.gridDim = dim3(g.blocks, a.ny);
+    cfg.blockDim = dim3(ADJ_BLOCK);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_adjoint_step, lam1, S0, lam0, a, E, gE, inv_T, g_tau, (int)inlet, g_uin);
+    return cudaLaunchKernelEx(&cfg, k_adjoint_step, lam1, S0, lam0, a, E, gE, inv_T, g_tau, (int)inlet, g_uin, g.shift);
 }
 
 cudaError_t launch_position_grad(const int *count, const int *ids, const double *gE, const double *x,
