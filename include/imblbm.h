@@ -141,9 +141,9 @@ int imb_step(imb_ctx *ctx, int n);
  * then n coupling cycles run, then the force F_out[2n] and torque T_out[n] of the last
  * cycle and the particle state x_out[2n], v_out[2n], omega_out[n] are read back (each
  * output may be NULL).  Everything is queued on the context stream and the call waits
- * once; for pinned host arrays the copies are asynchronous, and when every array given is
- * pinned memory the device can address (cudaHostAlloc'd or mapped), one kernel reads the
- * inputs and one writes the outputs through host memory instead.  Errors as imb_step and
+ * once; for pinned host arrays the copies are asynchronous, and when every array given lies
+ * whole in one pinned allocation or registration the device can address, 8-byte aligned,
+ * one kernel reads the inputs and one writes the outputs through host memory instead.  Errors as imb_step and
  * imb_set_kinematics.  After IMB_E_TIMEOUT the copies into the output arrays may still be
  * queued: the caller must keep those arrays alive and unused until imb_sync returns
  * IMB_OK or the context is destroyed. */
@@ -162,7 +162,10 @@ int imb_dem_step(imb_ctx *ctx, int n);
 int imb_sync(imb_ctx *ctx);
 
 /* Populations f_i(x, t) of Eq. 1 -- after streaming, before the collision of the
- * next step -- as 9 * nx * ny doubles, layout [q][y][x] (x fastest, no pitch). */
+ * next step -- as 9 * nx * ny doubles, layout [q][y][x] (x fastest, no pitch).
+ * Any host array will do, here and in the other calls that read fields back; one that lies
+ * whole in one pinned allocation or registration, 8-byte aligned, is written in place by
+ * the kernel, any other one through a device buffer and a copy, to the same values. */
 int imb_get_populations(imb_ctx *ctx, double *f);
 
 /* Macroscopic fields (Eqs. 3-4, 6) from f(x, t): density and velocity (with the

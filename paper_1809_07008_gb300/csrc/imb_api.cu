@@ -16,6 +16,7 @@
 
 #include "../../include/imblbm.h"
 #include "imb_device.cuh"
+#include "imb_host.h"
 #include "imb_kernels.h"
 
 using namespace imb;
@@ -632,13 +633,41 @@ static bool centres_inside(const double *x, int n, int nx, int ny) {
     return ok != 0;
 }
 
+// One driver call gives the kind of memory p points to, the address the device sees and the bounds
+// of the allocation or registration (zeros for memory CUDA doesn't know).  The first and the last
+// element of an array may lie in two registrations with pageable memory between them, and a copy
+// takes addresses that a store does not, so the bounds and the alignment are looked at.
+namespace imb {
+void *pinned_span(void *p, size_t bytes, size_t align) {
+    static const PFN_cuPointerGetAttributes_v7000 query = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &fn, 7000, cudaEnableDefault, &q);
+        return (PFN_cuPointerGetAttributes_v7000)(e == cudaSuccess && q == cudaDriverEntryPointSuccess ? fn : nullptr);
+    }();
+    if (!p || !bytes || !query) return nullptr;
+    CUpointer_attribute ids[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                 CU_POINTER_ATTRIBUTE_DEVICE_POINTER, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                 CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    unsigned type = 0, managed = 0;
+    CUdeviceptr dev = 0, start = 0;
+    size_t size = 0;
+    void *data[] = {&type, &managed, &dev, &start, &size};
+    if (query(5, ids, data, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) return nullptr;
+    if (type != CU_MEMORYTYPE_HOST || managed || !dev) return nullptr;
+    return span_covered((uintptr_t)dev, bytes, align, (uintptr_t)start, size) ? (void *)(uintptr_t)dev : nullptr;
+}
+}  // namespace imb
+
 extern "C" int imb_set_kinematics(imb_ctx *c, const double *x, const double *v, const double *omega) {
     if (!c) return IMB_E_INVALID_ARG;
     if (c->np == 0) return IMB_OK;
     if (!x || !v || !omega) return fail(c, IMB_E_INVALID_ARG, "bad kinematics arrays");
     if (!centres_inside(x, c->np, c->nx, c->ny))
         return fail(c, IMB_E_INVALID_ARG, "particle centre outside [0,nx) x [0,ny)");
-    const double *dx = device_view(x), *dv = device_view(v), *dw = device_view(omega);
+    CK(cudaSetDevice(c->device), "cudaSetDevice");
+    const size_t np = (size_t)c->np;
+    const double *dx = device_span(x, 2 * np), *dv = device_span(v, 2 * np), *dw = device_span(omega, np);
     if (dx && dv && dw) {   // one launch reads the three arrays from host memory
         CK(launch_kinematics_in(dx, dv, dw, c->x, c->v, c->w, c->np, c->stream), "upload kinematics");
         c->launches++;
@@ -878,7 +907,7 @@ extern "C" int imb_step_io(imb_ctx *c, int n, const double *x_in, const double *
     double *outs[5] = {F_out, T_out, x_out, v_out, omega_out}, *dev[5];
     bool mapped = true;
     for (int k = 0; k < 5; ++k) {
-        dev[k] = device_view(outs[k]);
+        dev[k] = device_span(outs[k], k == 1 || k == 4 ? np : 2 * np);
         if (outs[k] && !dev[k]) mapped = false;
     }
     if (np && mapped) {   // one launch writes every output into host memory
@@ -941,8 +970,9 @@ extern "C" int imb_get_macro(imb_ctx *c, double *rho, double *ux, double *uy) {
     // Pinned arrays the device can address are written by the gather itself, over the link the
     // copies would take, without the device buffer (24 B a cell allocated, written, read and
     // freed on every call).  8192 x 4096: 8.8 -> 4.3 ms.
+    const void *out[3] = {rho, ux, uy};
     double *hr = device_span(rho, n), *hx = device_span(ux, n), *hy = device_span(uy, n);
-    if (hr && hx && hy) {
+    if (hr && hx && hy && spans_disjoint(out, 3, n * sizeof(double))) {
         CK(launch_gather(c->fbuf[c->cur], c->p.storage, a, nullptr, hr, hx, hy, c->stream), "gather");
         c->launches++;
         return imb_sync(c);

@@ -28,25 +28,13 @@ static cudaError_t launch_dependent(void (*kernel)(P...), int grid, int block, i
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<A &&>(args)...);
 }
 
-// The device address of a pinned host array the device can address (page-locked and mapped,
-// as cudaHostAlloc / cudaHostRegister give under unified addressing), else NULL.
-template <typename T>
-static inline T *device_view(T *p) {
-    if (!p) return nullptr;
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();   // clear the error an unknown pointer leaves
-        return nullptr;
-    }
-    return at.type == cudaMemoryTypeHost ? static_cast<T *>(at.devicePointer) : nullptr;
-}
-
-// The same for an array of n elements: its first and its last one lie in such memory, the
-// right distance apart.
+// The device address of a pinned host array of n elements that a kernel can read and write in place:
+// aligned for its type, and the whole of it in one page-locked allocation or registration the
+// device can address (pinned_span); else NULL (the array then goes through a copy).
+void *pinned_span(void *p, size_t bytes, size_t align);
 template <typename T>
 static inline T *device_span(T *p, size_t n) {
-    T *a = device_view(p);
-    return a && n && device_view(p + (n - 1)) == a + (n - 1) ? a : nullptr;
+    return static_cast<T *>(pinned_span(const_cast<std::remove_const_t<T> *>(p), n * sizeof(T), alignof(T)));
 }
 
 struct PRec;

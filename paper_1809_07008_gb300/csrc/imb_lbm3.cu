@@ -23,6 +23,7 @@
 
 #include "../../include/imblbm.h"
 #include "imb_device.cuh"
+#include "imb_host.h"
 #include "imb_kernels.h"
 
 namespace imb3 {
@@ -877,7 +878,8 @@ extern "C" int imb3_get_macro(imb3_ctx *c, double *rho, double *ux, double *uy, 
     const size_t n = c->a.plane;
     // pinned arrays the device can address are written by the kernel itself (as imb_get_macro)
     double *h[4] = {imb::device_span(rho, n), imb::device_span(ux, n), imb::device_span(uy, n), imb::device_span(uz, n)};
-    if (h[0] && h[1] && h[2] && h[3]) {
+    const void *out[4] = {rho, ux, uy, uz};
+    if (h[0] && h[1] && h[2] && h[3] && imb::spans_disjoint(out, 4, n * sizeof(double))) {
         CK3(by_storage3(c->p.storage, [&](auto tag) {
                 using S = std::remove_pointer_t<decltype(tag)>;
                 k3_macro<S><<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>((const S *)c->buf[c->cur], c->a, h[0], h[1],

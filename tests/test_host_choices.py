@@ -37,3 +37,25 @@ int main() {
         }
 }
 """)
+
+
+def test_pinned_span_decision(tmp_path):
+    # an array is written in place only where it is aligned and one memory range holds all of it
+    run_cpp(tmp_path, """
+int main() {
+    const uintptr_t s = 0x10000;                                  // the range [s, s + 4096)
+    CHECK(span_covered(s, 4096, 8, s, 4096));
+    CHECK(span_covered(s + 4088, 8, 8, s, 4096));
+    CHECK(!span_covered(s, 4097, 8, s, 4096));
+    CHECK(!span_covered(s + 8, 4096, 8, s, 4096));
+    CHECK(!span_covered(s - 8, 16, 8, s, 4096));
+    CHECK(!span_covered(s, 8192, 8, s, 4096));                    // ends in a second registration
+    CHECK(!span_covered(s + 4, 64, 8, s, 4096));                  // not on a multiple of 8
+    CHECK(!span_covered(s + 4100, 0, 4, s, 4096) && !span_covered(s, 0, 8, s, 4096));
+    CHECK(!span_covered(s + 8, SIZE_MAX - 7, 8, s, 4096));        // no wrap-around
+    CHECK(!span_covered(s, 8, 8, 0, 0));                          // memory the driver doesn't know
+    const char *b = (const char *)s;
+    const void *apart[] = {b, b + 64, b + 128}, *meet[] = {b, b + 64, b + 120}, *twice[] = {b, b + 64, b + 64};
+    CHECK(spans_disjoint(apart, 3, 64) && !spans_disjoint(meet, 3, 64) && !spans_disjoint(twice, 3, 64));
+}
+""")
