@@ -319,6 +319,20 @@ __device__ __forceinline__ void drift(const DemArgs &d, double &px, double &py, 
     if (d.bc_y == BC_PERIODIC) py = wrap_axis(py, d.Ly);
 }
 
+// Whether a wall of an axis can touch a particle there, by the high words of the coordinate: below
+// lo = word(r) + 1 or from hi = word(L - r) on it may, else the particle is further than r from both
+// (a word holds 20 bits of the mantissa, so only what is within 1e-6 of touching goes on to the FP64
+// test; below zero the word is negative, NaN is above hi).  An axis without walls never.
+struct WallReach {
+    int lo, hi;
+    __device__ __forceinline__ bool low(double x) const { return __double2hiint(x) < lo; }
+    __device__ __forceinline__ bool high(double x) const { return __double2hiint(x) >= hi; }
+};
+__device__ __forceinline__ WallReach wall_reach(int bc, double L, double r) {
+    if (bc != BC_WALL) return {(int)0x80000000, 0x7fffffff};
+    return {__double2hiint(r) + 1, __double2hiint(L - r)};
+}
+
 // Eqs. 10-11, leapfrog kick-drift.
 __device__ __forceinline__ void integrate(const DemArgs &d, int p, double Fcx, double Fcy, double Tc,
                                           double &px, double &py, double &vx, double &vy, double &w) {
@@ -902,19 +916,7 @@ __device__ __forceinline__ void warp_islands(const DemArgs &d, WarpIslands &w, c
     double xiw[4];   // wall springs, in registers on the pair-parallel path
 #pragma unroll
     for (int q = 0; q < 4; ++q) xiw[q] = act ? d.wall_xi[4 * p + q] : 0.0;
-    // a wall within reach of a lane's particle in this cycle (a particle that moves further than
-    // skin / 2 raises IMB_E_SKIN); else no wall touches and the springs are released
-    bool near_wall = false;
-    if (act) {
-        const double g = rp + d.skin, x = w.st[0][0][lane], y = w.st[0][1][lane];
-        near_wall = (d.bc_x == BC_WALL && (x < g || d.Lx - x < g)) ||
-                    (d.bc_y == BC_WALL && (y < g || d.Ly - y < g));
-    }
-    const bool walls = __any_sync(0xffffffffu, near_wall);
-    if (!walls) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) xiw[q] = 0.0;
-    }
+    const WallReach reach_x = wall_reach(d.bc_x, d.Lx, rp), reach_y = wall_reach(d.bc_y, d.Ly, rp);
     // Sub-cycles without an overlap test: while nothing touches, a particle's speed along an axis
     // stays below |v| + N_sub |kick|, so two particles close their gap by at most the sum of these
     // bounds times dt a sub-cycle.  After a test in which no pair of the warp touched, as many
@@ -989,7 +991,12 @@ __device__ __forceinline__ void warp_islands(const DemArgs &d, WarpIslands &w, c
                     Tc += rp * w.f[2][k];
                     touched = true;
                 }
-                if (walls) touched |= wall_contacts(d, p, px, py, vx, vy, om, rp, mp, xiw, Fcx, Fcy, Tc);
+                if (reach_x.low(px) || reach_x.high(px) || reach_y.low(py) || reach_y.high(py)) {
+                    touched |= wall_contacts(d, p, px, py, vx, vy, om, rp, mp, xiw, Fcx, Fcy, Tc);
+                } else {   // no wall touches: the springs are released
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) xiw[q] = 0.0;
+                }
                 if (touched) integrate(d, p, Fcx, Fcy, Tc, px, py, vx, vy, om);
                 else coast(d, kick, px, py, vx, vy, om);
                 contact = touched;
@@ -1077,7 +1084,7 @@ struct ClusterDem {
     double xi[CL_Q], cn[CL_Q], R[CL_Q], RR[CL_Q];
     double f[3][CL_Q];                   // fx, fy, Ft on the contact's first particle
     uint32_t pa[CL_Q];                   // cluster address of st[0][0] of the second particle
-    int id[CL_P];
+    int id[CL_P], wall_hi[2][CL_P];      // WallReach::hi of the two axes
     unsigned short slot[CL_P][MAX_NBR + 4];   // contact of candidate j / wall, 0x8000: its second particle; 0xffff none
     unsigned short pi[CL_Q], touch[CL_Q];
     unsigned char nn[CL_P], kind[CL_Q], on[CL_Q];   // kind: 0 pair, 1 + wall
@@ -1100,6 +1107,21 @@ __device__ __forceinline__ unsigned long long morton_key(const DemArgs &d, int p
     for (int k = 0, x = b % d.nbx, y = b / d.nbx; k < 15; ++k)
         m |= (unsigned long long)(((x >> k) & 1) | (((y >> k) & 1) << 1)) << (2 * k);
     return (m << 32) | (unsigned)p;   // unique
+}
+
+// A contact of particle k with wall wl: its place in the block's table, -1 when that is full.
+__device__ __forceinline__ int add_wall(const DemArgs &d, ClusterDem &S, int k, int wl, double xi) {
+    const int e = atomicAdd(&S.ncon, 1);
+    if (e >= CL_Q) return -1;
+    S.pi[e] = (unsigned short)k;
+    S.pa[e] = 0;
+    S.kind[e] = (unsigned char)(1 + wl);
+    S.xi[e] = xi;
+    S.cn[e] = d.model == 1 ? 0.0 : damping_cn(d, S.mi[0][k]);
+    S.R[e] = S.r[k];
+    S.RR[e] = 0.0;
+    S.slot[k][MAX_NBR + wl] = (unsigned short)e;
+    return e;
 }
 
 __device__ __forceinline__ void store_cluster_state(const DemArgs &d, const ClusterDem &S, int nl) {
@@ -1189,25 +1211,17 @@ __global__ void __launch_bounds__(CL_THREADS) k_dem_cluster(const DemArgs d) {
                     if (d.nbr_id[q * MAX_NBR + jq] == p) S.slot[kq][jq] = (unsigned short)(e | 0x8000);
             }
         }
-        // walls the particle may reach within the cycle: it moves skin / 2 at most (else IMB_E_SKIN)
+        // walls within the skin; one that a particle reaches from further off is added on the way
+        S.wall_hi[0][k] = wall_reach(d.bc_x, d.Lx, rp).hi;
+        S.wall_hi[1][k] = wall_reach(d.bc_y, d.Ly, rp).hi;
         for (int wl = 0; wl < 4; ++wl) {
             if ((wl < 2 ? d.bc_x : d.bc_y) != BC_WALL) continue;
             const double c = wl < 2 ? d.x[2 * p] : d.x[2 * p + 1], L = wl < 2 ? d.Lx : d.Ly;
-            if (!(((wl & 1) ? L - c : c) < rp + d.skin)) continue;
-            const int e = atomicAdd(&S.ncon, 1);
-            if (e >= CL_Q) continue;
-            S.pi[e] = (unsigned short)k;
-            S.pa[e] = 0;
-            S.kind[e] = (unsigned char)(1 + wl);
-            S.xi[e] = d.wall_xi[4 * p + wl];
-            S.cn[e] = d.model == 1 ? 0.0 : damping_cn(d, mp);
-            S.R[e] = rp;
-            S.RR[e] = 0.0;
-            S.slot[k][MAX_NBR + wl] = (unsigned short)e;
+            if (((wl & 1) ? L - c : c) < rp + d.skin) add_wall(d, S, k, wl, d.wall_xi[4 * p + wl]);
         }
     }
     __syncthreads();
-    const int ncon = S.ncon;
+    int ncon = S.ncon;
     if (tid == 0 && ncon > CL_Q) atomicOr(&d.counters[7], 1);
     cluster_barrier();   // the blocks' states and the flag are in place
     if (__ldcg(&d.counters[7])) {   // a block's contacts don't fit its table: particle by particle
@@ -1244,12 +1258,32 @@ __global__ void __launch_bounds__(CL_THREADS) k_dem_cluster(const DemArgs d) {
         return;
     }
     const bool perx = d.bc_x == BC_PERIODIC, pery = d.bc_y == BC_PERIODIC;
+    const bool wallx = d.bc_x == BC_WALL, wally = d.bc_y == BC_WALL;
     const uint32_t R_OFF = (uint32_t)(offsetof(ClusterDem, r) - offsetof(ClusterDem, st));
     const double rkt = 1.0 / d.kt;
     for (int s = 0; s < d.N_sub; ++s) {
         const int cur = s & 1;
         const double(*st)[CL_P] = S.st[cur];
         const uint32_t so = (uint32_t)cur * 5u * CL_P * 8u;   // of st[cur] from st[0]
+        // a wall that a particle comes to from beyond the skin: its contact joins the table (read past
+        // ncon, which takes it up below) and is tested here
+        for (int u = tid; u < 2 * nl && (wallx || wally); u += CL_THREADS) {
+            const int c = u < nl ? 0 : 1, k = u - c * nl;
+            const double x = st[c][k], R = S.r[k];
+            const WallReach reach = {__double2hiint(R) + 1, S.wall_hi[c][k]};
+            for (int wl = 2 * c; wl < 2 * c + 2; ++wl) {
+                if (!((wl & 1) ? reach.high(x) : reach.low(x)) || !(c ? wally : wallx)) continue;
+                if (S.slot[k][MAX_NBR + wl] != 0xffff) continue;
+                const int e = add_wall(d, S, k, wl, 0.0);
+                if (e < 0) {
+                    set_err(d.err, ERR_SKIN);   // no room (and the particle moved more than the skin)
+                    continue;
+                }
+                const bool hit = ((wl & 1) ? (c ? d.Ly : d.Lx) - x : x) < R;
+                S.on[e] = hit;
+                if (hit) S.touch[atomicAdd(&S.ntouch, 1)] = (unsigned short)e;
+            }
+        }
         for (int t = tid; t < ncon; t += CL_THREADS) {
             const int i = S.pi[t], kd = S.kind[t];
             bool hit;
@@ -1337,6 +1371,7 @@ __global__ void __launch_bounds__(CL_THREADS) k_dem_cluster(const DemArgs d) {
             }
         }
         __syncthreads();
+        ncon = min(S.ncon, CL_Q);
         if (tid == 0) S.ntouch = 0;
         for (int u = tid; u < 3 * nl; u += CL_THREADS) {
             const int c = u < nl ? 0 : (u < 2 * nl ? 1 : 2), k = u - c * nl;
