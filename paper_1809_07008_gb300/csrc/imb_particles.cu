@@ -24,6 +24,7 @@
 #include <cstddef>
 
 #include "imb_device.cuh"
+#include "imb_host.h"
 #include "imb_kernels.h"
 
 namespace imb {
@@ -1041,21 +1042,6 @@ __device__ __forceinline__ void warp_islands(const DemArgs &d, WarpIslands &w, c
 }
 
 // ------------------------------------------------------------ large islands in one cluster
-// a / b for a constant b > 0 whose correctly rounded reciprocal y = RN(1 / b) is known, rounded
-// to nearest: a faithful quotient from the reciprocal, then one step with the exact remainder
-// (Markstein 1990: with y correctly rounded and q within an ulp, q + r y rounds to a / b).
-// Five FP64 operations, 64 cycles each, instead of the ten of a division.  Zeros, infinities,
-// NaN and exponents near the ends of the range, where the remainder may not be exact, divide.
-__device__ __forceinline__ double div_by(const double a, const double b, const double y) {
-    const unsigned ea = ((unsigned)__double2hiint(a) >> 20) & 0x7ffu, eb = ((unsigned)__double2hiint(b) >> 20) & 0x7ffu;
-    if (ea - 200u < 1600u && eb - 523u < 1000u) {
-        double q = a * y;
-        q = __fma_rn(__fma_rn(-b, q, a), y, q);
-        return __fma_rn(__fma_rn(-b, q, a), y, q);
-    }
-    return a / b;
-}
-
 // Particles of islands larger than a warp, up to CL_P CL_CTAS of them together: one cluster of
 // CL_CTAS blocks holds their state in shared memory (double-buffered), each block a contiguous
 // run of the particles in Morton order of their bins, and reads the other blocks' particles

@@ -59,3 +59,38 @@ int main() {
     CHECK(spans_disjoint(apart, 3, 64) && !spans_disjoint(meet, 3, 64) && !spans_disjoint(twice, 3, 64));
 }
 """)
+
+
+def test_div_by_equals_division(tmp_path):
+    # random significands at the edges of the windows of both operands, within and beyond them, zeros,
+    # infinities, NaN and subnormal values: the quotient of the division, to the bit
+    run_cpp(tmp_path, """
+#include <random>
+static uint64_t bits(double v) { uint64_t b; std::memcpy(&b, &v, 8); return b; }
+static bool same(double a, double b) {
+    const double q = div_by(a, b, 1.0 / b), d = a / b;
+    return bits(q) == bits(d) || (q != q && d != d);
+}
+int main() {
+    std::mt19937_64 g(1);
+    auto real = [&](int e) {   // significand with few or many bits, exponent e
+        uint64_t m = g() >> 12;
+        if (g() & 1) m &= ~0ull << (g() % 52);
+        if (g() & 1) m |= 0xfffffffffffffull >> (g() % 52);
+        return std::ldexp(1.0 + (double)(m & 0xfffffffffffffull) * 0x1p-52, e);
+    };
+    const int edge[] = {-1022, -823, -700, -401, -400, -399, -60, -1, 0, 1, 40, 398, 399, 400, 401, 500, 700, 776, 1023};
+    for (int ea : edge)
+        for (int eb : edge)
+            for (int k = 0; k < 4000; ++k) {
+                const double a = real(ea), b = real(eb);
+                CHECK(same(a, b) && same(-a, b));
+            }
+    for (int k = 0; k < 20000000; ++k) CHECK(same(real((int)(g() % 60) - 30), real((int)(g() % 40))));
+    const double odd[] = {0.0, -0.0, (double)INFINITY, -(double)INFINITY, (double)NAN, 5e-324, 1e-310};
+    for (double a : odd)
+        for (int eb : edge) CHECK(same(a, real(eb)));
+    for (double a : odd)
+        for (double b : {(double)INFINITY, 5e-324, 1e-310}) CHECK(same(a, b) && same(1.5, b));
+}
+""")
