@@ -235,7 +235,9 @@ int imb_binomial_schedule(int T, int snapshots, int *ops, int max_ops, int *n_op
  * single-lattice path), and n_disks[d] disks held at rest: their centres are
  * disk_xy[2j], disk_xy[2j+1] in the domain's cell units and radii disk_r[j], the
  * disks of domain 0 first, then those of domain 1, and so on.  Populations are
- * stored as f - w in `storage` (IMB_STORE_*).  Every step advances all domains
+ * stored as f - w in `storage` (IMB_STORE_*), two copies of 9 values a cell with rows padded
+ * to 32 (FP32) or 64 cells, without padding where the domains are narrow (a mean width
+ * below 64, with 16 bits 31, in small batches 8 cells) or memory is short.  Every step advances all domains
  * with the collision of Eq. 13 (B of Eq. 14 from the summed exact overlap area of
  * each cell, u_s = 0) and adds each domain's drag (Eq. 15, summed over its disks)
  * to an accumulator.  The library owns the batch; host arrays are copied.
@@ -253,7 +255,8 @@ int imb_batch_create(imb_batch **out, int n_domains, const int *nx, const int *n
 int imb_batch_run(imb_batch *b, int steps);
 
 /* Time `steps_per_trial` steps of each launch shape (blocks of 128, 256 or
- * 512 threads, where the kernel can launch them; one or two cells per lane along a row) on the batch itself, keep the
+ * 512 threads, where the kernel can launch them; one or two cells per lane along a row, always
+ * one where rows are not padded) on the batch itself, keep the
  * fastest, and put the state and the drag accumulators back as they were.  Outputs
  * (each may be NULL): the chosen block size, cells per lane and its ms per step. */
 int imb_batch_autotune(imb_batch *b, int steps_per_trial, int *block, int *cells_per_lane,

@@ -5,8 +5,8 @@
 // driven by a body force (Guo forcing, as in the single-lattice path), and holds fixed disks
 // whose summed solid ratio E per cell (exact overlap area, Sec. 2.3) is computed once; its
 // relaxation time may carry the Smagorinsky closure of the single-lattice path.  One
-// launch advances every domain by one step: each warp takes an equal run of row segments
-// (finding the domain of its first segment by binary search in the domains' first items),
+// launch advances every domain by one step: each warp takes an equal run of items of 32 or 64 cells
+// (finding the domain of its first item by binary search in the domains' first items),
 // pulls with the periodic wrap of the domain (Eq. 1), collides with the blend of Eq. 13
 // (B from Eq. 14, u_s = 0 for disks at rest) and adds the drag B (j - F) (Eq. 15) of the
 // nodes it stepped to the domain's accumulator.  Steps run as a replayed CUDA graph of two launches (A -> B,
@@ -21,6 +21,7 @@
 
 #include "../../include/imblbm.h"
 #include "imb_device.cuh"
+#include "imb_host.h"
 #include "imb_kernels.h"
 
 namespace imb {
@@ -30,10 +31,11 @@ struct BatchDomain {
     int item0[2];       // first work item of the domain, with one and with two cells per lane
     size_t off;         // element offset of the domain in the population buffers
     size_t row;         // elements from one row to the next
-    size_t e_off;       // offset of the domain's solid ratios, rows of 2 ceil(nx / 2) (even)
+    size_t e_off;       // offset of the domain's solid ratios
+    int plane;          // whole planes: elements of one (blocked rows: 0)
+    int e_row;          // solid ratios from one row to the next (blocked rows: even)
     float tau, omega0, Fx, Fy;
     float smag_coef;    // 18 sqrt(2) C^2 of the Smagorinsky closure (0: plain BGK)
-    float pad2;
 };
 
 // Layout of the populations: rows of blocks of 128 bytes per plane, the nine planes of a block one
@@ -41,6 +43,11 @@ struct BatchDomain {
 // reach every plane: with whole planes one after another a node's nine loads and nine stores took
 // some 40 of its 330 instructions for addresses.  The planes that a node pulls from the same row
 // (c_y = 0, 1, -1) are neighbours: slots 3 g, 3 g + 1, 3 g + 2 hold c_x = 0, 1, -1.
+//
+// Rows padded to whole blocks take up to 21 times the memory of their cells (three cells of 16
+// bits in a block of 64).  A batch of narrow domains, or one that the padding would push out of memory
+// (blocked_rows), holds whole planes instead ([slot][y][x], no padding) and is stepped with one cell a
+// lane.
 template <typename S> __host__ __device__ constexpr int segb() { return 128 / (int)sizeof(S); }
 __host__ __device__ constexpr int group_q(int g, int k) { return (g == 0 ? 0x310 : g == 1 ? 0x652 : 0x784) >> (4 * k) & 15; }
 __host__ __device__ constexpr int slot_of(int q) {
@@ -51,10 +58,23 @@ __host__ __device__ constexpr int slot_of(int q) {
 static_assert(cy_of(2) == 1 && cy_of(5) == 1 && cy_of(6) == 1 && cy_of(4) == -1 && cy_of(8) == -1 && cy_of(7) == -1 &&
                   cx_of(1) == 1 && cx_of(5) == 1 && cx_of(8) == 1 && cx_of(3) == -1 && cx_of(6) == -1 && cx_of(7) == -1,
               "groups of the planes by source row");
-// element offset of cell x in a row, slot 0
+// element offset of cell x in a blocked row, slot 0
 template <typename S> __host__ __device__ __forceinline__ int col_of(int x) {
     return x / segb<S>() * 9 * segb<S>() + x % segb<S>();
 }
+// where a cell of a row and a slot of it lie
+template <typename S> struct BlockedRows {
+    __device__ __forceinline__ explicit BlockedRows(const BatchDomain &) {}
+    __device__ __forceinline__ int col(int x) const { return col_of<S>(x); }
+    __device__ __forceinline__ int slot(int i) const { return i * segb<S>(); }
+};
+struct WholePlanes {
+    int plane;
+    __device__ __forceinline__ explicit WholePlanes(const BatchDomain &D) : plane(D.plane) {}
+    __device__ __forceinline__ int col(int x) const { return x; }
+    __device__ __forceinline__ int slot(int i) const { return i * plane; }   // 9 nx ny < 2^31 (checked)
+};
+template <typename S, bool BLOCKED> using Layout = std::conditional_t<BLOCKED, BlockedRows<S>, WholePlanes>;
 
 // The node of a domain whose disks are at rest.  With u_s = 0 the solid operator of Eq. 12
 // summed over the covering disks is B (f_{-q} - f^eq_{-q}(u) + f^eq_q(0) - f_q); in the
@@ -187,13 +207,14 @@ template <typename S, int CPL> struct Pulled;
 template <typename S> struct Pulled<S, 1> {
     S r[9];
     float e;
-    __device__ __forceinline__ void fetch(const S *const (&R)[3], const float *Er, int x, int nx) {
-        const int c = col_of<S>(x), cl = col_of<S>(x == 0 ? nx - 1 : x - 1), cr = col_of<S>(x == nx - 1 ? 0 : x + 1);
+    template <class L>
+    __device__ __forceinline__ void fetch(const S *const (&R)[3], const float *Er, int x, int nx, const L lay) {
+        const int c = lay.col(x), cl = lay.col(x == 0 ? nx - 1 : x - 1), cr = lay.col(x == nx - 1 ? 0 : x + 1);
 #pragma unroll
         for (int g = 0; g < 3; ++g) {
-            r[3 * g] = __ldg(R[g] + c + 3 * g * segb<S>());
-            r[3 * g + 1] = __ldg(R[g] + cl + (3 * g + 1) * segb<S>());
-            r[3 * g + 2] = __ldg(R[g] + cr + (3 * g + 2) * segb<S>());
+            r[3 * g] = __ldg(R[g] + c + lay.slot(3 * g));
+            r[3 * g + 1] = __ldg(R[g] + cl + lay.slot(3 * g + 1));
+            r[3 * g + 2] = __ldg(R[g] + cr + lay.slot(3 * g + 2));
         }
         e = __ldg(Er + x);
     }
@@ -201,9 +222,9 @@ template <typename S> struct Pulled<S, 1> {
 #pragma unroll
         for (int i = 0; i < 9; ++i) d[group_q(i / 3, i % 3)] = to_f32(r[i]);
     }
-    static __device__ __forceinline__ void store(S *p, const float (&d)[9]) {
+    template <class L> static __device__ __forceinline__ void store(S *p, const float (&d)[9], const L lay) {
 #pragma unroll
-        for (int q = 0; q < 9; ++q) Store<S>::st(p + slot_of(q) * segb<S>(), d[q]);
+        for (int q = 0; q < 9; ++q) Store<S>::st(p + lay.slot(slot_of(q)), d[q]);
     }
 };
 // The cells x (even) and x + 1.  A plane with c_x = 0 is one load of both; the others' sources
@@ -213,7 +234,7 @@ template <typename S> struct Pulled<S, 2> {
     typename Pair<S>::T c2[3];
     S l0[3], l1[3], r0[3], r1[3];
     float2 e;
-    __device__ __forceinline__ void fetch(const S *const (&R)[3], const float *Er, int x, int nx) {
+    __device__ __forceinline__ void fetch(const S *const (&R)[3], const float *Er, int x, int nx, const BlockedRows<S>) {
         constexpr int G = segb<S>();
         const int in = x % G, c = x / G * 9 * G + in;
         const int cl = x == 0 ? col_of<S>(nx - 1) : (in == 0 ? c - 8 * G - 1 : c - 1);
@@ -243,7 +264,7 @@ template <typename S> struct Pulled<S, 2> {
             for (int q = 0; q < 9; ++q) d[q].y = d[q].x;
         }
     }
-    static __device__ __forceinline__ void store(S *p, const float2 (&d)[9]) {
+    static __device__ __forceinline__ void store(S *p, const float2 (&d)[9], const BlockedRows<S>) {
 #pragma unroll
         for (int q = 0; q < 9; ++q)
             *reinterpret_cast<typename Pair<S>::T *>(p + slot_of(q) * segb<S>()) = Pair<S>::of(d[q]);
@@ -263,7 +284,7 @@ template <typename S> struct Pulled<S, 2> {
 // With the collision as a sum of d_q + d_-q and d_q - d_-q (half the operations) 156 us and twice
 // the FP32 error; two items ahead 148 us with that form, 176 us (spills) with this one; three
 // blocks an SM (80 registers, spills) 187 us; five of 128 threads 151 us.
-template <typename S, int CPL>
+template <typename S, int CPL, bool BLOCKED>
 __global__ void __launch_bounds__(256, CPL == 2 ? 2 : 3)
 k_batch_step(const S *__restrict__ fin, S *__restrict__ fout, const BatchDomain *__restrict__ dom,
              int ndom, int nitems, const float *__restrict__ E, double *drag, unsigned *err) {
@@ -294,12 +315,12 @@ k_batch_step(const S *__restrict__ fin, S *__restrict__ fout, const BatchDomain 
         const S *src = fin + D.off;
         S *out = fout + D.off;
         const float *Ed = E + D.e_off;
-        const int e_row = (nx + 1) / 2 * 2;
+        const Layout<S, BLOCKED> lay(D);
         auto fetch = [&] {
             if (y >= ny) return;   // past the end of the domain's last item
             const S *R[3] = {src + (size_t)y * D.row, src + (size_t)(y == 0 ? ny - 1 : y - 1) * D.row,
                              src + (size_t)(y == ny - 1 ? 0 : y + 1) * D.row};
-            r.fetch(R, Ed + (size_t)y * e_row, x, nx);
+            r.fetch(R, Ed + (size_t)y * D.e_row, x, nx, lay);
         };
         fetch();
         typename V::T fx = V::all(0.0f), fy = V::all(0.0f);
@@ -308,7 +329,7 @@ k_batch_step(const S *__restrict__ fin, S *__restrict__ fout, const BatchDomain 
             r.values(d, CPL == 2 && x + 1 == nx);
             const auto ec = r.e;
             const bool act = y < ny;
-            S *dst = out + (size_t)y * D.row + col_of<S>(x);
+            S *dst = out + (size_t)y * D.row + lay.col(x);
             x += 32 * CPL;
             while (x >= nx) {   // rows of fewer than 32 CPL cells: several at once
                 x -= width * CPL;
@@ -317,7 +338,7 @@ k_batch_step(const S *__restrict__ fin, S *__restrict__ fout, const BatchDomain 
             if (--n > 0) fetch();   // in flight during this item's arithmetic
             if (act) {
                 if (!rest_node<V>(d, ec, D, fx, fy)) unstable = true;   // Mach guard, also catches NaN
-                Pulled<S, CPL>::store(dst, d);
+                Pulled<S, CPL>::store(dst, d, lay);
             }
         }
         float sx = V::sum(fx), sy = V::sum(fy);   // leaving the domain: add its drag
@@ -350,7 +371,7 @@ __global__ void k_batch_solid(const BatchDomain *__restrict__ dom, const int *__
     const float lox = __fsub_rn((float)di, fx), loy = __fsub_rn((float)dk, fy);
     if (!covers(lox, loy, rf)) return;
     const int i = ((ci + di) % D.nx + D.nx) % D.nx, k = ((cj + dk) % D.ny + D.ny) % D.ny;
-    atomicAdd(&E[D.e_off + (size_t)k * ((D.nx + 1) / 2 * 2) + i], cell_disk_area(lox, loy, rf));
+    atomicAdd(&E[D.e_off + (size_t)k * D.e_row + i], cell_disk_area(lox, loy, rf));
 }
 
 // f(x, t) of one domain (the pull of its post-collision field), as FP64 f = w + (f - w)
@@ -365,8 +386,8 @@ __global__ void k_batch_gather(const S *__restrict__ fin, const BatchDomain *__r
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
         const int xs = (x - cx_of(q) + D.nx) % D.nx, ys = (y - cy_of(q) + D.ny) % D.ny;
-        out[(size_t)q * cells + c] =
-            (double)w_of(q) + (double)Store<S>::ld(fin + D.off + (size_t)ys * D.row + col_of<S>(xs) + slot_of(q) * segb<S>());
+        const size_t at = D.plane ? (size_t)slot_of(q) * D.plane + xs : (size_t)(col_of<S>(xs) + slot_of(q) * segb<S>());
+        out[(size_t)q * cells + c] = (double)w_of(q) + (double)Store<S>::ld(fin + D.off + (size_t)ys * D.row + at);
     }
 }
 
@@ -378,6 +399,7 @@ struct imb_batch {
     int device = 0, storage = 0, elem = 4, ndom = 0, nitems[2] = {0, 0}, ndisk = 0;
     size_t total = 0;          // elements per population buffer
     size_t cells = 0;
+    bool blocked = true;       // layout of the populations
     void *buf[2] = {nullptr, nullptr};
     int cur = 0;               // buffer holding the current post-collision field
     BatchDomain *dom = nullptr;
@@ -418,9 +440,9 @@ cudaError_t by_storage_b(int storage, F &&fn) {
     }
 }
 
-template <typename S, int CPL>
+template <typename S, int CPL, bool BLOCKED>
 cudaError_t launch_step_t(imb_batch *b, int from) {
-    auto k = k_batch_step<S, CPL>;
+    auto k = k_batch_step<S, CPL, BLOCKED>;
     if (b->grid == 0) {   // resident blocks of this configuration (set before any capture)
         int per = 0, sms = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, b->block, 0);
@@ -441,8 +463,9 @@ int max_block(imb_batch *b) {
     by_storage_b(b->storage, [&](auto tag) {
         using S = std::remove_pointer_t<decltype(tag)>;
         cudaFuncAttributes fa{};
-        cudaError_t e = b->cpl == 2 ? cudaFuncGetAttributes(&fa, k_batch_step<S, 2>)
-                                    : cudaFuncGetAttributes(&fa, k_batch_step<S, 1>);
+        cudaError_t e = !b->blocked   ? cudaFuncGetAttributes(&fa, k_batch_step<S, 1, false>)
+                        : b->cpl == 2 ? cudaFuncGetAttributes(&fa, k_batch_step<S, 2, true>)
+                                      : cudaFuncGetAttributes(&fa, k_batch_step<S, 1, true>);
         m = e == cudaSuccess ? fa.maxThreadsPerBlock : 0;
         return e;
     });
@@ -452,7 +475,9 @@ int max_block(imb_batch *b) {
 cudaError_t launch_step(imb_batch *b, int from) {
     return by_storage_b(b->storage, [&](auto tag) {
         using S = std::remove_pointer_t<decltype(tag)>;
-        return b->cpl == 2 ? launch_step_t<S, 2>(b, from) : launch_step_t<S, 1>(b, from);
+        return !b->blocked   ? launch_step_t<S, 1, false>(b, from)
+               : b->cpl == 2 ? launch_step_t<S, 2, true>(b, from)
+                             : launch_step_t<S, 1, true>(b, from);
     });
 }
 
@@ -489,7 +514,7 @@ extern "C" int imb_batch_create(imb_batch **out, int n_domains, const int *nx, c
     b->elem = storage == IMB_STORE_FP32 ? 4 : 2;
     b->ndom = n_domains;
     double rmax = 0.0;
-    size_t cells = 0, e_cells = 0;
+    size_t cells = 0, rows = 0, e_cells = 0, most = 0, padded = 0;
     long long items = 0, items2 = 0;   // work items of 32 and of 64 cells
     const size_t G = storage == IMB_STORE_FP32 ? segb<float>() : segb<__half>();
     int ndisk = 0;
@@ -504,9 +529,6 @@ extern "C" int imb_batch_create(imb_batch **out, int n_domains, const int *nx, c
         D.ny = ny[d];
         D.item0[0] = (int)items;
         D.item0[1] = (int)items2;
-        D.off = b->total;
-        D.row = (nx[d] + G - 1) / G * 9 * G;
-        D.e_off = e_cells;
         D.tau = (float)tau[d];
         D.omega0 = (float)(1.0 / tau[d]);
         D.Fx = (float)Fx[d];
@@ -514,8 +536,9 @@ extern "C" int imb_batch_create(imb_batch **out, int n_domains, const int *nx, c
         D.smag_coef = (float)(18.0 * std::sqrt(2.0) * C_smag[d] * C_smag[d]);
         b->hdom.push_back(D);
         cells += (size_t)nx[d] * ny[d];
-        e_cells += (size_t)(nx[d] + 1) / 2 * 2 * ny[d];
-        b->total += D.row * ny[d];
+        rows += (size_t)ny[d];
+        most = std::max(most, (size_t)nx[d] * ny[d]);
+        padded += (nx[d] + G - 1) / G * G * ny[d];
         items += ((long long)ny[d] * nx[d] + 31) / 32;
         items2 += ((long long)ny[d] * ((nx[d] + 1) / 2) + 31) / 32;
         ndisk += n_disks[d];
@@ -545,6 +568,18 @@ extern "C" int imb_batch_create(imb_batch **out, int n_domains, const int *nx, c
     b->ndisk = ndisk;
     b->cells = cells;
     cudaGetDevice(&b->device);
+    size_t mem_free = 0, mem_total = 0;
+    if (cudaMemGetInfo(&mem_free, &mem_total) != cudaSuccess) cudaGetLastError();
+    b->blocked = blocked_rows(cells, rows, padded, most, (size_t)b->elem, mem_free);
+    for (BatchDomain &D : b->hdom) {
+        D.off = b->total;
+        D.row = b->blocked ? (D.nx + G - 1) / G * 9 * G : (size_t)D.nx;
+        D.plane = b->blocked ? 0 : D.nx * D.ny;
+        D.e_off = e_cells;
+        D.e_row = b->blocked ? (D.nx + 1) / 2 * 2 : D.nx;
+        b->total += b->blocked ? D.row * D.ny : 9 * (size_t)D.plane;
+        e_cells += (size_t)D.e_row * D.ny;
+    }
     cudaError_t e;
     if ((e = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking)) != cudaSuccess ||
         (e = cudaMalloc(&b->buf[0], b->total * b->elem)) != cudaSuccess ||
@@ -642,6 +677,7 @@ extern "C" int imb_batch_autotune(imb_batch *b, int steps_per_trial, int *block,
     int bb = b->block, bc = b->cpl;
     for (int bl : blocks)
         for (int cp : cpls) {
+            if (cp == 2 && !b->blocked) continue;   // whole planes: one cell per lane either way
             b->block = bl;
             b->cpl = cp;
             b->grid = 0;
