@@ -5,6 +5,7 @@
 #include <cstddef>
 #include <cstdint>
 #include <cstring>
+#include <mutex>
 
 #ifdef __CUDACC__
 #define IMB_HD __host__ __device__ __forceinline__
@@ -29,6 +30,21 @@ inline bool spans_disjoint(const void *const *p, int n, size_t bytes) {
         }
     return true;
 }
+
+// What was asked once of every device (a kernel's attributes hold for the device they were set on), by
+// whichever thread comes first.
+template <typename T, int DEVICES = 64>
+class PerDevice {
+    std::once_flag once[DEVICES];
+    T value[DEVICES] = {};
+
+public:
+    template <typename F> T get(int device, F ask) {
+        if (device < 0 || device >= DEVICES) return ask();
+        std::call_once(once[device], [&] { value[device] = ask(); });
+        return value[device];
+    }
+};
 
 // Columns of a row to the blocks of the reverse step.  With the inlet and outlet columns transposed in the
 // same launch, column 0 must share a block with column 1 and column nx - 1 with column nx - 2.  Where the

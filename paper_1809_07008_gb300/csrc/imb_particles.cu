@@ -1537,10 +1537,13 @@ cudaError_t launch_dem_coupled(const DemArgs &d, int nblocks, cudaStream_t s) {
     return cudaLaunchCooperativeKernel((const void *)k_dem_coupled, dim3(nblocks), dim3(32), args, 0, s);
 }
 
-// Whether the device can hold the cluster (16 blocks are above the portable size of eight); asked
-// once, outside any capture.
+// Whether the current device can hold the cluster (16 blocks are above the portable size of eight);
+// asked once for a device, outside any capture, with the kernel's attributes set there.
 bool dem_cluster_fits() {
-    static const bool fits = [] {   // one device per process
+    static PerDevice<bool> fits;
+    int device = 0;
+    cudaGetDevice(&device);
+    return fits.get(device, [] {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(CL_CTAS);
         cfg.blockDim = dim3(CL_THREADS);
@@ -1559,8 +1562,7 @@ bool dem_cluster_fits() {
             cudaOccupancyMaxActiveClusters(&nc, k_dem_cluster, &cfg) == cudaSuccess && nc > 0;
         if (!ok) cudaGetLastError();
         return ok;
-    }();
-    return fits;
+    });
 }
 
 int dem_cluster_capacity() { return CL_P * CL_CTAS; }

@@ -17,7 +17,7 @@ def run_cpp(tmp_path, body):
     src, exe = tmp_path / "t.cpp", tmp_path / "t"
     src.write_text('#include "imb_host.h"\n#include <cstdio>\n#include <cstdlib>\nusing namespace imb;\n'
                    '#define CHECK(c) do { if (!(c)) { std::printf("failed: %s\\n", #c); std::exit(1); } } while (0)\n' + body)
-    subprocess.run([cxx, "-std=c++17", "-O2", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    subprocess.run([cxx, "-std=c++17", "-O2", "-pthread", "-I", CSRC, str(src), "-o", str(exe)], check=True)
     r = subprocess.run([str(exe)], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
 
@@ -118,5 +118,26 @@ int main() {
         if (nx >= 64 && 3.0 * 9 * padded * elem + 4.0 * padded + 72.0 * nx * ny < (double)mem - 1e8) CHECK(b);
         if (nx < 8) CHECK(!b);
     }
+}
+""")
+
+
+def test_asked_once_for_every_device(tmp_path):
+    # each device gets its own answer, asked once, whichever thread comes first
+    run_cpp(tmp_path, """
+#include <atomic>
+#include <thread>
+#include <vector>
+int main() {
+    static PerDevice<int, 4> v;
+    std::atomic<int> asked[6] = {};
+    std::vector<std::thread> t;
+    for (int k = 0; k < 16; ++k)
+        t.emplace_back([&] {
+            for (int d = 0; d < 6; ++d) CHECK(v.get(d, [&] { ++asked[d]; return 10 + d; }) == 10 + d);
+        });
+    for (auto &x : t) x.join();
+    for (int d = 0; d < 4; ++d) CHECK(asked[d] == 1);
+    CHECK(asked[4] == 16 && asked[5] == 16);   // beyond the table: asked every time
 }
 """)
