@@ -18,6 +18,7 @@
 #include <utility>
 
 #include "imb_device.cuh"
+#include "imb_host.h"
 #include "imb_kernels.h"
 #include "imb_pull.cuh"
 #include "imb_node.cuh"
@@ -604,7 +605,7 @@ k_stream_collide(const __grid_constant__ CUtensorMap tmap_n, const __grid_consta
             }
         }
         // hand the stage back: the last warp to finish with it, after the last unit of a tile,
-        // sums the tile's partials over the warps (FP64, fixed order) into the tile's force
+        // sums the tile's partials over the warps (fixed order, to FP64) into the tile's force
         // sums, then starts the copies of the unit NST ahead into the stage
         __syncwarp();
         int last = 0;
@@ -617,20 +618,12 @@ k_stream_collide(const __grid_constant__ CUtensorMap tmap_n, const __grid_consta
             if (SMALL || h == UPT - 1) {   // small lattices: the partials of each unit apart
                 double *tf = tile_force + ((size_t)ti.x * (SMALL ? UPT : 1) + (SMALL ? h : 0)) * (TILE_CAND * 3);
                 for (int i = lane; i < nc * 3; i += 32) {
-                    // the warps' sums in pairs of FP32 (the rounding of every add kept: 48 bits),
-                    // to FP64 at the end: eight FP64 adds and conversions in a row, 64 cycles each,
-                    // held back the copies of the next unit
+                    // the warps' sums (sum_terms: eight FP64 adds and conversions in a row, 64 cycles
+                    // each, held back the copies of the next unit)
                     float *pa = acc_t + i * WARPS;
-                    float hi = pa[0], lo = 0.0f;
-                    pa[0] = 0.0f;
+                    tf[i] = sum_terms<WARPS>(pa);
 #pragma unroll
-                    for (int w = 1; w < WARPS; ++w) {
-                        const float b = pa[w], t = __fadd_rn(hi, b), bb = __fsub_rn(t, hi);
-                        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, bb)), __fsub_rn(b, bb)));
-                        hi = t;
-                        pa[w] = 0.0f;
-                    }
-                    tf[i] = (double)hi + (double)lo;
+                    for (int w = 0; w < WARPS; ++w) pa[w] = 0.0f;
                 }
             }
             __syncwarp();

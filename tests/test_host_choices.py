@@ -141,3 +141,54 @@ int main() {
     CHECK(asked[4] == 16 && asked[5] == 16);   // beyond the table: asked every time
 }
 """)
+
+
+def test_sums_in_three_parts(tmp_path):
+    # eight FP32 terms of any exponents and signs, cancelling ones among them: no further from the exact sum
+    # than one FP64 rounding of it and 2^-68 of the terms; NaN, infinities and sums beyond FP32 as in FP64
+    run_cpp(tmp_path, """
+#include <random>
+#if defined(__x86_64__)
+typedef __float128 Quad;
+#else
+typedef long double Quad;   // 113 bits on Arm
+#endif
+static bool same(double a, double b) { return a == b || (a != a && b != b); }
+int main() {
+    std::mt19937_64 g(5);
+    auto term = [&](int spread) {
+        const float m = 1.0f + (float)(g() >> 41) * 0x1p-23f;
+        return std::ldexp(g() & 1 ? m : -m, (int)(g() % (2 * spread + 1)) - spread);
+    };
+    for (int spread : {0, 2, 8, 24, 40})
+        for (int k = 0; k < 1000000; ++k) {
+            float v[8];
+            for (float &x : v) x = term(spread);
+            if (k % 3 == 0) v[7] = -v[0], v[6] = -v[1];
+            if (k % 5 == 0) v[2] = 0.0f;
+            Quad exact = 0, size = 0;
+            Sum3 a, b;
+            for (int i = 0; i < 8; ++i) {
+                exact += v[i];
+                size += std::fabs(v[i]);
+                (i < 4 ? a : b).add(v[i]);
+            }
+            a.add(b);   // as lanes are joined
+            for (double got : {sum_terms<8>(v), a.value()}) {
+                Quad err = got - exact, bar = exact * 0x1.02p-53 + 0;
+                if (err < 0) err = -err;
+                if (bar < 0) bar = -bar;
+                CHECK(err <= bar + size * 0x1p-68);
+            }
+        }
+    const float inf = INFINITY, big = 3.0e38f;
+    const float cases[][8] = {{1, inf, 2, 3, 4, 5, 6, 7}, {1, -inf, 2, 3, 4, 5, 6, 7}, {inf, 0, 0, -inf, 0, 0, 0, 0},
+                              {1, NAN, 0, 0, 0, 0, 0, 0}, {big, big, big, 1, 0, 0, 0, 0}, {big, big, -big, -big, 5, 0, 0, 0},
+                              {inf, 0, 0, 0, 0, 0, 0, 0}, {0, 0, 0, 0, 0, 0, 0, 0}};
+    for (auto &c : cases) {
+        double d = 0.0;
+        for (float x : c) d += x;
+        CHECK(same(sum_terms<8>(c), d));
+    }
+}
+""")
