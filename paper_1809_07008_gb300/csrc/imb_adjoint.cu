@@ -46,13 +46,6 @@ __global__ void k_cell_E(const int *__restrict__ count, const float *__restrict_
     E[c] = e;
 }
 
-// a + b as a pair of FP32 (the rounding of the sum kept), added to the pair (hi, lo)
-__device__ __forceinline__ void pair_add(float &hi, float &lo, float b, float b_lo) {
-    const float t = __fadd_rn(hi, b), bb = __fsub_rn(t, hi);
-    lo = __fadd_rn(__fadd_rn(lo, b_lo), __fadd_rn(__fsub_rn(hi, __fsub_rn(t, bb)), __fsub_rn(b, bb)));
-    hi = t;
-}
-
 // sum of the nine directions, in the order of a butterfly over lanes
 __device__ __forceinline__ float tree9(const float (&v)[9]) {
     return (((v[0] + v[8]) + v[4]) + (v[2] + v[6])) + ((v[1] + v[5]) + (v[3] + v[7]));
@@ -65,8 +58,8 @@ __device__ __forceinline__ float tree9(const float (&v)[9]) {
 // and nx - 1 on to the threads of columns 1 and nx - 2, which hold the pulled f(t) they need, and
 // the row's d J / d u_in to g_uin (columns 0 and 1, and nx - 2 and nx - 1, share a block: adjoint_grid).
 //
-// d J / d tau is summed in pairs of FP32 over the block (an FP64 add takes a warp 64 cycles, and
-// every warp's shuffle tree took five of them).  The adjoint itself keeps the order of its sums:
+// d J / d tau is summed over a warp in three FP32 parts (Sum3: an FP64 add takes a warp 64 cycles, and
+// every warp's shuffle tree took five of them) and in FP64 from there on.  The adjoint itself keeps the order of its sums:
 // taken on opposite pairs it has fewer instructions and is no faster on 512 x 256 cells (42 us a
 // forward and reverse step, 84 before the launches and copies were saved), but where the adjoint front
 // has not reached the inlet d J / d u_in is rounding noise, which any other order changes whole.
@@ -77,10 +70,10 @@ __global__ void __launch_bounds__(ADJ_BLOCK) k_adjoint_step(const float *__restr
     cudaGridDependencySynchronize();   // launched as a dependent of the kernel before it
     cudaTriggerProgrammaticLaunchCompletion();
     __shared__ float edge[2][9];
-    __shared__ float2 part[8];
+    __shared__ double part[ADJ_BLOCK / 32];
     const int x = (int)(blockIdx.x * blockDim.x + threadIdx.x) - shift, y = blockIdx.y;
     const bool in = x >= 0 && x < a.nx;
-    float gt = 0.0f, gt_lo = 0.0f;
+    float gt = 0.0f, gt_B = 0.0f;   // the cell's d J / d tau, and through B
     lam1 += a.origin;   // node (0, 0) of plane 0 in the frame
     S0 += a.origin;
     lam0 += a.origin;
@@ -170,7 +163,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK) k_adjoint_step(const float *__restr
 #pragma unroll
             for (int q = 0; q < 9; ++q) lB += L[q] * (n[q] / tau + n[opp_of(q)] + w_of(q) * drho - d[q]);
             const float den = (1.0f - e) + tm;
-            pair_add(gt, gt_lo, lB * e * (1.0f - e) / (den * den), 0.0f);
+            gt_B = lB * e * (1.0f - e) / (den * den);
             if (Ec < 1.0f) gE[c] += (double)(lB * tm * (1.0f + tm) / (den * den));
         }
         if (inlet && (x == 1 || x == a.nx - 2)) {   // f(t) of the column, for the columns next to it
@@ -229,21 +222,30 @@ __global__ void __launch_bounds__(ADJ_BLOCK) k_adjoint_step(const float *__restr
 #pragma unroll
         for (int q = 0; q < 9; ++q) lam0[(size_t)q * a.plane + (size_t)y * a.pitch + x] = v[q];
     }
-    auto reduce = [&](int from) {
-        for (int o = from; o > 0; o >>= 1) {
-            const float h = __shfl_xor_sync(0xffffffffu, gt, o), l = __shfl_xor_sync(0xffffffffu, gt_lo, o);
-            pair_add(gt, gt_lo, h, l);
-        }
-    };
-    reduce(16);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = make_float2(gt, gt_lo);
+    Sum3 sum;
+    sum.add(gt);
+    sum.add(gt_B);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        Sum3 other;
+        other.hi = __shfl_xor_sync(0xffffffffu, sum.hi, o);
+        other.lo = __shfl_xor_sync(0xffffffffu, sum.lo, o);
+        other.lo2 = __shfl_xor_sync(0xffffffffu, sum.lo2, o);
+        sum.add(other);
+    }
+    double t = sum.value();
+    if (__any_sync(0xffffffffu, !sum.finite())) {   // a sum beyond FP32, an infinity or NaN
+        t = (double)gt + (double)gt_B;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    }
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = t;
     __syncthreads();
     if (threadIdx.x < 32) {
-        const float2 p = threadIdx.x < (blockDim.x >> 5) ? part[threadIdx.x] : make_float2(0.0f, 0.0f);
-        gt = p.x;
-        gt_lo = p.y;
-        reduce(4);   // at most eight warps
-        if (threadIdx.x == 0 && (gt != 0.0f || gt_lo != 0.0f)) atomicAdd(g_tau, (double)gt + (double)gt_lo);
+        t = threadIdx.x < ADJ_BLOCK / 32 ? part[threadIdx.x] : 0.0;
+#pragma unroll
+        for (int o = ADJ_BLOCK / 64; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (threadIdx.x == 0 && t != 0.0) atomicAdd(g_tau, t);
     }
 }
 

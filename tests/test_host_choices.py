@@ -192,3 +192,44 @@ int main() {
     }
 }
 """)
+
+
+def test_sums_joined_over_a_warp(tmp_path):
+    # 32 lanes of two terms each, joined over a butterfly as the reverse step does: every lane ends with the
+    # exact sum to one FP64 rounding and 2^-66 of the terms (FP64 additions: 2^-53 a level; a pair of FP32
+    # parts is 2^-46 off and fails)
+    run_cpp(tmp_path, """
+#include <random>
+#if defined(__x86_64__)
+typedef __float128 Quad;
+#else
+typedef long double Quad;
+#endif
+int main() {
+    std::mt19937_64 g(7);
+    for (int spread : {0, 3, 12, 30})
+        for (int k = 0; k < 20000; ++k) {
+            Sum3 s[32];
+            Quad exact = 0, size = 0;
+            for (auto &lane : s)
+                for (int i = 0; i < 2; ++i) {
+                    const float m = 1.0f + (float)(g() >> 41) * 0x1p-23f;
+                    const float x = std::ldexp(g() & 1 ? m : -m, (int)(g() % (2 * spread + 1)) - spread);
+                    lane.add(x);
+                    exact += x;
+                    size += std::fabs(x);
+                }
+            for (int o = 16; o > 0; o >>= 1) {
+                Sum3 n[32];
+                for (int l = 0; l < 32; ++l) n[l] = s[l], n[l].add(s[l ^ o]);
+                for (int l = 0; l < 32; ++l) s[l] = n[l];
+            }
+            for (auto &lane : s) {
+                Quad err = lane.value() - exact, bar = exact * 0x1.02p-53;
+                if (err < 0) err = -err;
+                if (bar < 0) bar = -bar;
+                CHECK(lane.finite() && err <= bar + size * 0x1p-66);
+            }
+        }
+}
+""")
