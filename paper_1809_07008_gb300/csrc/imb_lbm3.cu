@@ -207,30 +207,49 @@ __device__ __forceinline__ void fetch3(const S *__restrict__ fin, const Args3 &a
 // not once per cell: two slots, a third sphere in one column is added to its totals at once.
 // In a packed bed half the cells are covered, and a shuffle tree with FP64 atomics at every
 // covered warp-row put about 2.5 M atomics a step on 1500 addresses, which set the time: the
-// 240 x 100 x 100 bed's pass of 60 steps went from 18.4 to 12.2 ms.  The sums stay FP32 over the
-// column and the warp (256 terms at most) and FP64 beyond; their error against 64 bits is the
-// same (2.3e-6 of the outputs, set by the terms).  Registers are full at two blocks an SM, hence
-// shared memory.
+// 240 x 100 x 100 bed's pass of 60 steps went from 18.4 to 12.2 ms.  The sums over the column and the
+// warp (256 FP32 terms at most) are pairs of FP32 parts, what the first part rounds off kept in the second
+// (two_sum): no bits are lost where the terms went to FP64 one by one before, nor in the tree.  What
+// leaves the range of FP32 goes out in FP64.
+// Registers are full at two blocks an SM, hence shared memory.
 constexpr int FSLOTS = 2;
 struct ForceSums {
     int id[FSLOTS][256];
-    float v[FSLOTS][6][256];
+    float v[FSLOTS][6][256], lo[FSLOTS][6][256];
 };
+__device__ __forceinline__ float2 pair_sum(float2 a, float2 b) {
+    float e;
+    const float s = imb::two_sum(a.x, b.x, e);
+    return make_float2(s, (a.y + b.y) + e);
+}
 
 __device__ __forceinline__ void add_force3(ForceSums &sm, double *FT, const int sid, const float (&fo)[6]) {
     const int t = threadIdx.y * 32 + threadIdx.x;
+    float s[6], e[6], m = 0.0f;
 #pragma unroll
     for (int k = 0; k < FSLOTS; ++k) {
         const int id = sm.id[k][t];
         if (id == sid) {
 #pragma unroll
-            for (int c = 0; c < 6; ++c) sm.v[k][c][t] += fo[c];
+            for (int c = 0; c < 6; ++c) {
+                s[c] = imb::two_sum(sm.v[k][c][t], fo[c], e[c]);
+                m = fmaxf(m, fabsf(s[c]));
+            }
+            if (m == INFINITY) break;
+#pragma unroll
+            for (int c = 0; c < 6; ++c) {
+                sm.v[k][c][t] = s[c];
+                sm.lo[k][c][t] += e[c];
+            }
             return;
         }
         if (id < 0) {
             sm.id[k][t] = sid;
 #pragma unroll
-            for (int c = 0; c < 6; ++c) sm.v[k][c][t] = fo[c];
+            for (int c = 0; c < 6; ++c) {
+                sm.v[k][c][t] = fo[c];
+                sm.lo[k][c][t] = 0.0f;
+            }
             return;
         }
     }
@@ -257,27 +276,38 @@ __device__ __forceinline__ void flush_forces3(ForceSums &sm, double *FT) {
                 if (has) lead = __shfl_sync(FULL, id[k], __ffs(has) - 1);
             }
         if (!has) return;
-        float v[8];
+        float2 v[8];
+        int slot = -1;
 #pragma unroll
-        for (int c = 0; c < 8; ++c) v[c] = 0.0f;
+        for (int c = 0; c < 8; ++c) v[c] = make_float2(0.0f, 0.0f);
 #pragma unroll
         for (int k = 0; k < FSLOTS; ++k)
             if (id[k] == lead) {   // a sphere takes one slot of a thread
 #pragma unroll
-                for (int c = 0; c < 6; ++c) v[c] = sm.v[k][c][t];
+                for (int c = 0; c < 6; ++c) v[c] = make_float2(sm.v[k][c][t], sm.lo[k][c][t]);
                 id[k] = -1;
+                slot = k;
             }
+        auto with_lane = [&](float2 keep, float2 give, int o) {
+            return pair_sum(keep, make_float2(__shfl_xor_sync(FULL, give.x, o), __shfl_xor_sync(FULL, give.y, o)));
+        };
         const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
-        float w4[4], w2[2];
+        float2 w4[4], w2[2];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) w4[j] = (h4 ? v[j + 4] : v[j]) + __shfl_xor_sync(FULL, h4 ? v[j] : v[j + 4], 16);
+        for (int j = 0; j < 4; ++j) w4[j] = with_lane(h4 ? v[j + 4] : v[j], h4 ? v[j] : v[j + 4], 16);
 #pragma unroll
-        for (int j = 0; j < 2; ++j) w2[j] = (h3 ? w4[j + 2] : w4[j]) + __shfl_xor_sync(FULL, h3 ? w4[j] : w4[j + 2], 8);
-        float r = (h2 ? w2[1] : w2[0]) + __shfl_xor_sync(FULL, h2 ? w2[0] : w2[1], 4);
-        r += __shfl_xor_sync(FULL, r, 2);
-        r += __shfl_xor_sync(FULL, r, 1);
+        for (int j = 0; j < 2; ++j) w2[j] = with_lane(h3 ? w4[j + 2] : w4[j], h3 ? w4[j] : w4[j + 2], 8);
+        float2 r = with_lane(h2 ? w2[1] : w2[0], h2 ? w2[0] : w2[1], 4);
+        r = with_lane(r, r, 2);
+        r = with_lane(r, r, 1);
+        if (__any_sync(FULL, !(r.x - r.x == 0.0f))) {   // beyond FP32, an infinity or NaN: lane by lane
+            if (slot >= 0)
+                for (int c = 0; c < 6; ++c)
+                    atomicAdd(&FT[6 * lead + c], (double)sm.v[slot][c][t] + (double)sm.lo[slot][c][t]);
+            continue;
+        }
         const int c = lane >> 2;   // lanes 4 c .. 4 c + 3 hold the sum of component c
-        if ((lane & 3) == 0 && c < 6) atomicAdd(&FT[6 * lead + c], (double)r);
+        if ((lane & 3) == 0 && c < 6) atomicAdd(&FT[6 * lead + c], (double)r.x + (double)r.y);
     }
 }
 
