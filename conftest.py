@@ -1,4 +1,4 @@
-"""Lattices kept alive by a caught exception's traceback are released between tests.
+"""The lattices of earlier tests are released before the test that bounds a host wait.
 
 A test that catches an ImbError leaves its lattice in a reference cycle (exception, traceback, frame).
 Collected in the middle of a later test, its release frees device memory, which waits for the GPU:
@@ -8,4 +8,5 @@ import gc
 
 
 def pytest_runtest_setup(item):
-    gc.collect()
+    if item.name.startswith("test_host_wait_is_bounded"):
+        gc.collect()
