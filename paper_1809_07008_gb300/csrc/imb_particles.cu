@@ -1060,7 +1060,12 @@ __device__ __forceinline__ void warp_islands(const DemArgs &d, WarpIslands &w, c
 // one-warp blocks that went through L2 with a spinning barrier and evaluated each particle's
 // candidates one after another took 12 us a sub-cycle on 1000 stacked disks; this takes 4.2 us
 // (a coupling cycle of the 2048 x 1024 collapse, 100 sub-cycles: 1.37 -> 0.56 ms).
-constexpr int CL_CTAS = 16, CL_THREADS = 256, CL_P = 256, CL_Q = 1280;
+// The contact table takes what shared memory is left: ten contacts a particle.  A block with more
+// (sixteen candidates each and two walls, which the skin must be tens of cells wide for) sends the whole
+// cluster to the particles' candidates one after another, which is slower than the grid: with a table
+// of five contacts a particle 3600 disks of twelve candidates took 31 us a sub-cycle so, the grid
+// 24 us, this 13 us.  Slabs of 2000 and 4096 disks take 7.7 and 10.5 us (the grid 15.6 and 16.4).
+constexpr int CL_CTAS = 16, CL_THREADS = 256, CL_P = 256, CL_Q = 2560;
 
 struct ClusterDem {
     double st[2][5][CL_P];               // x, y, vx, vy, w
