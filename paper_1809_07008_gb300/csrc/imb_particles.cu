@@ -245,15 +245,19 @@ __device__ __forceinline__ void contact_law(const DemArgs &d, double nxv, double
 
 // Force on particle p of its candidate q in slot j (seen from p), with the pair's tangential
 // spring xi; the pair's damping constant is cached in the neighbour list.  Returns false (and
-// releases the spring) without overlap.
+// releases the spring) without overlap.  WORDS: the minimum image by nearest(), for callers whose
+// lanes nearly all go on to the force.  Where most candidates end at the overlap test its branches
+// cost more than min_image's compares, which an axis without periodic edges skips (k_dem_coupled on slabs of
+// 4097 and 8000 disks: 17.1 and 30.7 us a sub-cycle with nearest(), 16.5 and 29.7 with min_image).
+template <bool WORDS>
 __device__ __forceinline__ bool pair_force_xi(const DemArgs &d, const int p, const int j, const int q, double &xi,
                                               const double px, const double py, const double w, const double qx,
                                               const double qy, const double qvx, const double qvy, const double qw,
                                               const double vx, const double vy, double &fx, double &fy,
                                               double &Ft) {
     const double rp = d.r[p];
-    const double dx = nearest(qx - px, d.half_x, d.Lx);
-    const double dy = nearest(qy - py, d.half_y, d.Ly);
+    const double dx = WORDS ? nearest(qx - px, d.half_x, d.Lx) : min_image(qx - px, d.bc_x == BC_PERIODIC, d.nx);
+    const double dy = WORDS ? nearest(qy - py, d.half_y, d.Ly) : min_image(qy - py, d.bc_y == BC_PERIODIC, d.ny);
     const double d2 = dx * dx + dy * dy;
     const double R = rp + d.r[q];
     if (!(d2 < R * R)) {  // Eq. 7: no overlap, the spring is released
@@ -279,7 +283,7 @@ __device__ __forceinline__ bool pair_force(const DemArgs &d, const int p, const 
                                            const double qvx, const double qvy, const double qw,
                                            const double vx, const double vy, double &fx, double &fy,
                                            double &Ft) {
-    return pair_force_xi(d, p, j, d.nbr_id[p * MAX_NBR + j], d.nbr_xi[p * MAX_NBR + j], px, py, w, qx, qy, qvx,
+    return pair_force_xi<false>(d, p, j, d.nbr_id[p * MAX_NBR + j], d.nbr_xi[p * MAX_NBR + j], px, py, w, qx, qy, qvx,
                          qvy, qw, vx, vy, fx, fy, Ft);
 }
 
@@ -950,7 +954,7 @@ __device__ __forceinline__ void warp_islands(const DemArgs &d, WarpIslands &w, c
                 }
                 if (hit) {
                     double xi = w.xi[k], fx, fy, Ft;
-                    pair_force_xi(d, w.id[i], w.pj[k], w.id[l], xi, st[0][i], st[1][i], st[4][i], st[0][l], st[1][l],
+                    pair_force_xi<true>(d, w.id[i], w.pj[k], w.id[l], xi, st[0][i], st[1][i], st[4][i], st[0][l], st[1][l],
                                   st[2][l], st[3][l], st[4][l], st[2][i], st[3][i], fx, fy, Ft);
                     w.xi[k] = xi;
                     w.f[0][k] = fx;
