@@ -1044,12 +1044,22 @@ static bool one_wave(int storage, const LatticeArgs &a) {
     return a.tf_units == SMALL_UPT || a.nbx * a.nby <= stream_collide_resident_blocks(storage);
 }
 
+// Whether k_step_tail is.  Not where tiles outnumber the SMs in FP32 and no inlet or outlet column
+// keeps some of them longer: its blocks then take their places beside stream-collide blocks that are
+// still to finish their tiles (us a step, dependent / not: 400 x 400 fluid 14.4 / 11.8, 512 x 512 14.7 /
+// 12.1, 600 x 600 13.1 / 12.9; with inlet and outlet 17.3 / 17.8 and 17.9 / 18.3; 380 x 380 10.8 /
+// 11.3; FP16 10.3 / 10.4 and 10.8 / 10.8; many disks 14.7 / 14.7 and 15.2 / 15.5).
+template <typename S>
+static bool tail_early(int storage, const LatticeArgs &a) {
+    return one_wave(storage, a) && !(sizeof(S) == 4 && a.bc_x != BC_INLET_OUTLET && a.nbx * a.nby > device_sms());
+}
+
 static cudaError_t step_tail(void *f, int storage, const LatticeArgs &a, const double *tile_force, int nbf,
                              cudaStream_t s) {
     return by_storage(storage, [&](auto tag) {
         using S = std::remove_pointer_t<decltype(tag)>;
         const int nbg = (edge_nodes(a.nx, a.ny) + 255) / 256;
-        return launch_dependent(k_step_tail<S>, nbf + nbg, 256, 0, s, one_wave(storage, a), a, tile_force, (S *)f, nbf);
+        return launch_dependent(k_step_tail<S>, nbf + nbg, 256, 0, s, tail_early<S>(storage, a), a, tile_force, (S *)f, nbf);
     });
 }
 
