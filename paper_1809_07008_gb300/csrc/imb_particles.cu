@@ -1443,10 +1443,10 @@ __device__ __forceinline__ void dem_islands(const DemArgs &d, const int blk, con
     }
 }
 
-// The particles of one coupling cycle that need no grid barrier -- free particles, islands
-// of up to four, islands of five to 32 -- in one launch: the roles take consecutive block
-// ranges in that order and run side by side (the three sets of particles are disjoint), so
-// an island's chain of N_sub sub-cycles, bound by the latency of its FP64 instructions,
+// The particles of one coupling cycle that need no grid barrier -- islands of up to four, islands of
+// five to 32, free particles -- in one launch: the roles take consecutive block ranges in that
+// order (the longest chains start first) and run side by side (the three sets of particles are
+// disjoint), so an island's chain of N_sub sub-cycles, bound by the latency of its FP64 instructions,
 // overlaps the free particles' FP64 throughput and the other islands' chains.
 
 __global__ void __launch_bounds__(LOCAL_THREADS) k_dem_local(const DemArgs d, int nb_islands, int nb_small) {
