@@ -58,9 +58,11 @@ __device__ __forceinline__ float tree9(const float (&v)[9]) {
 // and nx - 1 on to the threads of columns 1 and nx - 2, which hold the pulled f(t) they need, and
 // the row's d J / d u_in to g_uin (columns 0 and 1, and nx - 2 and nx - 1, share a block: adjoint_grid).
 //
-// d J / d tau is summed over a warp in three FP32 parts (Sum3: an FP64 add takes a warp 64 cycles, and
-// every warp's shuffle tree took five of them) and in FP64 from there on.  The adjoint itself keeps the order of its sums:
-// taken on opposite pairs it has fewer instructions and is no faster on 512 x 256 cells (42 us a
+// d J / d tau is summed over the block in three FP32 parts (Sum3: an FP64 add takes a warp 64 cycles, and
+// every warp's shuffle tree took five of them; even the three conversions at the end of each warp's sum
+// kept the FP64 pipe busy for 29 % of the launch on 2048 x 1024 cells, 71 us against 67).  What leaves
+// FP32's range is summed in FP64.  The adjoint itself keeps the order of its sums:
+// taken on opposite pairs it has fewer instructions and is no faster on 512 x 256 cells (43 us a
 // forward and reverse step, 84 before the launches and copies were saved), but where the adjoint front
 // has not reached the inlet d J / d u_in is rounding noise, which any other order changes whole.
 __global__ void __launch_bounds__(ADJ_BLOCK) k_adjoint_step(const float *__restrict__ lam1, const float *__restrict__ S0,
@@ -70,7 +72,8 @@ __global__ void __launch_bounds__(ADJ_BLOCK) k_adjoint_step(const float *__restr
     cudaGridDependencySynchronize();   // launched as a dependent of the kernel before it
     cudaTriggerProgrammaticLaunchCompletion();
     __shared__ float edge[2][9];
-    __shared__ double part[ADJ_BLOCK / 32];
+    __shared__ float part[3][ADJ_BLOCK / 32];
+    __shared__ double part64[ADJ_BLOCK / 32];
     const int x = (int)(blockIdx.x * blockDim.x + threadIdx.x) - shift, y = blockIdx.y;
     const bool in = x >= 0 && x < a.nx;
     float gt = 0.0f, gt_B = 0.0f;   // the cell's d J / d tau, and through B
@@ -225,27 +228,50 @@ __global__ void __launch_bounds__(ADJ_BLOCK) k_adjoint_step(const float *__restr
     Sum3 sum;
     sum.add(gt);
     sum.add(gt_B);
+    auto join = [&](int from) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        Sum3 other;
-        other.hi = __shfl_xor_sync(0xffffffffu, sum.hi, o);
-        other.lo = __shfl_xor_sync(0xffffffffu, sum.lo, o);
-        other.lo2 = __shfl_xor_sync(0xffffffffu, sum.lo2, o);
-        sum.add(other);
-    }
-    double t = sum.value();
+        for (int o = from; o > 0; o >>= 1) {
+            Sum3 other;
+            other.hi = __shfl_xor_sync(0xffffffffu, sum.hi, o);
+            other.lo = __shfl_xor_sync(0xffffffffu, sum.lo, o);
+            other.lo2 = __shfl_xor_sync(0xffffffffu, sum.lo2, o);
+            sum.add(other);
+        }
+    };
+    join(16);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (__any_sync(0xffffffffu, !sum.finite())) {   // a sum beyond FP32, an infinity or NaN
-        t = (double)gt + (double)gt_B;
-#pragma unroll
+        double t = (double)gt + (double)gt_B;
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) part64[warp] = t;
     }
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = t;
+    if (lane == 0) {
+        part[0][warp] = sum.hi;
+        part[1][warp] = sum.lo;
+        part[2][warp] = sum.lo2;
+    }
     __syncthreads();
     if (threadIdx.x < 32) {
-        t = threadIdx.x < ADJ_BLOCK / 32 ? part[threadIdx.x] : 0.0;
-#pragma unroll
-        for (int o = ADJ_BLOCK / 64; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (threadIdx.x == 0 && t != 0.0) atomicAdd(g_tau, t);
+        constexpr int WARPS = ADJ_BLOCK / 32;
+        auto of_warp = [&](int w) {
+            Sum3 p;
+            if (w < WARPS) {
+                p.hi = part[0][w];
+                p.lo = part[1][w];
+                p.lo2 = part[2][w];
+            }
+            return p;
+        };
+        sum = of_warp(lane);
+        join(WARPS / 2);
+        if (lane == 0 && !(sum.hi == 0.0f && sum.lo == 0.0f)) {
+            double t = sum.value();
+            if (!sum.finite()) {
+                t = 0.0;
+                for (int w = 0; w < WARPS; ++w) t += of_warp(w).finite() ? of_warp(w).value() : part64[w];
+            }
+            atomicAdd(g_tau, t);
+        }
     }
 }
 

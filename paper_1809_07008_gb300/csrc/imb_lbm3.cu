@@ -209,8 +209,8 @@ __device__ __forceinline__ void fetch3(const S *__restrict__ fin, const Args3 &a
 // covered warp-row put about 2.5 M atomics a step on 1500 addresses, which set the time: the
 // 240 x 100 x 100 bed's pass of 60 steps went from 18.4 to 12.2 ms.  The sums over the column and the
 // warp (256 FP32 terms at most) are pairs of FP32 parts, what the first part rounds off kept in the second
-// (two_sum): no bits are lost where the terms went to FP64 one by one before, nor in the tree.  What
-// leaves the range of FP32 goes out in FP64.
+// (two_sum): no bits are lost where the terms went to FP64 one by one before, nor in the tree (plain FP32
+// sums ran the bed's pass in 8.5 ms, these in 9.0).  What leaves the range of FP32 goes out in FP64.
 // Registers are full at two blocks an SM, hence shared memory.
 constexpr int FSLOTS = 2;
 struct ForceSums {
@@ -346,8 +346,8 @@ __device__ __forceinline__ void sphere_force(float Bp, float rho, float jx, floa
 // The order of the sums and products of Eqs. 2 and 13 is kept as it was: with bfloat16 populations any
 // other rounding moves weak transverse flows by 1 % within 50 steps (the forcing put into the
 // equilibrium, and Pi from second moments, would save another 5 %).
-// Kernel time on 16 M cells with one sphere 506 -> 453 us FP32 (5.4 TB/s), 446 -> 355 us FP16; the
-// 240 x 100 x 100 packed bed (GEN) with the column sums 269 -> 119 us.
+// Kernel time on 16 M cells with one sphere 506 -> 459 us FP32 (5.3 TB/s), 446 -> 354 us FP16; the
+// 240 x 100 x 100 packed bed (GEN) with the column sums 269 -> 128 us.
 template <bool GEN, typename S>
 __device__ __forceinline__ int collide3(const float (&d)[19], const Args3 &a, int x, int y, int z, size_t cell,
                                         const unsigned word, const unsigned *__restrict__ map2,

@@ -1062,7 +1062,7 @@ __device__ __forceinline__ void warp_islands(const DemArgs &d, WarpIslands &w, c
 // What bounds it: the FP64 pipe takes 64 cycles per warp instruction whatever its mask, so the
 // time is the longest chain of instructions of the three rounds plus the barrier.  The grid of
 // one-warp blocks that went through L2 with a spinning barrier and evaluated each particle's
-// candidates one after another took 12 us a sub-cycle on 1000 stacked disks; this takes 4.2 us
+// candidates one after another took 12 us a sub-cycle on 1000 stacked disks; this takes 4.3 us
 // (a coupling cycle of the 2048 x 1024 collapse, 100 sub-cycles: 1.37 -> 0.56 ms).
 // The contact table takes what shared memory is left: ten contacts a particle.  A block with more
 // (sixteen candidates each and two walls, which the skin must be tens of cells wide for) sends the whole
