@@ -209,6 +209,7 @@ static DemArgs dem_args(imb_ctx *c) {
         if (periodic) std::memcpy(&b, &h, sizeof(b));
         return b;
     };
+    d.cluster_max = cluster_limit(c->p.N_sub);
     d.half_x = half(c->p.bc_x == IMB_BC_PERIODIC, d.Lx);
     d.half_y = half(c->p.bc_y == IMB_BC_PERIODIC, d.Ly);
     d.N_sub = c->p.N_sub;
@@ -696,7 +697,7 @@ static int dem_cycle(imb_ctx *c, bool zero_forces) {
             CK(launch_dem_cluster(d, c->stream), "dem cluster");
             c->launches++;
         }
-        if (!cluster || c->np > dem_cluster_capacity()) {
+        if (!cluster || c->np > d.cluster_max) {
             CK(launch_dem_coupled(d, dem_coupled_blocks(), c->stream), "dem coupled");
             c->launches++;
         }

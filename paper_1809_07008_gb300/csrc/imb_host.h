@@ -59,6 +59,15 @@ inline AdjointGrid adjoint_grid(int nx, bool inlet) {
     return {(nx + shift + ADJ_BLOCK - 1) / ADJ_BLOCK, shift};
 }
 
+// Particles of large islands that the DEM's cluster takes: what its blocks hold, and fewer where a cycle has
+// few sub-cycles.  Placing the particles (the ranks of the Morton order, the pairs across
+// blocks) grows faster than their number, 60 us with 4096, and the sub-cycles must win that back.  Cycles of
+// slabs of 1000, 2000 and 4096 disks, cluster / grid: one sub-cycle 128 / 129, 147 / 134 and 217 / 170 us,
+// two 133 / 146, 156 / 154 and 232 / 194, five 150 / 207, 189 / 218 and 283 / 249, ten 182 / 310, 235 /
+// 322 and 362 / 349, twenty 239 / 515, 333 / 525 and 535 / 556.
+constexpr int CLUSTER_PARTICLES = 4096;
+inline int cluster_limit(int N_sub) { return N_sub < 12 ? 1000 + 300 * (N_sub - 1) : CLUSTER_PARTICLES; }
+
 // Whether a batch holds its populations in rows padded to whole blocks (`padded` cells of `elem` bytes
 // with the padding) or in whole planes without any (`cells`).
 //

@@ -85,6 +85,7 @@ struct DemArgs {
     double dt, kn, kt, zeta, ct_ratio, mu, gx_eff, gy_eff, skin;
     double Lx, Ly;              // nx, ny
     long long half_x, half_y;   // bits of L / 2 on a periodic axis, else the largest integer
+    int cluster_max;            // particles of large islands that k_dem_cluster takes (cluster_limit)
     int model;                  // 0 linear spring-dashpot, 1 simplified Hertz-Mindlin
     double hm_kn0, hm_sn0, hm_kt0, hm_c0;   // 4/3 E*, 2 E*, 8 G*, 2 sqrt(5/6) |beta|
     double *x, *v, *w;          // primary state [2np], [2np], [np]
@@ -168,7 +169,6 @@ cudaError_t launch_bin_fill(const int *pbin, int np, int *bin_fill, const int *b
 cudaError_t launch_dem_neighbours(const DemArgs &d, cudaStream_t s);
 // islands of more than 32 particles: one cluster, then what it doesn't hold by the whole grid
 bool dem_cluster_fits();
-int dem_cluster_capacity();   // particles of large islands the cluster holds
 cudaError_t launch_dem_cluster(const DemArgs &d, cudaStream_t s);
 cudaError_t launch_dem_coupled(const DemArgs &d, int nblocks, cudaStream_t s);
 cudaError_t launch_dem_islands_setup(const DemArgs &d, cudaStream_t s);

@@ -1070,6 +1070,7 @@ __device__ __forceinline__ void warp_islands(const DemArgs &d, WarpIslands &w, c
 // of five contacts a particle 3600 disks of twelve candidates took 31 us a sub-cycle so, the grid
 // 24 us, this 13 us.  Slabs of 2000 and 4096 disks take 7.7 and 10.5 us (the grid 15.6 and 16.4).
 constexpr int CL_CTAS = 16, CL_THREADS = 256, CL_P = 256, CL_Q = 2560;
+static_assert(CL_P * CL_CTAS == CLUSTER_PARTICLES, "what the cluster's blocks hold together");
 
 struct ClusterDem {
     double st[2][5][CL_P];               // x, y, vx, vy, w
@@ -1136,7 +1137,7 @@ __global__ void __launch_bounds__(CL_THREADS) k_dem_cluster(const DemArgs d) {
     extern __shared__ __align__(16) unsigned char cl_smem[];
     ClusterDem &S = *reinterpret_cast<ClusterDem *>(cl_smem);
     const int n = d.counters[3];
-    if (n == 0 || n > CL_P * CL_CTAS) return;   // every block alike; a larger set: k_dem_coupled
+    if (n == 0 || n > d.cluster_max) return;   // every block alike; a larger set: k_dem_coupled
     const int tid = threadIdx.x, cta = blockIdx.x;
     // the particles' places: rank by Morton order, block by block
     unsigned long long *keys = reinterpret_cast<unsigned long long *>(cl_smem);
@@ -1573,8 +1574,6 @@ bool dem_cluster_fits() {
         return ok;
     });
 }
-
-int dem_cluster_capacity() { return CL_P * CL_CTAS; }
 
 cudaError_t launch_dem_cluster(const DemArgs &d, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};

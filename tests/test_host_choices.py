@@ -233,3 +233,13 @@ int main() {
         }
 }
 """)
+
+
+def test_cluster_limit(tmp_path):
+    # never beyond what the cluster holds, never less with more sub-cycles, all of it from twelve on
+    run_cpp(tmp_path, """
+int main() {
+    CHECK(cluster_limit(1) == 1000 && cluster_limit(12) == CLUSTER_PARTICLES && cluster_limit(1 << 20) == CLUSTER_PARTICLES);
+    for (int n = 1; n < 1000; ++n) CHECK(cluster_limit(n) <= cluster_limit(n + 1) && cluster_limit(n) <= CLUSTER_PARTICLES);
+}
+""")
