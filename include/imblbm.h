@@ -237,7 +237,8 @@ int imb_binomial_schedule(int T, int snapshots, int *ops, int max_ops, int *n_op
  * disks of domain 0 first, then those of domain 1, and so on.  Populations are
  * stored as f - w in `storage` (IMB_STORE_*), two copies of 9 values a cell with rows padded
  * to 32 (FP32) or 64 cells, without padding where the domains are narrow (a mean width
- * below 64, with 16 bits 31, in small batches 8 cells) or memory is short.  Every step advances all domains
+ * below 31, in small batches 8 cells; FP32 rows no multiple of 16 long below 100) or memory is
+ * short.  Every step advances all domains
  * with the collision of Eq. 13 (B of Eq. 14 from the summed exact overlap area of
  * each cell, u_s = 0) and adds each domain's drag (Eq. 15, summed over its disks)
  * to an accumulator.  The library owns the batch; host arrays are copied.

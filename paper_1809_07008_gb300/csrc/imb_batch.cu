@@ -516,7 +516,7 @@ extern "C" int imb_batch_create(imb_batch **out, int n_domains, const int *nx, c
     b->elem = storage == IMB_STORE_FP32 ? 4 : 2;
     b->ndom = n_domains;
     double rmax = 0.0;
-    size_t cells = 0, rows = 0, e_cells = 0, most = 0, padded = 0;
+    size_t cells = 0, rows = 0, ragged = 0, e_cells = 0, most = 0, padded = 0;
     long long items = 0, items2 = 0;   // work items of 32 and of 64 cells
     const size_t G = storage == IMB_STORE_FP32 ? segb<float>() : segb<__half>();
     int ndisk = 0;
@@ -539,6 +539,7 @@ extern "C" int imb_batch_create(imb_batch **out, int n_domains, const int *nx, c
         b->hdom.push_back(D);
         cells += (size_t)nx[d] * ny[d];
         rows += (size_t)ny[d];
+        if (nx[d] % 16) ragged += (size_t)ny[d];
         most = std::max(most, (size_t)nx[d] * ny[d]);
         padded += (nx[d] + G - 1) / G * G * ny[d];
         items += ((long long)ny[d] * nx[d] + 31) / 32;
@@ -572,7 +573,7 @@ extern "C" int imb_batch_create(imb_batch **out, int n_domains, const int *nx, c
     cudaGetDevice(&b->device);
     size_t mem_free = 0, mem_total = 0;
     if (cudaMemGetInfo(&mem_free, &mem_total) != cudaSuccess) cudaGetLastError();
-    b->blocked = blocked_rows(cells, rows, padded, most, (size_t)b->elem, mem_free);
+    b->blocked = blocked_rows(cells, rows, ragged, padded, most, (size_t)b->elem, mem_free);
     for (BatchDomain &D : b->hdom) {
         D.off = b->total;
         D.row = b->blocked ? (D.nx + G - 1) / G * 9 * G : (size_t)D.nx;

@@ -69,7 +69,8 @@ constexpr int CLUSTER_PARTICLES = 4096;
 inline int cluster_limit(int N_sub) { return N_sub < 12 ? 1000 + 300 * (N_sub - 1) : CLUSTER_PARTICLES; }
 
 // Whether a batch holds its populations in rows padded to whole blocks (`padded` cells of `elem` bytes
-// with the padding) or in whole planes without any (`cells`).
+// with the padding) or in whole planes without any (`cells`).  `ragged` of its `rows` are no multiple of 16
+// cells long.
 //
 // By speed: a blocked row ends in a part of a 32-byte sector that nothing else completes, and a narrow
 // row is mostly padding, so planes win on narrow rows; blocked rows need fewer instructions a cell, so
@@ -77,20 +78,22 @@ inline int cluster_limit(int N_sub) { return N_sub < 12 ? 1000 + 300 * (N_sub - 
 // blocked / planes, rows of 160 or 120 cells: 6 M cells FP32, width 3: 108 / 18, 33: 23 / 16, 50: 20 / 16, 65:
 // 19 / 16, 160: 14 / 15, 257: 15 / 15; FP16, 24: 23 / 15, 31: 12 / 15, 33: 18 / 15, 50: 13 / 15, 257: 11 /
 // 15; 0.3 M cells (22 MB) FP32, width 3: 123 / 38, 11: 32 / 34, 50: 28 / 32, 450: 23 / 31; 1.5 M cells FP16 (54
-// MB), 24: 29 / 17, 45: 13 / 17.  (FP32 rows of 65 to 250 cells in large batches would be up to 15 % faster in
-// planes where nx is no multiple of 8; the line is where blocked rows stop being the slower of the
-// two layouts the sweeps have had, so that no width is slower than with row segments of planes.)
+// MB), 24: 29 / 17, 45: 13 / 17.  (Ragged FP32 rows of 100 to 250 cells in large batches would be up to 10 % faster in
+// planes; the line is where blocked rows stop being the slower of the two layouts the sweeps have had, so
+// that no width is slower than with row segments of planes: 4 M cells in rows of 90, 70.8 us a step blocked, 68.6
+// in segments, 67.8 in planes; in rows of 64 60.5, 60.6 and 64.8.)
 //
 // By memory: the padding must not cost a call that planes leave room for: two buffers and one domain of
 // `most` cells read back as FP64, or three while the launch shapes are timed, with the solid ratios.
-inline bool blocked_rows(size_t cells, size_t rows, size_t padded, size_t most, size_t elem, size_t mem_free) {
+inline bool blocked_rows(size_t cells, size_t rows, size_t ragged, size_t padded, size_t most, size_t elem, size_t mem_free) {
     const double state = 9.0 * (double)cells * (double)elem, wide = 9.0 * (double)padded * (double)elem;
     const double ratios = 4.0 * (double)cells, even = 4.0 * (double)padded, read = 72.0 * (double)most;
     const double room = (double)mem_free - 64.0e6;   // contexts, tables, allocation granularity
     if (2.0 * wide + even + read > room && 2.0 * state + ratios + read <= (double)mem_free) return false;
     if (3.0 * wide + even > room && 3.0 * state + ratios <= (double)mem_free) return false;
-    const size_t width = 2.0 * state < 32.0e6 ? 8 : elem == 4 ? 64 : 31;   // mean width of the rows
-    return cells >= width * rows;
+    const bool small = 2.0 * state < 32.0e6;
+    if (cells < (size_t)(small ? 8 : 31) * rows) return false;   // mean width of the rows
+    return small || elem == 2 || cells >= 100 * ragged;
 }
 
 // a + b = s + e exactly, unless s overflows (TwoSum: Knuth, The Art of Computer Programming, Vol. 2, Sec. 4.2.2)

@@ -22,7 +22,7 @@ def empty(k, nx, ny):
 # a wide domain with disks among them
 SMALL = [empty(0, 3, 7), empty(1, 4, 201), W.c5_domain(2, 41, 24, 8.0, 0.15, 0.6, 3.0, 42), empty(3, 5, 97), empty(4, 7, 33),
          empty(5, 3, 400), W.c5_domain(6, 19, 21, 8.0, 0.15, 0.6, 3.0, 46), empty(7, 6, 64)]
-# below 64 in a large one (86 MB of FP32): the same three domains over and over, the last one odd
+# below 100 in a large one (86 MB of FP32): the same three domains over and over, the last one odd
 LARGE = [W.c5_domain(k % 3, 50 + k % 3, 60, 10.0, 0.2, 0.65, 2.0, 50 + k % 3) for k in range(398)] + [empty(9, 37, 41)]
 
 

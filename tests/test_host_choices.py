@@ -98,7 +98,8 @@ int main() {
 
 def test_batch_layout_leaves_room(tmp_path):
     # whatever batch and free memory: a batch whose unpadded buffers fit (two with the read-back, or three)
-    # fits in the layout it is given; rows of at least 64 cells are blocked where memory allows, narrow ones not
+    # fits in the layout it is given; rows of at least 100 cells, and of 32 or more where
+    # they fill their sectors, are blocked where memory allows, narrow ones not
     run_cpp(tmp_path, """
 #include <random>
 int main() {
@@ -108,14 +109,14 @@ int main() {
         const size_t nx = (size_t)log_uniform(3, 5000), ny = (size_t)log_uniform(3, 5000), n = (size_t)log_uniform(1, 1e5);
         const size_t elem = g() & 1 ? 4 : 2, G = 128 / elem, w = (nx + G - 1) / G * G;
         const size_t cells = n * nx * ny, rows = n * ny, padded = n * w * ny, mem = (size_t)log_uniform(1e8, 3e11);
-        const bool b = blocked_rows(cells, rows, padded, nx * ny, elem, mem);
+        const bool b = blocked_rows(cells, rows, nx % 16 ? rows : 0, padded, nx * ny, elem, mem);
         const size_t c = b ? padded : cells;
         const double slack = 1e6;   // what a few tables take
         if (2.0 * 9 * cells * elem + 4.0 * cells + 72.0 * nx * ny <= (double)mem)
             CHECK(2.0 * 9 * c * elem + 4.0 * (b ? n * ny * ((nx + 1) / 2 * 2) : cells) + 72.0 * nx * ny <= (double)mem + slack);
         if (3.0 * 9 * cells * elem + 4.0 * cells <= (double)mem)
             CHECK(3.0 * 9 * c * elem + 4.0 * (b ? n * ny * ((nx + 1) / 2 * 2) : cells) <= (double)mem + slack);
-        if (nx >= 64 && 3.0 * 9 * padded * elem + 4.0 * padded + 72.0 * nx * ny < (double)mem - 1e8) CHECK(b);
+        if ((nx >= 100 || (nx >= 32 && nx % 16 == 0)) && 3.0 * 9 * padded * elem + 4.0 * padded + 72.0 * nx * ny < (double)mem - 1e8) CHECK(b);
         if (nx < 8) CHECK(!b);
     }
 }
