@@ -17,6 +17,7 @@
 #include "imb_device.cuh"
 #include "imb_host.h"
 #include "imb_kernels.h"
+#include "imb_sums.h"
 #include "imb_pull.cuh"
 
 namespace imb {

@@ -18,7 +18,7 @@
 #include <utility>
 
 #include "imb_device.cuh"
-#include "imb_host.h"
+#include "imb_sums.h"
 #include "imb_kernels.h"
 #include "imb_pull.cuh"
 #include "imb_node.cuh"

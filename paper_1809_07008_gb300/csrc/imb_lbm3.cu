@@ -25,6 +25,7 @@
 #include "imb_device.cuh"
 #include "imb_host.h"
 #include "imb_kernels.h"
+#include "imb_sums.h"
 
 namespace imb3 {
 

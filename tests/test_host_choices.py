@@ -1,5 +1,5 @@
-"""Decisions the host takes before a launch (csrc/imb_host.h), compiled with the host compiler and
-checked over their whole range, without a GPU."""
+"""Decisions the host takes before a launch (csrc/imb_host.h) and the sums and the division that keep their
+bits (csrc/imb_sums.h), compiled with the host compiler and checked without a GPU."""
 import os
 import shutil
 import subprocess
@@ -15,7 +15,7 @@ def run_cpp(tmp_path, body):
     if not cxx:
         pytest.skip("no host compiler")
     src, exe = tmp_path / "t.cpp", tmp_path / "t"
-    src.write_text('#include "imb_host.h"\n#include <cstdio>\n#include <cstdlib>\nusing namespace imb;\n'
+    src.write_text('#include "imb_host.h"\n#include "imb_sums.h"\n#include <cstdio>\n#include <cstdlib>\nusing namespace imb;\n'
                    '#define CHECK(c) do { if (!(c)) { std::printf("failed: %s\\n", #c); std::exit(1); } } while (0)\n' + body)
     subprocess.run([cxx, "-std=c++17", "-O2", "-pthread", "-I", CSRC, str(src), "-o", str(exe)], check=True)
     r = subprocess.run([str(exe)], capture_output=True, text=True)
