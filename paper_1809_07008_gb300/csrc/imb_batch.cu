@@ -281,7 +281,7 @@ template <typename S> struct Pulled<S, 2> {
 // of the loads; the schedulers issue on half the cycles and DRAM moves 44 B a cell of the 40 it must
 // (16 bits), at 4.5 TB/s.  256 domains, 15.5 M cells, FP16, 100 steps at a time: 195 us a step with whole
 // planes one after another, rows cut into segments and one cell a lane, 149 us now (in runs of 5000 steps
-// 186 -> 140 us; 155 to 158 us on the box and day of the variants below); 12 domains of 0.28 M cells together,
+// 186 -> 138 us; 155 to 158 us where the variants below were timed); 12 domains of 0.28 M cells together,
 // FP32: 11.0 -> 9.6 us.
 // With the collision as a sum of d_q + d_-q and d_q - d_-q (half the operations) 156 us and twice
 // the FP32 error; two items ahead 148 us with that form, 176 us (spills) with this one; three
