@@ -148,32 +148,28 @@ __device__ __forceinline__ bool rest_node(typename V::T (&d)[9], const typename 
     const T tm = V::add(te, V::all(-0.5f));
     const T den = V::each(V::add(sub(one, ec), tm), [](float v) { return __fdividef(1.0f, v); });
     const T B = V::mul(V::mul(ec, tm), den);   // Eq. 14 (0 in uncovered cells)
-    // d*_q = (1 - B) [d_q - omega (d_q - w_q (even + odd))] + B [d_-q - w_q (back even - back odd)],
-    //   even = t + 4.5 rho (c.u)^2 + m (9 (c.u)(c.F) - 3 u.F),  odd = 3 c.j + m 3 c.F,  m = tau_eff - 1/2:
-    // the forcing (1 - omega / 2) S_q = omega m S_q goes into the equilibrium that is relaxed to;
-    //   back even = t - drho + 4.5 rho (c.u)^2,  back odd = 3 c.j
-    const T fl = sub(one, B), mo = V::mul(omega, neg), m3 = V::mul(V::all(3.0f), tm), m9 = V::mul(V::all(9.0f), tm);
+    // d*_q = (1 - B) d_q - (1 - B) omega n_q + B n_{-q} + w_q [(1 - B)(1 - omega / 2) S_q + B drho], summed from
+    // the smallest term up to d_q, which alone rounds at its own size;
+    //   n_{+-q} = d_{+-q} - w_q (t + 4.5 rho (c.u)^2 +- 3 c.j),  S_{+-q} = 9 (c.u)(c.F) - 3 u.F +- 3 c.F
+    const T fl = sub(one, B), flw = V::mul(V::mul(fl, neg), omega);
+    const T fls = V::mul(fl, V::fma(V::all(-0.5f), omega, one)), Bd = V::mul(B, drho);
     const T g = V::mul(V::all(-3.0f), V::fma(ux, V::all(D.Fx), V::mul(uy, V::all(D.Fy))));
     const T jx3 = V::mul(V::all(3.0f), jx), jy3 = V::mul(V::all(3.0f), jy);
     const T ux15 = V::mul(V::all(1.5f), ux), uy15 = V::mul(V::all(1.5f), uy);
-    const T base = V::fma(tm, g, t), back = V::mul(V::all(-1.5f), juu);
-    const T ox = V::fma(m3, V::all(D.Fx), jx3), oy = V::fma(m3, V::all(D.Fy), jy3);
-    const T hx = V::fma(m9, V::all(D.Fx), V::mul(V::all(1.5f), jx3)), hy = V::fma(m9, V::all(D.Fy), V::mul(V::all(1.5f), jy3));
-    const T f0 = V::fma(mo, V::fma(V::all(-w_of(0)), base, d[0]), d[0]);
-    d[0] = V::fma(fl, f0, V::mul(B, V::fma(V::all(-w_of(0)), back, d[0])));
-    const T u4[4] = {ux, uy, V::add(ux, uy), sub(uy, ux)}, h4[4] = {hx, hy, V::add(hx, hy), sub(hy, hx)};
+    const T n0 = V::fma(V::all(-w_of(0)), t, d[0]);
+    const T v0 = V::mul(V::all(w_of(0)), V::fma(fls, g, Bd));
+    d[0] = V::fma(fl, d[0], V::fma(flw, n0, V::fma(B, n0, v0)));
     const T v4[4] = {ux15, uy15, V::add(ux15, uy15), sub(uy15, ux15)}, j4[4] = {jx3, jy3, V::add(jx3, jy3), sub(jy3, jx3)};
-    const T o4[4] = {ox, oy, V::add(ox, oy), sub(oy, ox)};
+    const float F4[4] = {D.Fx, D.Fy, D.Fx + D.Fy, D.Fy - D.Fx};   // c.F
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int q = bpair_q(k), o = opp_of(q);
-        const T w = V::all(-w_of(q));
-        const T ev = V::fma(u4[k], h4[k], base), bk = V::fma(j4[k], v4[k], back);
-        const T fq = V::fma(mo, V::fma(w, V::add(ev, o4[k]), d[q]), d[q]);
-        const T fo = V::fma(mo, V::fma(w, sub(ev, o4[k]), d[o]), d[o]);
-        const T sq = V::fma(w, sub(bk, j4[k]), d[o]), so = V::fma(w, V::add(bk, j4[k]), d[q]);
-        d[q] = V::fma(fl, fq, V::mul(B, sq));
-        d[o] = V::fma(fl, fo, V::mul(B, so));
+        const T w = V::all(-w_of(q)), wp = V::all(w_of(q));
+        const T ev = V::fma(j4[k], v4[k], t), se = V::fma(V::all(6.0f * F4[k]), v4[k], g), so = V::all(3.0f * F4[k]);
+        const T nq = V::fma(w, V::add(ev, j4[k]), d[q]), no = V::fma(w, sub(ev, j4[k]), d[o]);
+        const T vq = V::mul(wp, V::fma(fls, V::add(se, so), Bd)), vo = V::mul(wp, V::fma(fls, sub(se, so), Bd));
+        d[q] = V::fma(fl, d[q], V::fma(flw, nq, V::fma(B, no, vq)));
+        d[o] = V::fma(fl, d[o], V::fma(flw, no, V::fma(B, nq, vo)));
     }
     fx = V::fma(B, V::add(jx, V::all(-D.Fx)), fx);
     fy = V::fma(B, V::add(jy, V::all(-D.Fy)), fy);
@@ -277,12 +273,14 @@ template <typename S> struct Pulled<S, 2> {
 // domain sizes, and the drag of a domain is summed in registers until the warp leaves it.  The
 // loads of the next item of the same domain are issued before the arithmetic of the current one.
 //
-// What bounds it: with two cells a lane the registers (120, two blocks an SM: 16 warps) and the latency
+// What bounds it: with two cells a lane the registers (128, two blocks an SM: 16 warps) and the latency
 // of the loads; the schedulers issue on half the cycles and DRAM moves 44 B a cell of the 40 it must
-// (16 bits), at 4.5 TB/s.  256 domains, 15.5 M cells, FP16, 100 steps at a time: 195 us a step with whole
-// planes one after another, rows cut into segments and one cell a lane, 149 us now (in runs of 5000 steps
-// 186 -> 138 us; 155 to 158 us where the variants below were timed); 12 domains of 0.28 M cells together,
-// FP32: 11.0 -> 9.6 us.
+// (16 bits), at 4.3 TB/s.  256 domains, 15.5 M cells, FP16, 100 steps at a time: 195 us a step with whole
+// planes one after another, rows cut into segments and one cell a lane, 154 us now (in runs of 5000 steps
+// 186 -> 139 us; 155 to 158 us where the variants below were timed); 12 domains of 0.28 M cells together,
+// FP32: 11.5 -> 9.4 us.  With the forcing inside the equilibrium that is relaxed to, d_q - omega (d_q - w_q E'_q),
+// 150 us, but one more rounding at the size of E' and of d_q: the drag's error against 64 bits was 8.3e-7 (rms over
+// 288 FP32 domains), 7.7e-7 with the former sums over direction pairs and 6.1e-7 with these.
 // With the collision as a sum of d_q + d_-q and d_q - d_-q (half the operations) 156 us and twice
 // the FP32 error; two items ahead 148 us with that form, 176 us (spills) with this one; three
 // blocks an SM (80 registers, spills) 187 us; five of 128 threads 151 us.
